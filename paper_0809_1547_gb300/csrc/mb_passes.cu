@@ -296,8 +296,7 @@ __global__ void __launch_bounds__(BX * BY) k_e_tma(StepArgs a, const __grid_cons
     constexpr int NW = BX * BY / 32;
     extern __shared__ unsigned char smem_raw[];
     __shared__ float wfl[6][NW];   // per-warp face-flux partials, summed plane by plane
-    unsigned char* smem = reinterpret_cast<unsigned char*>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
+    unsigned char* smem = align_smem(smem_raw);
     float* gbuf = reinterpret_cast<float*>(smem + S * Lay::kStage);
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + S * Lay::kStage + Lay::kGBytes);
     const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + BX * ty;
@@ -477,8 +476,7 @@ __global__ void __launch_bounds__(BX * BY) k_hg_tma(StepArgs a, const __grid_con
     }
     using Lay = TmaLayoutH<BX, BY>;
     extern __shared__ unsigned char smem_raw[];
-    unsigned char* smem = reinterpret_cast<unsigned char*>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
+    unsigned char* smem = align_smem(smem_raw);
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + S * Lay::kStage);
     const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + BX * ty;
     const int bx = idx % lay.gx, by = (idx / lay.gx) % lay.gy, bz = idx / (lay.gx * lay.gy);

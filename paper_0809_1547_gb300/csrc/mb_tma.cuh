@@ -13,6 +13,13 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// The dynamic shared memory from its first 128-byte boundary on, as an offset
+// from the array: an address taken through an integer loses its address
+// space, and every access through it becomes a generic one.
+__device__ __forceinline__ unsigned char* align_smem(unsigned char* raw) {
+    return raw + ((0u - smem_addr(raw)) & 127u);
+}
+
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count)
                  : "memory");
