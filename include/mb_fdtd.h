@@ -289,9 +289,13 @@ int mb_get_field_device(mb_ctx* ctx, int which, float* dev_out, double* scale);
 int mb_save_state(mb_ctx* ctx, void* host_blob, size_t* bytes);
 int mb_load_state(mb_ctx* ctx, const void* host_blob, size_t bytes);
 
-/* Time the candidate thread-block shapes of the two field passes on this
- * grid (the state is saved and restored around the trials) and keep the
- * fastest.  The choice is cached per grid shape for the process. */
+/* Time the candidate launches on this grid (the state is saved and restored
+ * around the trials) and keep the fastest: block shapes of the two field
+ * passes, the single-pass step, and on small grids (up to about 60^3 cells)
+ * a launch that advances up to 64 steps with the state in shared memory,
+ * used for calls of enough steps; mb_get_single_pass reports that one as
+ * off.  All give the same bits (the face-flux sums to FP32 rounding).  The
+ * choice is cached per grid shape for the process. */
 int mb_autotune(mb_ctx* ctx);
 
 /* Launch shape of the H pass and of the E pass, as {variant, bx, by, bz}:

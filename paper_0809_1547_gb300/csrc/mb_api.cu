@@ -308,6 +308,8 @@ int check_device_error(mb_ctx* c) {
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
     if (e) {
         cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream);
+        // blocks that gave up leave their step flags behind the others'
+        if (c->d_small) cudaMemsetAsync(c->d_small, 0, sizeof(unsigned) * (mb::kSmallFlagWords + 1), c->stream);
         return fail(c, MB_ERR_TIMEOUT, "a bounded device wait gave up (results of that step are invalid)");
     }
     return MB_OK;
@@ -803,7 +805,8 @@ int mb_destroy(mb_ctx* c) {
                     c->d_nonfinite, c->d_probe_cell, c->d_probe_omega, c->d_probe_acc,
                     c->d_face_omega, c->d_face_acc, c->d_face_acc32, c->d_glist, c->d_glist_scratch,
                     c->d_upload, c->d_keys, c->d_src_wave, c->d_err,
-                    c->d_fields2, c->d_psi2[0], c->d_psi2[1], c->d_psi2[2], c->d_flux_out};
+                    c->d_fields2, c->d_psi2[0], c->d_psi2[1], c->d_psi2[2], c->d_flux_out, c->d_small,
+                    c->d_small_x};
     for (void* b : bufs)
         if (b) cudaFree(b);
     for (const mb::DevPlaneProbe& q : c->planes) {

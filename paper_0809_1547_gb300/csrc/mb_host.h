@@ -97,6 +97,7 @@ constexpr int kVariant3D = 0;
 constexpr int kVariantZmarch = 1;
 constexpr int kVariantTma = 2;   // TMA-staged z-walk (nx % 16 == 0)
 constexpr int kVariantVec = 3;   // z-walk over quads of 4 x-cells, 16-byte accesses (nx % 4 == 0)
+constexpr int kVariantSmall = 4; // many steps per launch, state in shared memory (small grids; tune_f only)
 struct PassTune {
     int variant;
     dim3 block;
@@ -166,6 +167,33 @@ bool fused_tile_supported(int bx, int by);
 bool encode_fused(const StepArgs& a, int bx, int by, TmaFusedMaps* out);
 void launch_fused_step(const StepArgs& a, const DevPing& d, const PassTune& t,
                        const TmaFusedMaps& maps, cudaStream_t s);
+
+// Many steps of a small grid in one cooperative launch (mb_small.cu).  The
+// box of cells each block owns and the number of blocks per axis.
+struct SmallTile {
+    int tx, ty, tz, bx, by, bz;
+};
+constexpr int kSmallMaxProbes = 4;     // point probes advanced inside the launch
+constexpr int kSmallMaxBins = 1024;    // bins of each
+constexpr int kSmallMaxBlocks = 256;
+constexpr int kSmallFlagStride = 32;   // words between flags: a 128-byte line each (shared lines serialise the polls)
+constexpr int kSmallFlagWords = kSmallFlagStride * kSmallMaxBlocks;
+constexpr int kSmallMaxSteps = 64;     // steps per launch (entries of the sample buffer)
+struct SmallArgs {
+    StepArgs a;              // the copy holding the state
+    DevPing d;               // the other copy
+    SmallTile t;
+    unsigned* flags;         // a word per block (kSmallFlagStride apart): steps done, counted over all launches
+    unsigned* base;          // that count at the start of the launch
+    float4* xbuf;            // exchange buffer: two halves of (blocks, cells of a box) E values
+    float* samples;          // [kSmallMaxSteps][count][3]: E at the probes after each step
+    long long* sample_in;    // the step count kept for a's copy (d.sample: for the other)
+    DevPointProbes pp;
+    int nsteps;
+    double dt;
+};
+bool small_tile(const DevGrid& g, bool pml, int max_blocks, SmallTile* out);
+cudaError_t launch_step_small(const SmallArgs& A, cudaStream_t s);
 
 // Grid of the H + gain launch: nH H tiles (tile grid gx x gy x gz) and nG
 // gain blocks, each over q consecutive entries of the gain list.
@@ -386,6 +414,11 @@ struct mb_ctx {
     bool use_fused = false;
     mb::PassTune tune_f{mb::kVariantTma, dim3(32, 8, 1), 32};
     float* d_fields2 = nullptr;        // second copy of E, H (6 arrays)
+    // the small-grid launch: its boxes (bx = 0: not available), and the flag
+    // words, step base and probe samples on the device
+    mb::SmallTile small{0, 0, 0, 0, 0, 0};
+    unsigned* d_small = nullptr;
+    float4* d_small_x = nullptr;       // its exchange buffer
     float* d_psi2[3] = {nullptr, nullptr, nullptr};
     int parity = 0;
     std::map<std::pair<int, int>, std::pair<mb::TmaFusedMaps, mb::TmaFusedMaps>> fused_maps;
