@@ -26,7 +26,11 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#include <map>
+#include <mutex>
 #include <string>
+#include <tuple>
+#include <utility>
 #include <vector>
 
 namespace mb {
@@ -502,7 +506,9 @@ __global__ void __launch_bounds__(256, 6) k_adj_e_point(AdjArgs a) {
     warp_acc(a.acc + kAccSlots, gw, slot);
 }
 
-// Store slot of one step: E (arrays 0..2) and J, n1..n3 (arrays 9..14) of
+// Store slot of a segment's first state (the E pass keeps the others as it
+// computes them; this copy also serves the quad-vectorised E pass, which
+// does not): E (arrays 0..2) and J, n1..n3 (arrays 9..14) of
 // the field block, Hx and Hy of plane kp, and the step counter.  16-byte
 // moves when n_cells and the plane size are multiples of 4 (every array then
 // starts 16-byte aligned).  The stores are marked streaming (evict first), so
@@ -551,6 +557,10 @@ __global__ void k_adj_out(const double* geps, float* out, uint32_t n, double sca
 
 namespace {
 
+// Launch shapes of the recomputation per grid shape and CPML depth.
+std::mutex g_shape_mu;
+std::map<std::tuple<int, int, int, int>, std::pair<mb::PassTune, mb::PassTune>> g_shapes;
+
 struct NvtxScope {
     explicit NvtxScope(const char* name) { nvtxRangePushA(name); }
     ~NvtxScope() { nvtxRangePop(); }
@@ -573,6 +583,13 @@ int afail(mb_ctx* c, int code, const std::string& msg) {
     } while (0)
 
 }  // namespace
+
+void mb::adjoint_release(mb_ctx* c) {
+    if (c->d_adj_ws) cudaFree(c->d_adj_ws);
+    c->d_adj_ws = nullptr;
+    c->dev_bytes -= c->adj_ws_bytes;
+    c->adj_ws_bytes = 0;
+}
 
 extern "C" int mb_adjoint_energy_zface(mb_ctx* c, int n_steps, int ckpt_every, int z_plane,
                                        float* d_grad_eps, double* grad_pump, double* J_out) {
@@ -657,22 +674,45 @@ extern "C" int mb_adjoint_energy_zface(mb_ctx* c, int n_steps, int ckpt_every, i
     };
     // recompute a segment from the checkpoint restored into the context
     // (same pass kernels, probes and flux off), keeping every state
+    auto keep_to = [&](mb::StepArgs& x, int t) {   // the E pass of x writes slot t
+        x.keep = t < 0 ? nullptr : store + slot * t;
+        x.keep_zp = zp;
+        x.keep_n = slot_n + std::max(t, 0);
+    };
     auto recompute = [&](int len) -> cudaError_t {
         cudaError_t e = keep(0);
+        const bool own = te_r.variant != mb::kVariantVec;
         for (int t = 0; t < len && e == cudaSuccess; ++t) {
             mb::launch_h_pass(fa, th, maps_for(th), c->stream);
+            keep_to(fa, own ? t + 1 : -1);
             mb::launch_e_pass(fa, te_r, maps_for(te_r), c->stream);
-            e = keep(t + 1);
+            e = own ? cudaGetLastError() : keep(t + 1);
         }
+        keep_to(fa, -1);
         return e;
     };
 
-    MB_ACUDA(c, cudaMalloc((void**)&ckpt, sb * (nseg + 1)));
-    MB_ACUDA(c, cudaMalloc((void**)&store, sizeof(float) * slot * (K + 1)));
-    MB_ACUDA(c, cudaMalloc((void**)&adj, sizeof(float) * (18 * N + psi_total)));
-    MB_ACUDA(c, cudaMalloc((void**)&geps, sizeof(double) * N));
-    MB_ACUDA(c, cudaMalloc((void**)&acc, sizeof(double) * 2 * mb::kAccSlots));
-    MB_ACUDA(c, cudaMalloc((void**)&slot_n, sizeof(long long) * (K + 1)));
+    {
+        // one block of device memory for all of it, kept in the context for
+        // the next call where it is at most a sixteenth of the device's memory
+        // (allocating and freeing 8.6 GB took 3.5 ms of a 72 ms call)
+        const size_t part[6] = {sb * (nseg + 1), sizeof(float) * slot * (K + 1), sizeof(float) * (18 * N + psi_total),
+                                sizeof(double) * N, sizeof(double) * 2 * mb::kAccSlots, sizeof(long long) * (K + 1)};
+        size_t at[7] = {0};
+        for (int q = 0; q < 6; ++q) at[q + 1] = at[q] + (part[q] + 255) / 256 * 256;
+        if (c->adj_ws_bytes < at[6]) {
+            mb::adjoint_release(c);
+            MB_ACUDA(c, cudaMalloc((void**)&c->d_adj_ws, at[6]));
+            c->adj_ws_bytes = at[6];
+            c->dev_bytes += at[6];
+        }
+        ckpt = c->d_adj_ws + at[0];
+        store = reinterpret_cast<float*>(c->d_adj_ws + at[1]);
+        adj = reinterpret_cast<float*>(c->d_adj_ws + at[2]);
+        geps = reinterpret_cast<double*>(c->d_adj_ws + at[3]);
+        acc = reinterpret_cast<double*>(c->d_adj_ws + at[4]);
+        slot_n = reinterpret_cast<long long*>(c->d_adj_ws + at[5]);
+    }
 
     // forward sweep: a checkpoint at the start of every segment but the last,
     // whose states are kept as it runs (it is reversed first)
@@ -681,12 +721,30 @@ extern "C" int mb_adjoint_energy_zface(mb_ctx* c, int n_steps, int ckpt_every, i
         if ((rc = mb_step(c, K))) goto done;
     }
     fa.flux.on = 0;
-    if (nseg > 1) {
-        // The recomputation streams from HBM (the segment store evicts the
-        // state from L2), unlike the plain step the context was tuned for:
-        // time candidate shapes in its own sequence (store, H, E) from the
-        // start of the last segment, then put the state back (the store is
-        // still empty).
+    {
+    bool have_shape = nseg < 2;
+    if (!have_shape && c->ncell < mb::kSmallPassCells) {
+        // the same shapes as the passes' defaults at these sizes: trials would
+        // cost more than the segments they are for
+        th = te_r = mb::PassTune{mb::kVariant3D, dim3(64, 4, 1), 1};
+        have_shape = true;
+    }
+    const auto shape_key = std::make_tuple(c->nx, c->ny, c->nz, c->p.npml);
+    if (!have_shape) {
+        std::lock_guard<std::mutex> lk(g_shape_mu);
+        const auto it = g_shapes.find(shape_key);
+        if (it != g_shapes.end()) {
+            th = it->second.first;
+            te_r = it->second.second;
+            have_shape = true;
+        }
+    }
+    if (!have_shape) {
+        // The recomputation streams to HBM (the segment store's writes),
+        // unlike the plain step the context was tuned for: time candidate
+        // shapes in its own sequence from the start of the last segment, then
+        // put the state back (the store is still empty).  Once per grid shape
+        // and CPML depth in the process (5 ms at 96^3).
         if ((rc = mb::state_snapshot(c, ckpt + sb * (nseg - 1)))) goto done;
         std::vector<mb::PassTune> cand = {c->tune_h, c->tune_e};
         for (int kz : {4, 8, 16}) cand.push_back({mb::kVariantZmarch, dim3(32, 4, 1), kz});
@@ -702,16 +760,19 @@ extern "C" int mb_adjoint_energy_zface(mb_ctx* c, int n_steps, int ckpt_every, i
             float best = 1e30f;
             mb::PassTune pick = pass == 0 ? th : te_r;
             for (const mb::PassTune& t : cand) {
-                if (t.kz > 2 * c->nz || (t.variant == mb::kVariantTma && !maps_for(t))) continue;
+                if (t.kz > 2 * c->nz || t.variant == mb::kVariantVec ||
+                    (t.variant == mb::kVariantTma && !maps_for(t)))
+                    continue;
                 float tot = 0.0f;
                 for (int r = 0; r < 3; ++r) {
-                    MB_ACUDA(c, keep(0));
                     if (pass == 1) mb::launch_h_pass(fa, th, maps_for(th), c->stream);
+                    keep_to(fa, r % (K + 1));
                     cudaEventRecord(e0, c->stream);
                     if (pass == 0) mb::launch_h_pass(fa, t, maps_for(t), c->stream);
                     else mb::launch_e_pass(fa, t, maps_for(t), c->stream);
                     cudaEventRecord(e1, c->stream);
                     if (pass == 0) mb::launch_e_pass(fa, te_r, maps_for(te_r), c->stream);
+                    keep_to(fa, -1);
                     cudaEventSynchronize(e1);
                     float ms = 0.0f;
                     cudaEventElapsedTime(&ms, e0, e1);
@@ -725,18 +786,27 @@ extern "C" int mb_adjoint_energy_zface(mb_ctx* c, int n_steps, int ckpt_every, i
             if (pass == 0) th = pick;
             else te_r = pick;
         }
+        {
+            std::lock_guard<std::mutex> lk(g_shape_mu);
+            g_shapes[shape_key] = {th, te_r};
+        }
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
         MB_ACUDA(c, cudaGetLastError());
         if ((rc = mb::state_restore(c, ckpt + sb * (nseg - 1)))) goto done;
     }
+    }
 
     {
         const int len = n_steps - (nseg - 1) * K;
         MB_ACUDA(c, keep(0));
+        const bool own = c->tune_e.variant != mb::kVariantVec;
         for (int t = 0; t < len; ++t) {
-            MB_ACUDA(c, mb::enqueue_step(c));
-            MB_ACUDA(c, keep(t + 1));
+            keep_to(c->args, own ? t + 1 : -1);
+            const cudaError_t e = mb::enqueue_step(c);
+            keep_to(c->args, -1);
+            MB_ACUDA(c, e);
+            if (!own) MB_ACUDA(c, keep(t + 1));
         }
     }
     if ((rc = mb::state_snapshot(c, ckpt + sb * nseg))) goto done;
@@ -826,9 +896,10 @@ extern "C" int mb_adjoint_energy_zface(mb_ctx* c, int n_steps, int ckpt_every, i
 done:
     if (c->stream) cudaStreamSynchronize(c->stream);
     if (seg_graph) cudaGraphExecDestroy(seg_graph);
-    void* bufs[] = {ckpt, store, adj, geps, acc, slot_n};
-    for (void* p : bufs)
-        if (p) cudaFree(p);
+    {
+        size_t free_b = 0, total_b = 0;
+        if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || c->adj_ws_bytes > total_b / 16) mb::adjoint_release(c);
+    }
     mb::restore_single_pass(c, was_single_pass);
     return rc;
 }

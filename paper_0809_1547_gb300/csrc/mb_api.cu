@@ -752,6 +752,9 @@ static int create_ctx(mb_ctx** out, const int grid[3], int gnz, int kz0, int own
             c->tune_e = it->second.e;
             c->tune_f = it->second.f;
             c->use_fused = it->second.fused;   // second copy allocated at the first step
+        } else if (ncell < mb::kSmallPassCells) {
+            c->tune_h = mb::PassTune{mb::kVariant3D, dim3(64, 4, 1), 1};
+            c->tune_e = mb::PassTune{mb::kVariantZmarch, dim3(32, 4, 1), mb::kSmallPassPlanes};
         }
     }
     *out = c;
@@ -800,6 +803,7 @@ int mb_destroy(mb_ctx* c) {
         cudaStreamSynchronize(c->stream);
     }
     drop_graphs(c);
+    mb::adjoint_release(c);
     void* bufs[] = {c->d_fields, c->d_mat, c->d_inv_eps, c->d_lut, c->d_psi[0], c->d_psi[1],
                     c->d_psi[2], c->d_coef, c->d_ctr, c->d_flux, c->d_partial, c->d_energy,
                     c->d_nonfinite, c->d_probe_cell, c->d_probe_omega, c->d_probe_acc,

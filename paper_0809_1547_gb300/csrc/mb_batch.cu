@@ -237,6 +237,9 @@ int mb_batch_create(mb_batch** out, int B, const int* grids, double dx, double d
         if (rc) return bail(rc);
         b->inst.push_back(c);
     }
+    int64_t largest = 0;
+    for (mb_ctx* c : b->inst) largest = std::max(largest, c->ncell);
+    if (largest < mb::kSmallPassCells) b->kz = mb::kSmallPassPlanes;
     cudaError_t e = cudaMalloc((void**)&b->d_bar, sizeof(unsigned) * 2);
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_err, sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_tick, sizeof(unsigned long long));

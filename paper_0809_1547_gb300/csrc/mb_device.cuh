@@ -120,7 +120,39 @@ struct StepArgs {
     long long* step_ctr;
     // Set (bit 0) when a bounded device wait gave up; read by the host.
     int* err;
+    // The adjoint's segment store (null: none): the E pass also writes the
+    // state it leaves, E (3 arrays of ncell), J and n1..n3 of the gain cells
+    // (6 arrays) and Hx, Hy of the plane below keep_zp (2 planes), to keep,
+    // and the step count to *keep_n.
+    float* keep;
+    int keep_zp;
+    long long* keep_n;
 };
+
+// The cell's part of the segment store, streaming (read back once, after
+// gigabytes of later stores).
+__device__ __forceinline__ void keep_cell(const StepArgs& a, uint32_t c, int k, float ex, float ey, float ez,
+                                          bool gain, float jx, float jy, float jz, float n1, float n2, float n3,
+                                          float hx_k, float hy_k) {
+    const size_t N = a.g.ncell;
+    float* p = a.keep + c;
+    __stcs(p, ex);
+    __stcs(p + N, ey);
+    __stcs(p + 2 * N, ez);
+    if (gain) {
+        __stcs(p + 3 * N, jx);
+        __stcs(p + 4 * N, jy);
+        __stcs(p + 5 * N, jz);
+        __stcs(p + 6 * N, n1);
+        __stcs(p + 7 * N, n2);
+        __stcs(p + 8 * N, n3);
+    }
+    if (k == a.keep_zp) {
+        float* h = a.keep + 9 * N + (c - a.g.nxy * (uint32_t)k);
+        __stcs(h, hx_k);
+        __stcs(h + a.g.nxy, hy_k);
+    }
+}
 
 // Where a cell update writes the CPML memories it advances: the step's own
 // arrays (in-place passes) or the other copy of them (single-pass step).
@@ -604,7 +636,9 @@ __device__ __forceinline__ void e_compute(const StepArgs& a, int i, int j, int k
                             fl, ex1, ey1, ez1, psi_in_place(a), flux_plane);
 }
 
-template <bool FLUX, bool PML>
+// KEEP: the cell's part of the segment store is written too (a form of its
+// own: as a test in every launch it cost the ensemble's members 4 %).
+template <bool FLUX, bool PML, bool KEEP = false>
 __device__ __forceinline__ void e_apply(const StepArgs& a, int i, int j, int k, uint32_t c,
                                         const HNb& h, uint8_t m, float ex0, float ey0, float ez0,
                                         bool gain, float jx, float jy, float jz, float n1, float n2,
@@ -621,9 +655,10 @@ __device__ __forceinline__ void e_apply(const StepArgs& a, int i, int j, int k, 
         f.n2[c] = n2;
         f.n3[c] = n3;
     }
+    if (KEEP) keep_cell(a, c, k, ex1, ey1, ez1, gain, jx, jy, jz, n1, n2, n3, h.hx_k, h.hy_k);
 }
 
-template <bool FLUX, bool PML>
+template <bool FLUX, bool PML, bool KEEP = false>
 __device__ __forceinline__ void e_core(const StepArgs& a, int i, int j, int k, uint32_t c,
                                        const HNb& h, long long n, float fl[6],
                                        bool flux_plane = true) {
@@ -641,7 +676,7 @@ __device__ __forceinline__ void e_core(const StepArgs& a, int i, int j, int k, u
         n2 = f.n2[c];
         n3 = f.n3[c];
     }
-    e_apply<FLUX, PML>(a, i, j, k, c, h, m, ex0, ey0, ez0, gain, jx, jy, jz, n1, n2, n3, n, fl,
+    e_apply<FLUX, PML, KEEP>(a, i, j, k, c, h, m, ex0, ey0, ez0, gain, jx, jy, jz, n1, n2, n3, n, fl,
                        flux_plane);
 }
 

@@ -103,6 +103,13 @@ struct PassTune {
     dim3 block;
     int kz;
 };
+// Grids of fewer cells take one thread per cell in the H pass and walks of 4
+// planes in the E pass by default (and in a batch of such grids): walks of 32
+// and 16 planes leave most of the GPU without a warp and pay each plane's
+// latency in turn (H 17-19 us against 7, E 22 against 9 at 24 x 22 x 20 to
+// 48^3; at 96^3 the longer walks are the faster).
+constexpr int64_t kSmallPassCells = 400000;
+constexpr int kSmallPassPlanes = 4;
 
 // Polls of a bounded mbarrier wait before the kernel gives up (~0.1-1 s).
 constexpr int kWaitLimit = 1 << 20;
@@ -296,6 +303,9 @@ void restore_single_pass(mb_ctx* c, bool on);
 // running on the second stream (event waits only; never blocks the host).
 void join_probes(mb_ctx* c);
 
+// Frees the adjoint's device memory kept in the context.
+void adjoint_release(mb_ctx* c);
+
 // d/dW_p of the reduced population propagator (g, G, mk of DevGain).
 void gain_pump_derivative(const mb_ctx* c, float dg[3], float dG[3][3], float dmk[3]);
 
@@ -414,6 +424,9 @@ struct mb_ctx {
     bool use_fused = false;
     mb::PassTune tune_f{mb::kVariantTma, dim3(32, 8, 1), 32};
     float* d_fields2 = nullptr;        // second copy of E, H (6 arrays)
+    // the adjoint's device memory, kept between calls (mb_adjoint.cu)
+    char* d_adj_ws = nullptr;
+    size_t adj_ws_bytes = 0;
     // the small-grid launch: its boxes (bx = 0: not available), and the flag
     // words, step base and probe samples on the device
     mb::SmallTile small{0, 0, 0, 0, 0, 0};

@@ -54,6 +54,7 @@ __global__ void __launch_bounds__(512) k_hg_zmarch(StepArgs a, HGLayout lay, int
 
 // ------------------------------------------------------------ E launches
 
+template <bool KEEP>
 __global__ void __launch_bounds__(512, 2) k_e_3d(StepArgs a) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -68,17 +69,18 @@ __global__ void __launch_bounds__(512, 2) k_e_3d(StepArgs a) {
     if (valid) {
         const uint32_t c = (uint32_t)i + (uint32_t)a.g.nx * j + a.g.nxy * k;
         const HNb h = load_h_nbrs(a, i, j, k, c);
-        if (face) e_core<true, true>(a, i, j, k, c, h, n, fl);
-        else if (pml) e_core<false, true>(a, i, j, k, c, h, n, fl);
-        else e_core<false, false>(a, i, j, k, c, h, n, fl);
+        if (face) e_core<true, true, KEEP>(a, i, j, k, c, h, n, fl);
+        else if (pml) e_core<false, true, KEEP>(a, i, j, k, c, h, n, fl);
+        else e_core<false, false, KEEP>(a, i, j, k, c, h, n, fl);
     }
     if (face) flux_warp_reduce(a.flux, fl, warp_slot());
     finish_step(a);
 }
 
+template <bool KEEP>
 __global__ void __launch_bounds__(512, 2) k_e_zmarch(StepArgs a, int kz) {
     const long long n = a.step_ctr[0];
-    e_tile_zmarch(a, blockIdx.x, blockIdx.y, blockIdx.z, kz, n, warp_slot());
+    e_tile_zmarch<KEEP>(a, blockIdx.x, blockIdx.y, blockIdx.z, kz, n, warp_slot());
     finish_step(a);
 }
 
@@ -289,7 +291,7 @@ bool vec_supported(const StepArgs& a) { return a.g.nx % 4 == 0; }
 // complete on per-slot mbarriers, S - 1 planes ahead of the compute.  The
 // -z neighbour plane of Hx, Hy stays in registers; J and n of gain cells
 // are loaded one plane ahead, once that plane's material tile has landed.
-template <int BX, int BY, int S>
+template <int BX, int BY, int S, bool KEEP>
 __global__ void __launch_bounds__(BX * BY) k_e_tma(StepArgs a, const __grid_constant__ TmaMaps maps,
                                                    int kz) {
     using Lay = TmaLayoutE<BX, BY>;
@@ -407,13 +409,13 @@ __global__ void __launch_bounds__(BX * BY) k_e_tma(StepArgs a, const __grid_cons
                 n3 = *gslot(b, 5);
             }
             if (fk)
-                e_apply<true, true>(a, i, j, k, c, h, m, Ex[tid], Ey[tid], Ez[tid], pg, jx, jy, jz, n1,
+                e_apply<true, true, KEEP>(a, i, j, k, c, h, m, Ex[tid], Ey[tid], Ez[tid], pg, jx, jy, jz, n1,
                                     n2, n3, n, fl);
             else if (w_pml || plane_in_z_slab(a, k))
-                e_apply<false, true>(a, i, j, k, c, h, m, Ex[tid], Ey[tid], Ez[tid], pg, jx, jy, jz, n1,
+                e_apply<false, true, KEEP>(a, i, j, k, c, h, m, Ex[tid], Ey[tid], Ez[tid], pg, jx, jy, jz, n1,
                                      n2, n3, n, fl);
             else
-                e_apply<false, false>(a, i, j, k, c, h, m, Ex[tid], Ey[tid], Ez[tid], pg, jx, jy, jz,
+                e_apply<false, false, KEEP>(a, i, j, k, c, h, m, Ex[tid], Ey[tid], Ez[tid], pg, jx, jy, jz,
                                       n1, n2, n3, n, fl);
             hx_km1 = h.hx;
             hy_km1 = h.hy;
@@ -612,17 +614,23 @@ void launch_h_pass(const StepArgs& a, const PassTune& t, const TmaMaps* tma, cud
     }
 }
 
-template <int BX, int BY>
-static void launch_e_tma(const StepArgs& a, const PassTune& t, const TmaMaps& maps, cudaStream_t s) {
+template <int BX, int BY, bool KEEP>
+static void launch_e_tma_as(const StepArgs& a, const PassTune& t, const TmaMaps& maps, cudaStream_t s) {
     const int smem = TmaLayoutE<BX, BY>::smem_bytes(kTmaStages);
     static bool attr_set = false;   // per instantiation, once per process
     if (!attr_set) {
-        cudaFuncSetAttribute(k_e_tma<BX, BY, kTmaStages>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(k_e_tma<BX, BY, kTmaStages, KEEP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              smem);
         attr_set = true;
     }
     dim3 grid((a.g.nx + BX - 1) / BX, (a.g.ny + BY - 1) / BY, (a.g.nz + t.kz - 1) / t.kz);
-    k_e_tma<BX, BY, kTmaStages><<<grid, dim3(BX, BY, 1), smem, s>>>(a, maps, t.kz);
+    k_e_tma<BX, BY, kTmaStages, KEEP><<<grid, dim3(BX, BY, 1), smem, s>>>(a, maps, t.kz);
+}
+
+template <int BX, int BY>
+static void launch_e_tma(const StepArgs& a, const PassTune& t, const TmaMaps& maps, cudaStream_t s) {
+    if (a.keep) launch_e_tma_as<BX, BY, true>(a, t, maps, s);
+    else launch_e_tma_as<BX, BY, false>(a, t, maps, s);
 }
 
 bool tma_e_supported(const StepArgs& a) {
@@ -694,11 +702,14 @@ void launch_e_pass(const StepArgs& a, const PassTune& t, const TmaMaps* tma, cud
     } else if (t.variant != kVariant3D) {
         dim3 grid((a.g.nx + t.block.x - 1) / t.block.x, (a.g.ny + t.block.y - 1) / t.block.y,
                   (a.g.nz + t.kz - 1) / t.kz);
-        k_e_zmarch<<<grid, dim3(t.block.x, t.block.y, 1), 0, s>>>(a, t.kz);
+        const dim3 b(t.block.x, t.block.y, 1);
+        if (a.keep) k_e_zmarch<true><<<grid, b, 0, s>>>(a, t.kz);
+        else k_e_zmarch<false><<<grid, b, 0, s>>>(a, t.kz);
     } else {
         dim3 grid((a.g.nx + t.block.x - 1) / t.block.x, (a.g.ny + t.block.y - 1) / t.block.y,
                   (a.g.nz + t.block.z - 1) / t.block.z);
-        k_e_3d<<<grid, t.block, 0, s>>>(a);
+        if (a.keep) k_e_3d<true><<<grid, t.block, 0, s>>>(a);
+        else k_e_3d<false><<<grid, t.block, 0, s>>>(a);
     }
 }
 

@@ -207,6 +207,7 @@ __device__ __forceinline__ void finish_step(const StepArgs& a, long long* sample
             atomicExch((unsigned long long*)(a.step_ctr + 1), 0ULL);
             const unsigned long long prev = atomicAdd((unsigned long long*)a.step_ctr, 1ULL);
             if (sample) *sample = (long long)prev + 1;
+            if (a.keep) *a.keep_n = (long long)prev + 1;
         }
     }
 }
@@ -215,7 +216,7 @@ __device__ __forceinline__ void finish_step(const StepArgs& a, long long* sample
 // face-plane cells (flux terms summed into fl over the walk, taken on the
 // planes plane_has_flux names; w_xy is warp-uniform); PML_XY: the tile
 // touches an x or y CPML slab (else only z-slab planes take the CPML code).
-template <bool FACE, bool PML_XY>
+template <bool FACE, bool PML_XY, bool KEEP = false>
 __device__ __forceinline__ void e_walk(const StepArgs& a, int i, int j, int k0, int k1, long long n,
                                        float fl[6], bool w_xy = false) {
     const int nx = a.g.nx;
@@ -240,10 +241,10 @@ __device__ __forceinline__ void e_walk(const StepArgs& a, int i, int j, int k0, 
         h.hz_j = (j > 0) ? __ldg(Hz + c - nx) : 0.0f;
         h.hy_i = (i > 0) ? __ldg(Hy + c - 1) : 0.0f;
         h.hz_i = (i > 0) ? __ldg(Hz + c - 1) : 0.0f;
-        if (FACE || PML_XY) e_core<FACE, true>(a, i, j, k, c, h, n, fl,
+        if (FACE || PML_XY) e_core<FACE, true, KEEP>(a, i, j, k, c, h, n, fl,
                                                !FACE || plane_has_flux(a.flux, true, w_xy, k));
-        else if (plane_in_z_slab(a, k)) e_core<false, true>(a, i, j, k, c, h, n, fl);
-        else e_core<false, false>(a, i, j, k, c, h, n, fl);
+        else if (plane_in_z_slab(a, k)) e_core<false, true, KEEP>(a, i, j, k, c, h, n, fl);
+        else e_core<false, false, KEEP>(a, i, j, k, c, h, n, fl);
         hx_km1 = h.hx;
         hy_km1 = h.hy;
     }
@@ -251,6 +252,7 @@ __device__ __forceinline__ void e_walk(const StepArgs& a, int i, int j, int k0, 
 
 // E walk of tile (bx, by, bz) for step n (flux of face tiles included).
 // Every thread of the block must call it (warp-wide flux reduction).
+template <bool KEEP = false>
 __device__ __forceinline__ void e_tile_zmarch(const StepArgs& a, int bx, int by, int bz, int kz,
                                               long long n, unsigned slot) {
     const int i = bx * blockDim.x + threadIdx.x;
@@ -265,12 +267,12 @@ __device__ __forceinline__ void e_tile_zmarch(const StepArgs& a, int bx, int by,
     if (face) {
         float fl[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         const bool w_xy = __any_sync(0xffffffffu, valid && cells_on_xy_face(a.flux, i, 1, j));
-        if (valid) e_walk<true, true>(a, i, j, k0, k1, n, fl, w_xy);
+        if (valid) e_walk<true, true, KEEP>(a, i, j, k0, k1, n, fl, w_xy);
         flux_warp_reduce(a.flux, fl, slot);
     } else if (valid) {
         float* none = nullptr;
-        if (pml_xy) e_walk<false, true>(a, i, j, k0, k1, n, none);
-        else e_walk<false, false>(a, i, j, k0, k1, n, none);
+        if (pml_xy) e_walk<false, true, KEEP>(a, i, j, k0, k1, n, none);
+        else e_walk<false, false, KEEP>(a, i, j, k0, k1, n, none);
     }
 }
 
