@@ -332,14 +332,6 @@ void launch_probes(mb_ctx* c) { launch_probes(c, c->args, c->d_ctr, c->stream); 
 
 bool has_probes(const mb_ctx* c) { return !c->probes.empty() || c->face.on || !c->planes.empty(); }
 
-void sum_flux_slots(const double* slots, double fl[6]) {
-    for (int q = 0; q < 6; ++q) {
-        double v = 0.0;
-        for (int t = 0; t < mb::kFluxSlots; ++t) v += slots[q * mb::kFluxSlots + t];
-        fl[q] = v;
-    }
-}
-
 // Launches of one step: the field launches (2 for the two passes, 1 for the
 // single-pass step) plus the probes.
 int launches_per_step(const mb_ctx* c, bool fused) {
@@ -701,7 +693,7 @@ static int create_ctx(mb_ctx** out, const int grid[3], int gnz, int kz0, int own
     if ((rc = alloc((void**)&c->d_flux_out, sizeof(double) * 6))) return bail(rc);
     c->n_partial = 1024;
     if ((rc = alloc((void**)&c->d_partial, sizeof(double) * c->n_partial))) return bail(rc);
-    if ((rc = alloc((void**)&c->d_energy, sizeof(double)))) return bail(rc);
+    if ((rc = alloc((void**)&c->d_energy, sizeof(double) * 9))) return bail(rc);
     if ((rc = alloc((void**)&c->d_nonfinite, sizeof(int)))) return bail(rc);
     if ((rc = alloc((void**)&c->d_err, sizeof(int)))) return bail(rc);
 
@@ -807,7 +799,7 @@ int mb_destroy(mb_ctx* c) {
     void* bufs[] = {c->d_fields, c->d_mat, c->d_inv_eps, c->d_lut, c->d_psi[0], c->d_psi[1],
                     c->d_psi[2], c->d_coef, c->d_ctr, c->d_flux, c->d_partial, c->d_energy,
                     c->d_nonfinite, c->d_probe_cell, c->d_probe_omega, c->d_probe_acc,
-                    c->d_face_omega, c->d_face_acc, c->d_face_acc32, c->d_glist, c->d_glist_scratch,
+                    c->d_face_omega, c->d_face_acc, c->d_face_acc32, c->d_face_spec, c->d_plane_out, c->d_glist, c->d_glist_scratch,
                     c->d_upload, c->d_keys, c->d_src_wave, c->d_err,
                     c->d_fields2, c->d_psi2[0], c->d_psi2[1], c->d_psi2[2], c->d_flux_out, c->d_small,
                     c->d_small_x};
@@ -1022,6 +1014,7 @@ int mb_add_face_probes(mb_ctx* c, int stride, int every, int n_freq, double lam_
     if (c->d_face_acc) { cudaFree(c->d_face_acc); c->d_face_acc = nullptr; }
     if (c->d_face_acc32) { cudaFree(c->d_face_acc32); c->d_face_acc32 = nullptr; }
     if (c->d_face_omega) { cudaFree(c->d_face_omega); c->d_face_omega = nullptr; }
+    if (c->d_face_spec) { cudaFree(c->d_face_spec); c->d_face_spec = nullptr; }
     mb::DevFaceProbes& F = c->face;
     std::memset(&F, 0, sizeof(F));
     const int n3[3] = {c->nx, c->ny, c->nz};
@@ -1087,6 +1080,7 @@ int mb_add_face_probes(mb_ctx* c, int stride, int every, int n_freq, double lam_
     MB_CUDA(c, cudaMemset(c->d_face_acc, 0, sizeof(double2) * (accn ? accn : 1)));
     MB_CUDA(c, cudaMalloc((void**)&c->d_face_acc32, sizeof(float2) * (accn ? accn : 1)));
     MB_CUDA(c, cudaMemset(c->d_face_acc32, 0, sizeof(float2) * (accn ? accn : 1)));
+    MB_CUDA(c, cudaMalloc((void**)&c->d_face_spec, sizeof(double) * (mb::kFaceSpecChunks + 1) * (size_t)n_freq));
     F.omega = c->d_face_omega;
     F.acc = c->d_face_acc;
     F.acc32 = c->d_face_acc32;
@@ -1233,16 +1227,11 @@ int mb_plane_energy_density(mb_ctx* c, int k, double* out) {
     if (int rc = check_ctx(c)) return rc;
     if (k < 0 || k >= c->nz || !out) return fail(c, MB_ERR_ARG, "bad plane");
     const size_t nxy = (size_t)c->nx * c->ny;
-    double* d = nullptr;
-    MB_CUDA(c, cudaMalloc((void**)&d, sizeof(double) * nxy));
-    mb::launch_plane_energy(c->args.f, c->args.g, k, c->d_lut + 128, d, c->stream);
-    cudaError_t e = cudaMemcpyAsync(out, d, sizeof(double) * nxy, cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    cudaFree(d);
-    if (e != cudaSuccess) return fail(c, MB_ERR_CUDA, cudaGetErrorString(e));
-    const double u0 = kEps0 * c->E0 * c->E0;
-    for (size_t p = 0; p < nxy; ++p) out[p] *= u0;
-    return check_device_error(c);
+    if (!c->d_plane_out) MB_CUDA(c, cudaMalloc((void**)&c->d_plane_out, sizeof(double) * nxy));
+    mb::launch_plane_energy(c->args.f, c->args.g, k, c->d_lut + 128, kEps0 * c->E0 * c->E0, c->d_plane_out,
+                            c->stream);
+    MB_CUDA(c, cudaMemcpyAsync(out, c->d_plane_out, sizeof(double) * nxy, cudaMemcpyDeviceToHost, c->stream));
+    return check_device_error(c);   // (waits for the stream)
 }
 
 // The six face energies (J) summed and scaled on the device into d_flux_out.
@@ -1339,36 +1328,19 @@ int mb_face_spectrum(mb_ctx* c, int face, double* out_S, double* out_lam) {
     if (!c->face.on) return fail(c, MB_ERR_STATE, "no face probes");
     if (face < 0 || face > 5 || !out_S) return fail(c, MB_ERR_ARG, "bad face or null output");
     const int K = c->face.nfreq;
-    const int np = c->face.npts[face];
-    std::vector<double2> acc((size_t)np * 4 * K);
-    std::vector<float2> acc32((size_t)np * 4 * K);
-    if (np) {
-        const size_t at = (size_t)c->face.offset[face] * 4 * K;
-        MB_CUDA(c, cudaMemcpyAsync(acc.data(), c->d_face_acc + at, sizeof(double2) * acc.size(),
-                                   cudaMemcpyDeviceToHost, c->stream));
-        MB_CUDA(c, cudaMemcpyAsync(acc32.data(), c->d_face_acc32 + at, sizeof(float2) * acc32.size(),
-                                   cudaMemcpyDeviceToHost, c->stream));
-        MB_CUDA(c, cudaStreamSynchronize(c->stream));
-        // the FP64 sums plus the FP32 sums since their last flush
-        for (size_t q = 0; q < acc.size(); ++q) {
-            acc[q].x += (double)acc32[q].x;
-            acc[q].y += (double)acc32[q].y;
-        }
-    }
     const double w = c->face.every * c->dt;
     const double scale = (c->E0 * w) * (c->E0 / c->eta0 * w) * std::pow(c->face.stride * c->dx, 2);
     const double sign = (face % 2) ? 1.0 : -1.0;
-    for (int k = 0; k < K; ++k) {
-        double s = 0.0;
-        for (int q = 0; q < np; ++q) {
-            const double2 Ea = acc[((size_t)q * 4 + 0) * K + k], Eb = acc[((size_t)q * 4 + 1) * K + k];
-            const double2 Ha = acc[((size_t)q * 4 + 2) * K + k], Hb = acc[((size_t)q * 4 + 3) * K + k];
-            // Re(Ea conj(Hb) - Eb conj(Ha))
-            s += (Ea.x * Hb.x + Ea.y * Hb.y) - (Eb.x * Ha.x + Eb.y * Ha.y);
-        }
-        out_S[k] = sign * s * scale;
-        if (out_lam) out_lam[k] = c->face_lam[k];
+    if (c->face.npts[face]) {
+        double* res = c->d_face_spec + (size_t)mb::kFaceSpecChunks * K;
+        mb::launch_face_spectrum(c->face, face, sign * scale, c->d_face_spec, res, c->stream);
+        MB_CUDA(c, cudaGetLastError());
+        MB_CUDA(c, cudaMemcpyAsync(out_S, res, sizeof(double) * K, cudaMemcpyDeviceToHost, c->stream));
+        MB_CUDA(c, cudaStreamSynchronize(c->stream));
+    } else {
+        std::fill(out_S, out_S + K, 0.0);
     }
+    if (out_lam) std::copy(c->face_lam.begin(), c->face_lam.end(), out_lam);
     return MB_OK;
 }
 
@@ -1385,23 +1357,19 @@ int mb_energy(mb_ctx* c, double* out_U, double* out_flux6) {
         *q += off;
     f.mat += off;
     if (f.inv_eps) f.inv_eps += off;
-    mb::launch_energy(f, own, c->d_lut + 128, c->d_partial, c->n_partial, c->d_nonfinite,
+    mb::launch_energy(f, own, c->d_lut + 128, c->d_partial, c->n_partial, c->d_nonfinite, c->d_flux, c->d_err,
                       c->d_energy, c->stream);
     MB_CUDA(c, cudaGetLastError());
-    double U = 0, slots[6 * mb::kFluxSlots], fl[6];
-    int bad = 0;
-    MB_CUDA(c, cudaMemcpyAsync(&U, c->d_energy, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    MB_CUDA(c, cudaMemcpyAsync(slots, c->d_flux, sizeof(slots), cudaMemcpyDeviceToHost, c->stream));
-    MB_CUDA(c, cudaMemcpyAsync(&bad, c->d_nonfinite, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    double r[9];   // the sum, the faces, the flags
+    MB_CUDA(c, cudaMemcpyAsync(r, c->d_energy, sizeof(r), cudaMemcpyDeviceToHost, c->stream));
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
-    sum_flux_slots(slots, fl);
-    *out_U = 0.5 * kEps0 * c->E0 * c->E0 * c->dx * c->dx * c->dx * U;
+    *out_U = 0.5 * kEps0 * c->E0 * c->E0 * c->dx * c->dx * c->dx * r[0];
     if (out_flux6) {
         const double f = c->dt * c->E0 * (c->E0 / c->eta0) * c->dx * c->dx;
-        for (int q = 0; q < 6; ++q) out_flux6[q] = fl[q] * f;
+        for (int q = 0; q < 6; ++q) out_flux6[q] = r[1 + q] * f;
     }
-    if (bad) return fail(c, MB_ERR_NONFINITE, "non-finite field values");
-    return check_device_error(c);
+    if (r[7] != 0.0) return fail(c, MB_ERR_NONFINITE, "non-finite field values");
+    return r[8] != 0.0 ? check_device_error(c) : MB_OK;
 }
 
 int mb_gain_list(mb_ctx* c, uint32_t* host_out, int64_t* count) {

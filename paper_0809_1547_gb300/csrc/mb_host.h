@@ -254,9 +254,14 @@ int batch_blocks_per_sm(dim3 block);
 
 void launch_plane_dft(const DevPlaneProbe& pp, const DevFields& f, const DevGrid& g,
                       const long long* ctr, double dt, cudaStream_t s);
-// Energy density of the cells of plane z = k in units of eps0 E0^2 (FP64).
-void launch_plane_energy(const DevFields& f, const DevGrid& g, int k, const float* lut_eps,
+// Energy density of the cells of plane z = k in units of eps0 E0^2 / u0 (FP64).
+void launch_plane_energy(const DevFields& f, const DevGrid& g, int k, const float* lut_eps, double u0,
                          double* out, cudaStream_t s);
+// The outward spectrum of a face (nfreq doubles) into out; scratch holds
+// kFaceSpecChunks * nfreq doubles.
+constexpr int kFaceSpecChunks = 64;
+void launch_face_spectrum(const DevFaceProbes& fp, int face, double scale, double* scratch, double* out,
+                          cudaStream_t s);
 void launch_philox(const uint4* ctr, uint32_t k0, uint32_t k1, uint4* out, int n, cudaStream_t s);
 // out[q] = scale * sum_t slots[q kFluxSlots + t] (slots in order), q < 6.
 void launch_flux_sum(const double* slots, double* out, double scale, cudaStream_t s);
@@ -281,7 +286,8 @@ void launch_mat_keys(const float* eps, int64_t N, uint32_t* keys, uint32_t* firs
 void launch_mat_ids(const float* eps, const uint8_t* gain, int64_t N, const uint32_t* keys, int n,
                     bool dense, bool gain_on, uint8_t* mat, float* inv_eps, cudaStream_t s);
 void launch_energy(const DevFields& f, int64_t ncell, const float* lut_eps, double* partial,
-                   int nparts, int* nonfinite, double* out, cudaStream_t s);
+                   int nparts, int* nonfinite, const double* slots, const int* err, double* out,
+                   cudaStream_t s);
 
 // Message returned by mb_last_error(NULL) on this thread.
 void set_thread_error(const std::string& msg);
@@ -391,6 +397,8 @@ struct mb_ctx {
     double* d_face_omega = nullptr;
     double2* d_face_acc = nullptr;
     float2* d_face_acc32 = nullptr;
+    double* d_face_spec = nullptr;     // face spectrum: partial sums, then the result
+    double* d_plane_out = nullptr;     // plane energy density (read-back staging, made on first use)
     int64_t face_points = 0;
 
     // material

@@ -6,12 +6,14 @@
 //   k_plane_dft   running DFT of E on a whole z-plane (mode maps)
 //   k_plane_energy  energy density of the cells of a z-plane (snapshots)
 //   k_energy_*    two-pass deterministic reduction of the field energy
+//   k_face_spectrum  outward spectrum of a face from its points' sums
 //   k_philox      the noise generator on given counters
 //
 // The probes run after the E pass of step n, whose last block has already
 // advanced the step counter to n + 1: E^{n+1} is sampled at t_{n+1}.
 #include "mb_host.h"
 
+#include <algorithm>
 #include <cstdio>
 
 namespace mb {
@@ -112,48 +114,114 @@ __global__ void __launch_bounds__(256) k_face_dft(DevFaceProbes fp, DevFields f,
     }
 }
 
-// Energy, pass 1: per-block partial sums of eps_r |E_s|^2 + |H_s|^2 (FP64)
-// into `partial` (one double per block), non-finite values flagged.
+__device__ __forceinline__ double block_sum(double acc) {
+    __shared__ double red[32];
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (lane == 0) red[warp] = acc;
+    __syncthreads();
+    if (warp == 0) {
+        acc = (lane < (int)(blockDim.x >> 5)) ? red[lane] : 0.0;
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    }
+    return acc;
+}
+
+// Energy, pass 1: per-block partial sums of eps_r |E_s|^2 + |H_s|^2 into
+// `partial` (one double per block), non-finite values flagged.  VEC: four
+// cells per thread and pass in 16-byte loads (every array 16-byte aligned).
+template <bool VEC>
 __global__ void __launch_bounds__(256) k_energy_partial(DevFields f, int64_t ncell,
                                                         const float* lut_eps, double* partial,
                                                         int* nonfinite) {
-    double acc = 0.0;
+    PairSum acc;
+    double dense = 0.0;   // a dense map holds 1/eps_r: its cells divide in FP64
     bool bad = false;
-    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncell;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        const float e2 = f.ex[c] * f.ex[c] + f.ey[c] * f.ey[c] + f.ez[c] * f.ez[c];
-        const float h2 = f.hx[c] * f.hx[c] + f.hy[c] * f.hy[c] + f.hz[c] * f.hz[c];
-        const double eps = f.inv_eps ? 1.0 / (double)f.inv_eps[c] : (double)lut_eps[f.mat[c] & 0x7f];
-        const double v = eps * (double)e2 + (double)h2;
+    auto one = [&](float ex, float ey, float ez, float hx, float hy, float hz, uint8_t m, int64_t c) {
+        const float e2 = ex * ex + ey * ey + ez * ez;
+        const float h2 = hx * hx + hy * hy + hz * hz;
         bad |= !isfinite(e2) || !isfinite(h2);
-        acc += v;
+        if (f.inv_eps) dense += 1.0 / (double)f.inv_eps[c] * (double)e2 + (double)h2;
+        else acc.cell(__ldg(lut_eps + (m & 0x7f)), e2, h2);
+    };
+    const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+    if (VEC) {
+        auto at4 = [](const float* p, int64_t q) { return __ldg(reinterpret_cast<const float4*>(p) + q); };
+        for (int64_t q = t0; q < ncell / 4; q += stride) {
+            const float4 ex = at4(f.ex, q), ey = at4(f.ey, q), ez = at4(f.ez, q);
+            const float4 hx = at4(f.hx, q), hy = at4(f.hy, q), hz = at4(f.hz, q);
+            const uchar4 m = __ldg(reinterpret_cast<const uchar4*>(f.mat) + q);
+            one(ex.x, ey.x, ez.x, hx.x, hy.x, hz.x, m.x, 4 * q);
+            one(ex.y, ey.y, ez.y, hx.y, hy.y, hz.y, m.y, 4 * q + 1);
+            one(ex.z, ey.z, ez.z, hx.z, hy.z, hz.z, m.z, 4 * q + 2);
+            one(ex.w, ey.w, ez.w, hx.w, hy.w, hz.w, m.w, 4 * q + 3);
+        }
     }
-    __shared__ double red[32];
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) red[warp] = acc;
-    __syncthreads();
-    if (warp == 0) {
-        acc = (lane < (int)(blockDim.x >> 5)) ? red[lane] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-        if (lane == 0) partial[blockIdx.x] = acc;
-    }
+    for (int64_t c = (VEC ? ncell / 4 * 4 : 0) + t0; c < ncell; c += stride)
+        one(f.ex[c], f.ey[c], f.ez[c], f.hx[c], f.hy[c], f.hz[c], f.mat[c], c);
+    const double v = block_sum(acc.value() + dense);
+    if (threadIdx.x == 0) partial[blockIdx.x] = v;
     if (bad) atomicOr(nonfinite, 1);
 }
 
-// Energy, pass 2: one block sums the partials in a fixed order.
-__global__ void k_energy_final(const double* partial, int nparts, double* out) {
-    __shared__ double red[32];
+// Energy, pass 2: one block sums the partials in a fixed order, and the face
+// slots, into out: [0] the energy sum, [1..6] the faces, [7] the non-finite
+// flag, [8] the device error flag (one copy brings all of it to the host).
+__global__ void k_energy_final(const double* partial, int nparts, const double* slots, const int* nonfinite,
+                               const int* err, double* out) {
     double acc = 0.0;
     for (int q = threadIdx.x; q < nparts; q += blockDim.x) acc += partial[q];
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    acc = block_sum(acc);
+    if (threadIdx.x == 0) {
+        out[0] = acc;
+        out[7] = *nonfinite ? 1.0 : 0.0;
+        out[8] = *err ? 1.0 : 0.0;
+    }
+    const int q = (int)threadIdx.x - 32;   // faces: the slots in order
+    if (q >= 0 && q < 6) {
+        double v = 0.0;
+        for (int t = 0; t < kFluxSlots; ++t) v += slots[q * kFluxSlots + t];
+        out[1 + q] = v;
+    }
+}
+
+// Face spectrum: block (group of 32 bins, chunk of points), a warp per point
+// in turn: partial[chunk][bin] = sum over the chunk's points of
+// Re(Ea conj(Hb) - Eb conj(Ha)) with the FP64 sums plus the FP32 sums since
+// their last flush.  On the device because the sums are 6 x 3 MB at 160^3
+// (six copies and 1.3 M host terms took 3.3 ms) and the result 1 KB.
+__global__ void __launch_bounds__(256) k_face_spectrum(DevFaceProbes fp, int face, int chunks, double* partial) {
+    __shared__ double red[8][32];
+    const int K = fp.nfreq, np = fp.npts[face];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) red[warp] = acc;
+    const int kk = blockIdx.x * 32 + lane;
+    const int p0 = (int)((int64_t)np * blockIdx.y / chunks), p1 = (int)((int64_t)np * (blockIdx.y + 1) / chunks);
+    double s = 0.0;
+    if (kk < K)
+        for (int p = p0 + warp; p < p1; p += 8) {
+            const int64_t at = ((int64_t)(fp.offset[face] + p) * 4) * K + kk;
+            double2 v[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const double2 d = fp.acc[at + (int64_t)r * K];
+                const float2 e = fp.acc32[at + (int64_t)r * K];
+                v[r] = make_double2(d.x + (double)e.x, d.y + (double)e.y);
+            }
+            s += (v[0].x * v[3].x + v[0].y * v[3].y) - (v[1].x * v[2].x + v[1].y * v[2].y);
+        }
+    red[warp][lane] = s;
     __syncthreads();
-    if (warp == 0) {
-        acc = (lane < (int)(blockDim.x >> 5)) ? red[lane] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-        if (lane == 0) *out = acc;
+    if (warp == 0 && kk < K) {
+        for (int w = 1; w < 8; ++w) s += red[w][lane];
+        partial[(size_t)blockIdx.y * K + kk] = s;
+    }
+}
+// out[k] = scale * sum over the chunks, in order.
+__global__ void k_face_spectrum_sum(const double* partial, int chunks, int K, double scale, double* out) {
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < K; k += gridDim.x * blockDim.x) {
+        double s = 0.0;
+        for (int c = 0; c < chunks; ++c) s += partial[(size_t)c * K + k];
+        out[k] = s * scale;
     }
 }
 
@@ -222,15 +290,15 @@ __global__ void k_plane_dft(DevPlaneProbe pp, DevFields f, DevGrid g, const long
     }
 }
 
-// Energy density of plane z = k: (eps_r |E|^2 + |H|^2) / 2 in units of eps0 E0^2.
-__global__ void k_plane_energy(DevFields f, DevGrid g, int k, const float* lut_eps, double* out) {
+// Energy density of plane z = k in J/m^3: u0 (eps_r |E|^2 + |H|^2) / 2.
+__global__ void k_plane_energy(DevFields f, DevGrid g, int k, const float* lut_eps, double u0, double* out) {
     const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= g.nxy) return;
     const uint32_t c = p + g.nxy * (uint32_t)k;
     const double eps = f.inv_eps ? 1.0 / (double)f.inv_eps[c] : (double)lut_eps[f.mat[c] & 0x7f];
     const double ex = f.ex[c], ey = f.ey[c], ez = f.ez[c];
     const double hx = f.hx[c], hy = f.hy[c], hz = f.hz[c];
-    out[p] = 0.5 * (eps * (ex * ex + ey * ey + ez * ez) + (hx * hx + hy * hy + hz * hz));
+    out[p] = 0.5 * (eps * (ex * ex + ey * ey + ez * ez) + (hx * hx + hy * hy + hz * hz)) * u0;
 }
 
 void launch_plane_dft(const DevPlaneProbe& pp, const DevFields& f, const DevGrid& g,
@@ -239,10 +307,19 @@ void launch_plane_dft(const DevPlaneProbe& pp, const DevFields& f, const DevGrid
     k_plane_dft<<<blocks, 256, 0, s>>>(pp, f, g, ctr, dt);
 }
 
-void launch_plane_energy(const DevFields& f, const DevGrid& g, int k, const float* lut_eps,
+void launch_plane_energy(const DevFields& f, const DevGrid& g, int k, const float* lut_eps, double u0,
                          double* out, cudaStream_t s) {
     const unsigned blocks = (g.nxy + 255) / 256;
-    k_plane_energy<<<blocks, 256, 0, s>>>(f, g, k, lut_eps, out);
+    k_plane_energy<<<blocks, 256, 0, s>>>(f, g, k, lut_eps, u0, out);
+}
+
+int face_spectrum_chunks(int np) { return std::max(1, std::min(kFaceSpecChunks, np / 8)); }
+
+void launch_face_spectrum(const DevFaceProbes& fp, int face, double scale, double* scratch, double* out,
+                          cudaStream_t s) {
+    const int chunks = face_spectrum_chunks(fp.npts[face]);
+    k_face_spectrum<<<dim3((fp.nfreq + 31) / 32, chunks, 1), 256, 0, s>>>(fp, face, chunks, scratch);
+    k_face_spectrum_sum<<<(fp.nfreq + 127) / 128, 128, 0, s>>>(scratch, chunks, fp.nfreq, scale, out);
 }
 
 __global__ void k_flux_sum(const double* slots, double* out, double scale) {
@@ -560,9 +637,12 @@ void launch_flux_sum(const double* slots, double* out, double scale, cudaStream_
 }
 
 void launch_energy(const DevFields& f, int64_t ncell, const float* lut_eps, double* partial,
-                   int nparts, int* nonfinite, double* out, cudaStream_t s) {
-    k_energy_partial<<<nparts, 256, 0, s>>>(f, ncell, lut_eps, partial, nonfinite);
-    k_energy_final<<<1, 1024, 0, s>>>(partial, nparts, out);
+                   int nparts, int* nonfinite, const double* slots, const int* err, double* out, cudaStream_t s) {
+    bool vec = reinterpret_cast<uintptr_t>(f.mat) % 4 == 0;
+    for (const float* p : {f.ex, f.ey, f.ez, f.hx, f.hy, f.hz}) vec = vec && reinterpret_cast<uintptr_t>(p) % 16 == 0;
+    if (vec) k_energy_partial<true><<<nparts, 256, 0, s>>>(f, ncell, lut_eps, partial, nonfinite);
+    else k_energy_partial<false><<<nparts, 256, 0, s>>>(f, ncell, lut_eps, partial, nonfinite);
+    k_energy_final<<<1, 1024, 0, s>>>(partial, nparts, slots, nonfinite, err, out);
 }
 
 }  // namespace mb

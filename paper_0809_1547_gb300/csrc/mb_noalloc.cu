@@ -68,22 +68,23 @@ bool current_context_id(unsigned long long* id) {
     return get_id(ctx, id) == CUDA_SUCCESS;
 }
 
-// Pass 1: block b sums w |E|^2 + |H|^2 over cells [b C, (b+1) C) in FP64.
+// Pass 1: block b sums w |E|^2 + |H|^2 over cells [b C, (b+1) C) (PairSum per
+// thread, FP64 across threads).
 __global__ void __launch_bounds__(kNoAllocThreads)
 k_energy_partial_static(const float* ex, const float* ey, const float* ez, const float* hx,
                         const float* hy, const float* hz, const float* eps_r, int64_t ncell,
                         NoAllocScratch* scratch) {
     const int64_t begin = blockIdx.x * kNoAllocCellsPerBlock;
     const int64_t end = begin + kNoAllocCellsPerBlock < ncell ? begin + kNoAllocCellsPerBlock : ncell;
-    double acc = 0.0;
+    mb::PairSum sum;
     bool bad = false;
     for (int64_t c = begin + threadIdx.x; c < end; c += kNoAllocThreads) {
         const float e2 = ex[c] * ex[c] + ey[c] * ey[c] + ez[c] * ez[c];
         const float h2 = hx[c] * hx[c] + hy[c] * hy[c] + hz[c] * hz[c];
-        const double w = eps_r ? (double)eps_r[c] : 1.0;
         bad |= !isfinite(e2) || !isfinite(h2);
-        acc += w * (double)e2 + (double)h2;
+        sum.cell(eps_r ? eps_r[c] : 1.0f, e2, h2);
     }
+    double acc = sum.value();
     __shared__ double red[kNoAllocThreads / 32];
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
