@@ -206,7 +206,11 @@ int capture_steps(mb_ctx* c, int steps, int p, bool fused, cudaGraphExec_t* out)
     // which step s + 1 only reads, so they run on the second stream beside
     // step s + 1; step s + 2 (which rewrites that copy) waits for them, and
     // the chunk ends with the second stream joined.
-    const bool fork = fused && has_probes(c) && c->aux_stream;
+    // Two-pass steps: point and plane probes read only E, which the next
+    // step's H pass reads too, so they run beside it; its E pass waits (a
+    // point probe's launch is 6.5 us of dependent latencies, 6 % of a 139^3
+    // step).  Face probes also read H, which the H pass rewrites: in line.
+    const bool fork = has_probes(c) && c->aux_stream && (fused || (steps > 1 && !c->face.on));
     if (fork) ensure_events(c, steps);
     cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
@@ -227,8 +231,17 @@ int capture_steps(mb_ctx* c, int steps, int p, bool fused, cudaGraphExec_t* out)
                 p = 1 - p;
             } else {
                 mb::launch_h_pass(c->args, c->tune_h, mh, c->stream);
+                if (fork && s >= 1) cudaStreamWaitEvent(c->stream, c->join_ev[s - 1], 0);
                 mb::launch_e_pass(c->args, c->tune_e, me, c->stream);
-                launch_probes(c);
+                if (fork) {
+                    // the counter the probes sample is advanced by the E passes alone
+                    cudaEventRecord(c->fork_ev[s], c->stream);
+                    cudaStreamWaitEvent(c->aux_stream, c->fork_ev[s], 0);
+                    launch_probes(c, c->args, c->d_ctr, c->aux_stream);
+                    cudaEventRecord(c->join_ev[s], c->aux_stream);
+                } else {
+                    launch_probes(c);
+                }
             }
         }
         if (fork) cudaStreamWaitEvent(c->stream, c->join_ev[steps - 1], 0);
