@@ -98,13 +98,13 @@ __device__ __forceinline__ void adj_point_cell(const AdjArgs& a, int i, int j, i
     gw = 0.0f;
     if (valid) {
         const uint32_t N = a.g.ncell;
-        const uint32_t c = (uint32_t)i + (uint32_t)a.g.nx * j + a.g.nxy * k;
+        const uint32_t c = cell_place(a.g, i, j, k);
         const float e0x = __ldcs(a.x0.ex + c), e0y = __ldcs(a.x0.ey + c), e0z = __ldcs(a.x0.ez + c);
         const float e1x = __ldcs(a.x1.ex + c), e1y = __ldcs(a.x1.ey + c), e1z = __ldcs(a.x1.ez + c);
         float l0x = 0.0f, l0y = 0.0f, l0z = 0.0f;
         // objective: mx Hy(k-1) - my Hx(k-1) on the plane k = zp
         if (k == a.zp && i >= a.rx0 && i < a.rx1 && j >= a.ry0 && j < a.ry1) {
-            const uint32_t cp = (uint32_t)i + (uint32_t)a.g.nx * j;
+            const uint32_t cp = (uint32_t)i + (uint32_t)a.g.px * j;
             const float hxk = __ldcs(a.x1.hpx + cp), hyk = __ldcs(a.x1.hpy + cp);
             l1x += 0.5f * hyk;
             l1y -= 0.5f * hxk;
@@ -205,7 +205,7 @@ __device__ __forceinline__ void adj_point_cell(const AdjArgs& a, int i, int j, i
             l0z += kE * tz;
             const float ldn = G.cJE * (e0x * tx + e0y * ty + e0z * tz);
             float z0, z1, z2;
-            langevin_normals(c, (uint32_t)*a.n_ptr, G.key0, G.key1, z0, z1, z2);
+            langevin_normals(cell_number(a.g, i, j, k), (uint32_t)*a.n_ptr, G.key0, G.key1, z0, z1, z2);
             const float damp = n2 > 0.0f ? 0.5f * G.cJN * rsqrtf(n2 + G.nfloor) : 0.0f;
             a.ln[c] = ln1 + ldn;
             a.ln[c + N] = ln2 - ldn + damp * (z0 * tx + z1 * ty + z2 * tz);
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(256) k_adj_point(AdjArgs a) {
     float l1x = 0.0f, l1y = 0.0f, l1z = 0.0f;
     if (valid) {
         const uint32_t N = a.g.ncell;
-        const uint32_t c = (uint32_t)i + (uint32_t)a.g.nx * j + a.g.nxy * k;
+        const uint32_t c = cell_place(a.g, i, j, k);
         l1x = a.le[c];
         l1y = a.le[c + N];
         l1z = a.le[c + 2 * N];
@@ -265,7 +265,7 @@ __device__ __forceinline__ WCoef w_coef(const AdjArgs& a, int i, int j, int k) {
     WCoef w{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (i >= a.g.nx || j >= a.g.ny || k >= a.g.nz) return w;
     const uint32_t N = a.g.ncell;
-    const uint32_t c = (uint32_t)i + (uint32_t)a.g.nx * j + a.g.nxy * k;
+    const uint32_t c = cell_place(a.g, i, j, k);
     const float S = a.S;
     const float ux = a.mu[c], uy = a.mu[c + N], uz = a.mu[c + 2 * N];
     w.xy = S * ux;
@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(256) k_adj_h(AdjArgs a) {
                                                        in_slab(k, nz, L) || in_slab(k + 1, nz, L)));
     if (!valid) return;
     const uint32_t N = a.g.ncell;
-    const uint32_t c = (uint32_t)i + (uint32_t)nx * j + a.g.nxy * k;
+    const uint32_t c = cell_place(a.g, i, j, k);
     float hx = a.lh[c], hy = a.lh[c + N], hz = a.lh[c + 2 * N];
     // objective: H sites of the layer k = zp - 1
     if (k + 1 == a.zp && i >= a.rx0 && i < a.rx1 && j >= a.ry0 && j < a.ry1) {
@@ -336,8 +336,8 @@ __global__ void __launch_bounds__(256) k_adj_h(AdjArgs a) {
             wi.zx = S * a.mu[c + 1 + 2 * N];
         }
         if (j + 1 < ny) {
-            wj.xy = S * a.mu[c + nx];
-            wj.zy = -S * a.mu[c + nx + 2 * N];
+            wj.xy = S * a.mu[c + a.g.px];
+            wj.zy = -S * a.mu[c + a.g.px + 2 * N];
         }
         if (k + 1 < nz) {
             wk.xz = -S * a.mu[c + a.g.nxy];
@@ -389,7 +389,7 @@ __device__ __forceinline__ WCoef v_coef(const AdjArgs& a, int i, int j, int k) {
     WCoef v{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (i < 0 || j < 0 || k < 0) return v;
     const uint32_t N = a.g.ncell;
-    const uint32_t c = (uint32_t)i + (uint32_t)a.g.nx * j + a.g.nxy * k;
+    const uint32_t c = cell_place(a.g, i, j, k);
     const float S = a.S;
     const float hx = a.lh[c], hy = a.lh[c + N], hz = a.lh[c + 2 * N];
     v.xy = -S * hx;
@@ -446,7 +446,7 @@ __device__ __forceinline__ void adj_e_gather(const AdjArgs& a, int i, int j, int
     WCoef v0, vi, vj, vk;
     if (!pml) {
         const float S = a.S;
-        const uint32_t nx = a.g.nx, nxy = a.g.nxy;
+        const uint32_t px = a.g.px, nxy = a.g.nxy;
         v0 = v_plain(S, a.lh[c], a.lh[c + N], a.lh[c + 2 * N]);
         vi = vj = vk = WCoef{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         if (i >= 1) {
@@ -454,8 +454,8 @@ __device__ __forceinline__ void adj_e_gather(const AdjArgs& a, int i, int j, int
             vi.yx = S * a.lh[c - 1 + N];
         }
         if (j >= 1) {
-            vj.zy = S * a.lh[c - nx + 2 * N];
-            vj.xy = -S * a.lh[c - nx];
+            vj.zy = S * a.lh[c - px + 2 * N];
+            vj.xy = -S * a.lh[c - px];
         }
         if (k >= 1) {
             vk.yz = -S * a.lh[c - nxy + N];
@@ -478,7 +478,7 @@ __global__ void __launch_bounds__(256) k_adj_e(AdjArgs a) {
     const int k = blockIdx.z;
     if (i >= a.g.nx || j >= a.g.ny) return;
     const uint32_t N = a.g.ncell;
-    const uint32_t c = (uint32_t)i + (uint32_t)a.g.nx * j + a.g.nxy * k;
+    const uint32_t c = cell_place(a.g, i, j, k);
     float lx, ly, lz;
     adj_e_gather(a, i, j, k, c, true, lx, ly, lz);
     a.le[c] = lx;
@@ -498,7 +498,7 @@ __global__ void __launch_bounds__(256, 6) k_adj_e_point(AdjArgs a) {
     const bool valid = i < a.g.nx && j < a.g.ny;
     const bool pml = __any_sync(0xffffffffu, valid && near_slab_lo(a, i, j, k));
     float lx = 0.0f, ly = 0.0f, lz = 0.0f;
-    if (valid) adj_e_gather(a, i, j, k, (uint32_t)i + (uint32_t)a.g.nx * j + a.g.nxy * k, pml, lx, ly, lz);
+    if (valid) adj_e_gather(a, i, j, k, cell_place(a.g, i, j, k), pml, lx, ly, lz);
     float obj, gw;
     adj_point_cell(a, i, j, k, valid, lx, ly, lz, obj, gw);
     const unsigned slot = block_slot();
@@ -545,10 +545,12 @@ __global__ void k_keep(const float* __restrict__ F, float* __restrict__ dst, uin
     }
 }
 
-// Output: grad[c] = scale * geps[c].
-__global__ void k_adj_out(const double* geps, float* out, uint32_t n, double scale) {
-    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x)
-        out[c] = (float)(scale * geps[c]);
+// Output: grad of the grid's cell c = scale * geps at its place.
+__global__ void k_adj_out(const double* geps, float* out, uint32_t n, uint32_t nx, uint32_t px, double scale) {
+    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
+        const uint32_t r = c / nx;
+        out[c] = (float)(scale * geps[r * px + (c - r * nx)]);
+    }
 }
 
 }  // namespace
@@ -605,9 +607,9 @@ extern "C" int mb_adjoint_energy_zface(mb_ctx* c, int n_steps, int ckpt_every, i
     if (zp < 1 || zp >= c->nz) return afail(c, MB_ERR_ARG, "z plane must satisfy 1 <= p < n_z");
     const int K = std::min(ckpt_every > 0 ? ckpt_every : 200, n_steps);
     const int nseg = (n_steps + K - 1) / K;
-    const size_t N = (size_t)c->ncell;
+    const size_t N = (size_t)c->pcell;
     const size_t sb = mb::state_device_bytes(c);
-    const size_t nxy = (size_t)c->nx * c->ny;
+    const size_t nxy = (size_t)c->px * c->ny;
     const size_t slot = 9 * N + 2 * nxy;   // floats per stored step: E, J, n1..n3, Hx/Hy of one plane
     const size_t psi_total = c->psi_elems[0] + c->psi_elems[1] + c->psi_elems[2];
     NvtxScope range("mb_adjoint_energy_zface");
@@ -880,7 +882,7 @@ extern "C" int mb_adjoint_energy_zface(mb_ctx* c, int n_steps, int ckpt_every, i
         const double KJ = c->dt * c->E0 * (c->E0 / c->eta0) * c->dx * c->dx;
         if (d_grad_eps) {
             const int blocks = (int)std::min<size_t>((N + 255) / 256, 4096);
-            mb::k_adj_out<<<blocks, 256, 0, c->stream>>>(geps, d_grad_eps, (uint32_t)N, KJ);
+            mb::k_adj_out<<<blocks, 256, 0, c->stream>>>(geps, d_grad_eps, (uint32_t)c->ncell, (uint32_t)c->nx, (uint32_t)c->px, KJ);
             MB_ACUDA(c, cudaGetLastError());
         }
         MB_ACUDA(c, cudaMemcpyAsync(acc_h, acc, sizeof(acc_h), cudaMemcpyDeviceToHost, c->stream));

@@ -103,13 +103,13 @@ float* field_ptr(mb_ctx* c, int which) {
     // layout: ex ey ez hx hy hz (current copy), px py pz jx jy jz n1 n2 n3
     if (which < MB_EX || which > MB_N3 || which == MB_N0) return nullptr;
     const int slot = which < MB_N0 ? which : which - 1;
-    if (slot < 6) return eh_of(c, c->parity) + (int64_t)slot * c->ncell;
-    return c->d_fields + (int64_t)slot * c->ncell;
+    if (slot < 6) return eh_of(c, c->parity) + (int64_t)slot * c->pcell;
+    return c->d_fields + (int64_t)slot * c->pcell;
 }
 
 // Points the step arguments' E, H and CPML memories at copy p.
 void point_args_at(mb::StepArgs& a, const mb_ctx* c, int p) {
-    const int64_t N = c->ncell;
+    const int64_t N = c->pcell;
     float* F = eh_of(c, p);
     a.f.ex = F + 0 * N; a.f.ey = F + 1 * N; a.f.ez = F + 2 * N;
     a.f.hx = F + 3 * N; a.f.hy = F + 4 * N; a.f.hz = F + 5 * N;
@@ -139,9 +139,9 @@ void z_cpml_bounds(const mb_ctx* c, mb::DevCpml& m) {
 
 void build_args(mb_ctx* c) {
     mb::StepArgs& a = c->args;
-    a.g = {c->nx, c->ny, c->nz, (uint32_t)c->nx * (uint32_t)c->ny, (uint32_t)c->ncell};
+    a.g = {c->nx, c->ny, c->nz, (uint32_t)c->px * (uint32_t)c->ny, (uint32_t)c->pcell, c->px};
     float* F = c->d_fields;
-    const int64_t N = c->ncell;
+    const int64_t N = c->pcell;
     a.f.px = F + 6 * N; a.f.py = F + 7 * N; a.f.pz = F + 8 * N;
     a.f.jx = F + 9 * N; a.f.jy = F + 10 * N; a.f.jz = F + 11 * N;
     a.f.n1 = F + 12 * N; a.f.n2 = F + 13 * N; a.f.n3 = F + 14 * N;
@@ -189,6 +189,7 @@ void build_args(mb_ctx* c) {
     a.step_ctr = c->d_ctr;
     a.err = c->d_err;
     a.glist.cell = c->d_glist;
+    a.glist.number = c->px != c->nx ? c->d_glist_num : nullptr;
     a.glist.count = c->glist_count;
 }
 
@@ -272,8 +273,8 @@ int check_ctx(mb_ctx* c) {
 
 std::vector<StatePart> state_parts(mb_ctx* c) {
     std::vector<StatePart> v;
-    v.push_back({eh_of(c, c->parity), sizeof(float) * 6 * (size_t)c->ncell});
-    v.push_back({c->d_fields + 6 * c->ncell, sizeof(float) * 9 * (size_t)c->ncell});
+    v.push_back({eh_of(c, c->parity), sizeof(float) * 6 * (size_t)c->pcell, 6});
+    v.push_back({c->d_fields + 6 * c->pcell, sizeof(float) * 9 * (size_t)c->pcell, 9});
     for (int w = 0; w < 3; ++w)
         if (c->psi_elems[w]) v.push_back({psi_of(c, c->parity, w), sizeof(float) * c->psi_elems[w]});
     v.push_back({c->d_ctr, sizeof(long long) * 2});
@@ -287,6 +288,76 @@ std::vector<StatePart> state_parts(mb_ctx* c) {
     for (const mb::DevPlaneProbe& q : c->planes)
         v.push_back({q.acc, sizeof(double2) * 3 * (size_t)q.nfreq * c->nx * c->ny});
     return v;
+}
+
+size_t host_bytes(const mb_ctx* c, const StatePart& p) {
+    return p.arrays ? sizeof(float) * (size_t)p.arrays * c->ncell : p.bytes;
+}
+
+// Padded rows are packed and spread by a kernel (a 2-D device copy of rows of
+// 157 floats measured 13 us more than the plain copy; the kernel as much as
+// it).  To and from the host they cross packed, an array at a time through
+// the material's upload buffer (2.7 M cells: a field read 1.7 ms as without
+// padding; packed on the host 2.7 ms); before a material is set, through a
+// host buffer, with zeros in the padding as the device's rows hold.
+cudaError_t rows_out(const mb_ctx* c, void* packed, const void* rows, size_t esize, int arrays, cudaMemcpyKind kind) {
+    if (c->px == c->nx)
+        return cudaMemcpyAsync(packed, rows, esize * (size_t)arrays * c->ncell, kind, c->stream);
+    const int64_t nrow = (int64_t)c->ny * c->nz;
+    const size_t to = esize * c->nx, from = esize * c->px;
+    if (kind == cudaMemcpyDeviceToDevice) {
+        mb::launch_rows(rows, c->px, packed, c->nx, c->nx, nrow * arrays, (int)esize, c->stream);
+        return cudaGetLastError();
+    }
+    if (c->upload_bytes >= to * nrow) {
+        for (int q = 0; q < arrays; ++q) {
+            mb::launch_rows((const char*)rows + from * nrow * q, c->px, c->d_upload, c->nx, c->nx, nrow, (int)esize,
+                            c->stream);
+            cudaError_t e = cudaMemcpyAsync((char*)packed + to * nrow * q, c->d_upload, to * nrow, kind, c->stream);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaGetLastError();
+    }
+    std::unique_ptr<char[]> tmp(new (std::nothrow) char[from * nrow]);
+    if (!tmp) return cudaErrorMemoryAllocation;
+    for (int q = 0; q < arrays; ++q) {
+        const char* src = (const char*)rows + from * nrow * q;
+        char* dst = (char*)packed + to * nrow * q;
+        cudaError_t e = cudaMemcpyAsync(tmp.get(), src, from * nrow, kind, c->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        if (e != cudaSuccess) return e;
+        for (int64_t r = 0; r < nrow; ++r) std::memcpy(dst + to * r, tmp.get() + from * r, to);
+    }
+    return cudaSuccess;
+}
+cudaError_t rows_in(const mb_ctx* c, void* rows, const void* packed, size_t esize, int arrays, cudaMemcpyKind kind) {
+    if (c->px == c->nx)
+        return cudaMemcpyAsync(rows, packed, esize * (size_t)arrays * c->ncell, kind, c->stream);
+    const int64_t nrow = (int64_t)c->ny * c->nz;
+    const size_t to = esize * c->px, from = esize * c->nx;
+    if (kind == cudaMemcpyDeviceToDevice) {
+        mb::launch_rows(packed, c->nx, rows, c->px, c->nx, nrow * arrays, (int)esize, c->stream);
+        return cudaGetLastError();
+    }
+    if (c->upload_bytes >= from * nrow) {
+        for (int q = 0; q < arrays; ++q) {
+            cudaError_t e = cudaMemcpyAsync(c->d_upload, (const char*)packed + from * nrow * q, from * nrow, kind,
+                                            c->stream);
+            if (e != cudaSuccess) return e;
+            mb::launch_rows(c->d_upload, c->nx, (char*)rows + to * nrow * q, c->px, c->nx, nrow, (int)esize, c->stream);
+        }
+        return cudaGetLastError();
+    }
+    std::unique_ptr<char[]> tmp(new (std::nothrow) char[to * nrow]());
+    if (!tmp) return cudaErrorMemoryAllocation;
+    for (int q = 0; q < arrays; ++q) {
+        const char* src = (const char*)packed + from * nrow * q;
+        for (int64_t r = 0; r < nrow; ++r) std::memcpy(tmp.get() + to * r, src + from * r, from);
+        cudaError_t e = cudaMemcpyAsync((char*)rows + to * nrow * q, tmp.get(), to * nrow, kind, c->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // Tensor maps for a TMA tuning over the current copy (encoded once per tile
@@ -639,6 +710,18 @@ static int create_ctx(mb_ctx** out, const int grid[3], int gnz, int kz0, int own
     c->ny = grid[1];
     c->nz = grid[2];
     c->ncell = ncell;
+    c->px = c->nx;
+    // rows of whole 16-byte words, which the single-pass step's tensor maps
+    // need (139^3: 95.6 us a step against 103 for the two passes), where the
+    // added cells are few (at most a sixteenth; below 48 cells a row they may
+    // be more) and memory for that step's second copy of the state is left
+    const int px = (c->nx + 3) / 4 * 4;
+    const int64_t pcell = (int64_t)px * c->ny * c->nz;
+    size_t mem_free = 0, mem_total = 0;
+    if (px != c->nx && (px - c->nx) * 16 <= c->nx && pcell < (int64_t(1) << 32) &&
+        cudaMemGetInfo(&mem_free, &mem_total) == cudaSuccess && 2 * sizeof(float) * 15 * (size_t)pcell <= mem_free)
+        c->px = px;
+    c->pcell = (int64_t)c->px * c->ny * c->nz;
     c->slab = slab;
     c->gnz = gnz;
     c->kz0 = kz0;
@@ -675,8 +758,9 @@ static int create_ctx(mb_ctx** out, const int grid[3], int gnz, int kz0, int own
         return MB_OK;
     };
     int rc;
-    if ((rc = alloc((void**)&c->d_fields, sizeof(float) * 15 * (size_t)ncell))) return bail(rc);
-    if ((rc = alloc((void**)&c->d_mat, (size_t)ncell))) return bail(rc);
+    rc = alloc((void**)&c->d_fields, sizeof(float) * 15 * (size_t)c->pcell);
+    if (rc) return bail(rc);
+    if ((rc = alloc((void**)&c->d_mat, (size_t)c->pcell))) return bail(rc);
     if ((rc = alloc((void**)&c->d_lut, sizeof(float) * 256))) return bail(rc);
     const int L = prm.npml;
     c->psi_elems[0] = L ? (size_t)4 * c->nz * c->ny * 2 * L : 0;
@@ -724,8 +808,8 @@ static int create_ctx(mb_ctx** out, const int grid[3], int gnz, int kz0, int own
     } while (0)
     MB_CREATE_CUDA(cudaMemcpy(c->d_coef, coef.data(), sizeof(float) * ncoef, cudaMemcpyHostToDevice));
     MB_CREATE_CUDA(cudaMemcpy(c->d_lut, lut.data(), sizeof(float) * 256, cudaMemcpyHostToDevice));
-    MB_CREATE_CUDA(cudaMemset(c->d_fields, 0, sizeof(float) * 15 * (size_t)ncell));
-    MB_CREATE_CUDA(cudaMemset(c->d_mat, 0, (size_t)ncell));
+    MB_CREATE_CUDA(cudaMemset(c->d_fields, 0, sizeof(float) * 15 * (size_t)c->pcell));
+    MB_CREATE_CUDA(cudaMemset(c->d_mat, 0, (size_t)c->pcell));
     for (int w = 0; w < 3; ++w)
         if (c->psi_elems[w]) MB_CREATE_CUDA(cudaMemset(c->d_psi[w], 0, sizeof(float) * c->psi_elems[w]));
     MB_CREATE_CUDA(cudaMemset(c->d_ctr, 0, sizeof(long long) * 4));
@@ -799,7 +883,7 @@ int mb_destroy(mb_ctx* c) {
     void* bufs[] = {c->d_fields, c->d_mat, c->d_inv_eps, c->d_lut, c->d_psi[0], c->d_psi[1],
                     c->d_psi[2], c->d_coef, c->d_ctr, c->d_flux, c->d_partial, c->d_energy,
                     c->d_nonfinite, c->d_probe_cell, c->d_probe_omega, c->d_probe_acc,
-                    c->d_face_omega, c->d_face_acc, c->d_face_acc32, c->d_face_spec, c->d_plane_out, c->d_glist, c->d_glist_scratch,
+                    c->d_face_omega, c->d_face_acc, c->d_face_acc32, c->d_face_spec, c->d_plane_out, c->d_glist, c->d_glist_num, c->d_glist_scratch,
                     c->d_upload, c->d_keys, c->d_src_wave, c->d_err,
                     c->d_fields2, c->d_psi2[0], c->d_psi2[1], c->d_psi2[2], c->d_flux_out, c->d_small,
                     c->d_small_x};
@@ -845,7 +929,8 @@ int mb_set_material(mb_ctx* c, const float* eps_map, const uint8_t* gain_mask, d
         have = need;
         return true;
     };
-    const size_t up_bytes = 5 * (size_t)N;
+    const bool rows = c->px != c->nx;
+    const size_t up_bytes = 5 * (size_t)N + 16;
     const size_t key_bytes = 2 * sizeof(uint32_t) * mb::kMatKeys + 2 * sizeof(int);
     if (!grow((void**)&c->d_upload, c->upload_bytes, up_bytes) ||
         !grow((void**)&c->d_keys, c->keys_bytes, key_bytes))
@@ -893,11 +978,11 @@ int mb_set_material(mb_ctx* c, const float* eps_map, const uint8_t* gain_mask, d
         c->h_lut_eps[q] = lut_eps[q];
     }
     if (dense && !c->d_inv_eps) {
-        cudaError_t e = cudaMalloc((void**)&c->d_inv_eps, sizeof(float) * (size_t)N);
+        cudaError_t e = cudaMalloc((void**)&c->d_inv_eps, sizeof(float) * (size_t)c->pcell);
         if (e != cudaSuccess) { cudaGetLastError(); return fail(c, MB_ERR_OOM, "dense eps map allocation failed"); }
-        c->dev_bytes += sizeof(float) * (size_t)N;
+        c->dev_bytes += sizeof(float) * (size_t)c->pcell;
     }
-    const size_t nsc = mb::gain_list_scratch(N);
+    const size_t nsc = mb::gain_list_scratch(c->pcell);
     if (nsc > c->glist_scratch_n) {
         if (c->d_glist_scratch) cudaFree(c->d_glist_scratch);
         c->d_glist_scratch = nullptr;
@@ -906,11 +991,21 @@ int mb_set_material(mb_ctx* c, const float* eps_map, const uint8_t* gain_mask, d
         if (e != cudaSuccess) { cudaGetLastError(); return fail(c, MB_ERR_OOM, "gain list allocation failed"); }
         c->glist_scratch_n = nsc;
     }
-    mb::launch_mat_ids(d_eps, d_gain, N, c->d_keys, (int)keys.size(), dense, N_a > 0.0, c->d_mat,
-                       c->d_inv_eps, c->stream);
+    if (rows) {
+        // padded rows: the packed map in the upload's place, cell by cell, then spread
+        mb::launch_mat_ids(d_eps, d_gain, N, c->d_keys, (int)keys.size(), dense, N_a > 0.0, d_gain, d_eps, c->stream);
+        MB_CUDA(c, rows_in(c, c->d_mat, d_gain, 1, 1, cudaMemcpyDeviceToDevice));
+        if (dense) {
+            MB_CUDA(c, cudaMemsetAsync(c->d_inv_eps, 0x3f, sizeof(float) * (size_t)c->pcell, c->stream));   // (padding: not zero)
+            MB_CUDA(c, rows_in(c, c->d_inv_eps, d_eps, 4, 1, cudaMemcpyDeviceToDevice));
+        }
+    } else {
+        mb::launch_mat_ids(d_eps, d_gain, N, c->d_keys, (int)keys.size(), dense, N_a > 0.0, c->d_mat,
+                           c->d_inv_eps, c->stream);
+    }
     MB_CUDA(c, cudaMemcpyAsync(c->d_lut, lut.data(), sizeof(float) * 256, cudaMemcpyHostToDevice, c->stream));
     // gain cells in increasing order: the two-pass step's Lorentz blocks run over this list
-    mb::launch_gain_count(c->d_mat, N, c->d_glist_scratch, c->stream);
+    mb::launch_gain_count(c->d_mat, c->pcell, c->d_glist_scratch, c->stream);
     uint32_t n_gain32 = 0;
     MB_CUDA(c, cudaMemcpyAsync(&n_gain32, c->d_glist_scratch + (nsc - 2), sizeof(uint32_t),
                                cudaMemcpyDeviceToHost, c->stream));
@@ -919,16 +1014,19 @@ int mb_set_material(mb_ctx* c, const float* eps_map, const uint8_t* gain_mask, d
     if (n_gain > c->glist_capacity || !c->d_glist) {
         if (c->d_glist) {
             cudaFree(c->d_glist);
-            c->dev_bytes -= sizeof(uint32_t) * c->glist_capacity;
-            c->d_glist = nullptr;
+            cudaFree(c->d_glist_num);
+            c->dev_bytes -= sizeof(uint32_t) * c->glist_capacity * (rows ? 2 : 1);
+            c->d_glist = c->d_glist_num = nullptr;
         }
         const size_t cap = n_gain ? n_gain : 1;
         cudaError_t e = cudaMalloc((void**)&c->d_glist, sizeof(uint32_t) * cap);
+        if (e == cudaSuccess && rows) e = cudaMalloc((void**)&c->d_glist_num, sizeof(uint32_t) * cap);
         if (e != cudaSuccess) { cudaGetLastError(); return fail(c, MB_ERR_OOM, "gain list allocation failed"); }
         c->glist_capacity = cap;
-        c->dev_bytes += sizeof(uint32_t) * cap;
+        c->dev_bytes += sizeof(uint32_t) * cap * (rows ? 2 : 1);
     }
-    if (n_gain) mb::launch_gain_scatter(c->d_mat, N, c->d_glist_scratch, c->d_glist, c->stream);
+    if (n_gain) mb::launch_gain_scatter(c->d_mat, c->pcell, c->d_glist_scratch, c->d_glist, c->stream);
+    if (n_gain && rows) mb::launch_gain_numbers(c->d_glist, n_gain32, c->nx, c->px, c->d_glist_num, c->stream);
     // dense maps (no table) take the per-cell array; n_lut counts the table
     c->n_lut = dense ? 128 : (int)lut_eps.size();
     c->h_lut_ie[0] = lut[0];
@@ -938,7 +1036,7 @@ int mb_set_material(mb_ctx* c, const float* eps_map, const uint8_t* gain_mask, d
     c->W_p = pump;
     c->glist_count = (uint32_t)n_gain;
     // reset P, J and the populations (N0 = N_a, n1 = n2 = n3 = 0)
-    MB_CUDA(c, cudaMemsetAsync(c->d_fields + 6 * N, 0, sizeof(float) * 9 * (size_t)N, c->stream));
+    MB_CUDA(c, cudaMemsetAsync(c->d_fields + 6 * c->pcell, 0, sizeof(float) * 9 * (size_t)c->pcell, c->stream));
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
     c->have_material = true;
     build_args(c);
@@ -967,7 +1065,7 @@ int mb_add_point_probe(mb_ctx* c, const int ijk[3], int n_freq, double lam_min, 
         return fail(c, MB_ERR_ARG, "all point probes of a context share one bin count");
     cudaStreamSynchronize(c->stream);
     mb::PointProbeHost pr;
-    pr.cell = ijk[0] + (int64_t)c->nx * (ijk[1] + (int64_t)c->ny * ijk[2]);
+    pr.cell = ijk[0] + (int64_t)c->px * (ijk[1] + (int64_t)c->ny * ijk[2]);
     pr.nfreq = n_freq;
     for (int k = 0; k < n_freq; ++k) {
         const double lam = n_freq == 1 ? lam_min : lam_min + (lam_max - lam_min) * k / (n_freq - 1);
@@ -1122,7 +1220,7 @@ int mb_set_source(mb_ctx* c, const int ijk[3], int comp, double lam, double t0, 
     MB_CUDA(c, cudaMemcpy(c->d_src_wave, wave.data(), sizeof(float) * wave.size(), cudaMemcpyHostToDevice));
     c->src.on = 1;
     c->src.comp = comp;
-    c->src.cell = ijk[0] + (int64_t)c->nx * (ijk[1] + (int64_t)c->ny * ijk[2]);
+    c->src.cell = ijk[0] + (int64_t)c->px * (ijk[1] + (int64_t)c->ny * ijk[2]);
     c->src.n0 = n0;
     c->src.count = (int)(n1 - n0);
     c->src.wave = c->d_src_wave;
@@ -1159,7 +1257,7 @@ int mb_set_source_cw(mb_ctx* c, const int ijk[3], int comp, double lam, double t
     MB_CUDA(c, cudaMemcpy(c->d_src_wave, wave.data(), sizeof(float) * wave.size(), cudaMemcpyHostToDevice));
     c->src.on = 1;
     c->src.comp = comp;
-    c->src.cell = ijk[0] + (int64_t)c->nx * (ijk[1] + (int64_t)c->ny * ijk[2]);
+    c->src.cell = ijk[0] + (int64_t)c->px * (ijk[1] + (int64_t)c->ny * ijk[2]);
     c->src.n0 = n0;
     c->src.count = n_steps;
     c->src.wave = c->d_src_wave;
@@ -1349,8 +1447,8 @@ int mb_energy(mb_ctx* c, double* out_U, double* out_flux6) {
     if (!out_U) return fail(c, MB_ERR_ARG, "null output");
     MB_CUDA(c, cudaMemsetAsync(c->d_nonfinite, 0, sizeof(int), c->stream));
     // the context's own planes (all of them but a z-slab's ghost planes)
-    const int64_t off = (int64_t)c->own_lo * c->nx * c->ny;
-    const int64_t own = (int64_t)(c->own_hi - c->own_lo) * c->nx * c->ny;
+    const int64_t off = (int64_t)c->own_lo * c->px * c->ny;   // (padding: zero fields)
+    const int64_t own = (int64_t)(c->own_hi - c->own_lo) * c->px * c->ny;
     mb::DevFields f = c->args.f;
     for (float** q : {&f.ex, &f.ey, &f.ez, &f.hx, &f.hy, &f.hz, &f.px, &f.py, &f.pz, &f.jx, &f.jy,
                       &f.jz, &f.n1, &f.n2, &f.n3})
@@ -1379,7 +1477,8 @@ int mb_gain_list(mb_ctx* c, uint32_t* host_out, int64_t* count) {
     *count = (int64_t)c->glist_count;
     if (!host_out || c->glist_count == 0) return MB_OK;
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
-    MB_CUDA(c, cudaMemcpy(host_out, c->d_glist, sizeof(uint32_t) * c->glist_count, cudaMemcpyDeviceToHost));
+    MB_CUDA(c, cudaMemcpy(host_out, c->px != c->nx ? c->d_glist_num : c->d_glist,
+                          sizeof(uint32_t) * c->glist_count, cudaMemcpyDeviceToHost));
     return MB_OK;
 }
 
@@ -1388,7 +1487,8 @@ int mb_get_material(mb_ctx* c, uint8_t* host_out) {
     if (!host_out) return fail(c, MB_ERR_ARG, "null output");
     if (!c->have_material) return fail(c, MB_ERR_STATE, "no material set");
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
-    MB_CUDA(c, cudaMemcpy(host_out, c->d_mat, (size_t)c->ncell, cudaMemcpyDeviceToHost));
+    MB_CUDA(c, rows_out(c, host_out, c->d_mat, 1, 1, cudaMemcpyDeviceToHost));
+    MB_CUDA(c, cudaStreamSynchronize(c->stream));
     return MB_OK;
 }
 
@@ -1419,17 +1519,17 @@ int mb_get_field(mb_ctx* c, int which, float* host_out) {
     if (which == MB_N0) {
         std::vector<float> a((size_t)N), b((size_t)N), d((size_t)N);
         std::vector<uint8_t> m((size_t)N, 0);
-        MB_CUDA(c, cudaMemcpyAsync(a.data(), field_ptr(c, MB_N1), 4 * N, cudaMemcpyDeviceToHost, c->stream));
-        MB_CUDA(c, cudaMemcpyAsync(b.data(), field_ptr(c, MB_N2), 4 * N, cudaMemcpyDeviceToHost, c->stream));
-        MB_CUDA(c, cudaMemcpyAsync(d.data(), field_ptr(c, MB_N3), 4 * N, cudaMemcpyDeviceToHost, c->stream));
+        MB_CUDA(c, rows_out(c, a.data(), field_ptr(c, MB_N1), 4, 1, cudaMemcpyDeviceToHost));
+        MB_CUDA(c, rows_out(c, b.data(), field_ptr(c, MB_N2), 4, 1, cudaMemcpyDeviceToHost));
+        MB_CUDA(c, rows_out(c, d.data(), field_ptr(c, MB_N3), 4, 1, cudaMemcpyDeviceToHost));
         if (c->have_material)
-            MB_CUDA(c, cudaMemcpyAsync(m.data(), c->d_mat, (size_t)N, cudaMemcpyDeviceToHost, c->stream));
+            MB_CUDA(c, rows_out(c, m.data(), c->d_mat, 1, 1, cudaMemcpyDeviceToHost));
         MB_CUDA(c, cudaStreamSynchronize(c->stream));
         for (int64_t q = 0; q < N; ++q)
             host_out[q] = (m[q] & 0x80) ? (float)(c->N_a * (1.0 - (double)a[q] - (double)b[q] - (double)d[q])) : 0.0f;
         return MB_OK;
     }
-    MB_CUDA(c, cudaMemcpyAsync(tmp.data(), field_ptr(c, which), 4 * N, cudaMemcpyDeviceToHost, c->stream));
+    MB_CUDA(c, rows_out(c, tmp.data(), field_ptr(c, which), 4, 1, cudaMemcpyDeviceToHost));
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
     const double s = field_scale(c, which);
     for (int64_t q = 0; q < N; ++q) host_out[q] = (float)(s * (double)tmp[q]);
@@ -1446,7 +1546,8 @@ int mb_set_field(mb_ctx* c, int which, const float* host_in) {
     std::vector<float> tmp((size_t)N);
     for (int64_t q = 0; q < N; ++q) tmp[q] = (float)(s * (double)host_in[q]);
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
-    MB_CUDA(c, cudaMemcpy(field_ptr(c, which), tmp.data(), 4 * N, cudaMemcpyHostToDevice));
+    MB_CUDA(c, rows_in(c, field_ptr(c, which), tmp.data(), 4, 1, cudaMemcpyHostToDevice));
+    MB_CUDA(c, cudaStreamSynchronize(c->stream));
     return MB_OK;
 }
 
@@ -1454,7 +1555,7 @@ int mb_get_field_device(mb_ctx* c, int which, float* dev_out, double* scale) {
     if (int rc = check_ctx(c)) return rc;
     if (!dev_out || which < 0 || which >= MB_NUM_FIELDS || which == MB_N0)
         return fail(c, MB_ERR_ARG, "bad field id (N0 is not stored) or null output");
-    MB_CUDA(c, cudaMemcpyAsync(dev_out, field_ptr(c, which), 4 * c->ncell, cudaMemcpyDeviceToDevice, c->stream));
+    MB_CUDA(c, rows_out(c, dev_out, field_ptr(c, which), 4, 1, cudaMemcpyDeviceToDevice));
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
     if (scale) *scale = field_scale(c, which);
     return MB_OK;
@@ -1465,7 +1566,7 @@ int mb_save_state(mb_ctx* c, void* host_blob, size_t* bytes) {
     if (!bytes) return fail(c, MB_ERR_ARG, "null size");
     auto parts = state_parts(c);
     size_t total = 4 * sizeof(int64_t);
-    for (auto& p : parts) total += p.bytes;
+    for (auto& p : parts) total += host_bytes(c, p);
     if (!host_blob) {
         *bytes = total;
         return MB_OK;
@@ -1476,8 +1577,9 @@ int mb_save_state(mb_ctx* c, void* host_blob, size_t* bytes) {
     std::memcpy(o, hdr, sizeof(hdr));
     o += sizeof(hdr);
     for (auto& p : parts) {
-        MB_CUDA(c, cudaMemcpyAsync(o, p.ptr, p.bytes, cudaMemcpyDeviceToHost, c->stream));
-        o += p.bytes;
+        if (p.arrays) MB_CUDA(c, rows_out(c, o, p.ptr, 4, p.arrays, cudaMemcpyDeviceToHost));
+        else MB_CUDA(c, cudaMemcpyAsync(o, p.ptr, p.bytes, cudaMemcpyDeviceToHost, c->stream));
+        o += host_bytes(c, p);
     }
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
     *bytes = total;
@@ -1489,16 +1591,18 @@ int mb_load_state(mb_ctx* c, const void* host_blob, size_t bytes) {
     if (!host_blob) return fail(c, MB_ERR_ARG, "null blob");
     auto parts = state_parts(c);
     size_t total = 4 * sizeof(int64_t);
-    for (auto& p : parts) total += p.bytes;
+    for (auto& p : parts) total += host_bytes(c, p);
     const int64_t* hdr = (const int64_t*)host_blob;
     if (bytes != total || hdr[0] != 0x4D42464454445331LL || hdr[1] != c->ncell || hdr[2] != (int64_t)parts.size())
         return fail(c, MB_ERR_ARG, "blob does not match this context's layout");
     const char* o = (const char*)host_blob + 4 * sizeof(int64_t);
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
     for (auto& p : parts) {
-        MB_CUDA(c, cudaMemcpy(p.ptr, o, p.bytes, cudaMemcpyHostToDevice));
-        o += p.bytes;
+        if (p.arrays) MB_CUDA(c, rows_in(c, p.ptr, o, 4, p.arrays, cudaMemcpyHostToDevice));
+        else MB_CUDA(c, cudaMemcpyAsync(p.ptr, o, p.bytes, cudaMemcpyHostToDevice, c->stream));
+        o += host_bytes(c, p);
     }
+    MB_CUDA(c, cudaStreamSynchronize(c->stream));
     c->n = hdr[3];
     return MB_OK;
 }

@@ -59,8 +59,15 @@ void point_args_at(mb::StepArgs& a, const mb_ctx* c, int p);
 // Device buffers that make up the evolving state (in blob order).
 struct StatePart {
     void* ptr;
-    size_t bytes;
+    size_t bytes;     // on the device
+    int arrays = 0;   // grid arrays of floats among them (rows px apart; a host blob holds n_x of each row)
 };
+size_t host_bytes(const mb_ctx* c, const StatePart& p);
+
+// Copies of `arrays` consecutive grid arrays of esize-byte elements between
+// the device's rows and a packed buffer (host or device).
+cudaError_t rows_out(const mb_ctx* c, void* packed, const void* rows, size_t esize, int arrays, cudaMemcpyKind kind);
+cudaError_t rows_in(const mb_ctx* c, void* rows, const void* packed, size_t esize, int arrays, cudaMemcpyKind kind);
 std::vector<StatePart> state_parts(mb_ctx* c);
 
 // Tensor maps of the two-pass TMA launches over the current copy, else nullptr.

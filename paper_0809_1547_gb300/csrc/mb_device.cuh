@@ -21,10 +21,22 @@
 namespace mb {
 
 // Cell offsets are 32-bit: a realization holds fewer than 2^32 cells.
+// Rows of the field arrays are px cells apart: n_x, or n_x rounded up to a
+// multiple of 4 (16 bytes, what bulk tensor copies ask of a row) on grids
+// where that costs little memory.  A cell's place is c = i + px j + nxy k;
+// the cells past n_x of a row hold zeros and are never written.  The noise
+// and the host see the grid's own numbering, i + n_x (j + n_y k).
 struct DevGrid {
     int nx, ny, nz;
-    uint32_t nxy, ncell;
+    uint32_t nxy, ncell;   // px ny, px ny nz
+    int px;
 };
+__device__ __forceinline__ uint32_t cell_place(const DevGrid& g, int i, int j, int k) {
+    return (uint32_t)i + (uint32_t)g.px * j + g.nxy * k;
+}
+__device__ __forceinline__ uint32_t cell_number(const DevGrid& g, int i, int j, int k) {
+    return (uint32_t)i + (uint32_t)g.nx * ((uint32_t)j + (uint32_t)g.ny * k);
+}
 
 // The face flux is accumulated into kFluxSlots FP64 slots per face (spread
 // over L2 to avoid serialising the atomics); read-outs sum the slots.
@@ -102,6 +114,7 @@ struct DevFlux {
 // update runs over this list so that whole warps do gain work.
 struct DevGainList {
     const uint32_t* cell;
+    const uint32_t* number;   // their numbers in the grid (null: the places are the numbers)
     uint32_t count;
 };
 
@@ -250,37 +263,37 @@ struct HNb {
 // beyond the last cell are zero.
 __device__ __forceinline__ ENb load_e_nbrs(const StepArgs& a, int i, int j, int k, uint32_t c) {
     const DevFields& f = a.f;
-    const int nx = a.g.nx;
+    const int nx = a.g.nx, px = a.g.px;
     const uint32_t nxy = a.g.nxy;
     ENb e;
     e.ex = __ldg(f.ex + c);
     e.ey = __ldg(f.ey + c);
     e.ez = __ldg(f.ez + c);
     const bool xi = i + 1 < nx, yj = j + 1 < a.g.ny, zk = k + 1 < a.g.nz;
-    e.ex_j1 = yj ? __ldg(f.ex + c + nx) : 0.0f;
+    e.ex_j1 = yj ? __ldg(f.ex + c + px) : 0.0f;
     e.ex_k1 = zk ? __ldg(f.ex + c + nxy) : 0.0f;
     e.ey_i1 = xi ? __ldg(f.ey + c + 1) : 0.0f;
     e.ey_k1 = zk ? __ldg(f.ey + c + nxy) : 0.0f;
     e.ez_i1 = xi ? __ldg(f.ez + c + 1) : 0.0f;
-    e.ez_j1 = yj ? __ldg(f.ez + c + nx) : 0.0f;
+    e.ez_j1 = yj ? __ldg(f.ez + c + px) : 0.0f;
     return e;
 }
 
 // H is read-only during the E pass; fields before the first cell are zero.
 __device__ __forceinline__ HNb load_h_nbrs(const StepArgs& a, int i, int j, int k, uint32_t c) {
     const DevFields& f = a.f;
-    const int nx = a.g.nx;
+    const int px = a.g.px;
     const uint32_t nxy = a.g.nxy;
     HNb h;
     h.hx = __ldg(f.hx + c);
     h.hy = __ldg(f.hy + c);
     h.hz = __ldg(f.hz + c);
-    h.hx_j = (j > 0) ? __ldg(f.hx + c - nx) : 0.0f;
+    h.hx_j = (j > 0) ? __ldg(f.hx + c - px) : 0.0f;
     h.hx_k = (k > 0) ? __ldg(f.hx + c - nxy) : 0.0f;
     h.hy_i = (i > 0) ? __ldg(f.hy + c - 1) : 0.0f;
     h.hy_k = (k > 0) ? __ldg(f.hy + c - nxy) : 0.0f;
     h.hz_i = (i > 0) ? __ldg(f.hz + c - 1) : 0.0f;
-    h.hz_j = (j > 0) ? __ldg(f.hz + c - nx) : 0.0f;
+    h.hz_j = (j > 0) ? __ldg(f.hz + c - px) : 0.0f;
     return h;
 }
 
@@ -445,7 +458,7 @@ __device__ __forceinline__ void h_core(const StepArgs& a, int i, int j, int k, u
 }
 
 __device__ __forceinline__ void h_update_cell(const StepArgs& a, int i, int j, int k) {
-    const uint32_t c = (uint32_t)i + (uint32_t)a.g.nx * j + a.g.nxy * k;
+    const uint32_t c = cell_place(a.g, i, j, k);
     h_core<true>(a, i, j, k, c, load_e_nbrs(a, i, j, k, c));
 }
 
@@ -713,7 +726,7 @@ __device__ __forceinline__ void e_core(const StepArgs& a, int i, int j, int k, u
 template <bool FLUX>
 __device__ __forceinline__ void e_update_cell(const StepArgs& a, int i, int j, int k,
                                               long long n, float fl[6]) {
-    const uint32_t c = (uint32_t)i + (uint32_t)a.g.nx * j + a.g.nxy * k;
+    const uint32_t c = cell_place(a.g, i, j, k);
     e_core<FLUX, true>(a, i, j, k, c, load_h_nbrs(a, i, j, k, c), n, fl);
 }
 

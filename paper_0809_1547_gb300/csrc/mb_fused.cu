@@ -97,7 +97,11 @@ __device__ __forceinline__ void e_plain(float S, const HNb& h, float ie, float e
     ez1 = fmaf(ie, fmaf(S, cz, -jz), ez0);
 }
 
-template <int BX, int BY, int S>
+// MATG: the material bytes come by plain loads two planes ahead, kept in
+// registers, instead of with the tensor copies (whose byte rows must be
+// multiples of 16: n_x = 320, 448, ...; every other n_x has rows of a
+// multiple of 4 cells only).
+template <int BX, int BY, int S, bool MATG>
 __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
                                                         const __grid_constant__ TmaFusedMaps maps,
                                                         int kz) {
@@ -150,7 +154,7 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
     auto issue = [&](int s, int p) {
         unsigned char* q = smem + s * Lay::kStage;
         const int k = k0 + p;
-        mbar_arrive_expect_tx(&bar[s], p < planes ? Lay::kTx : Lay::kTxE);
+        mbar_arrive_expect_tx(&bar[s], p < planes ? Lay::kTx - (MATG ? Lay::kMW : 0) : Lay::kTxE);
         tma_load_3d_hint(q + 0 * Lay::kEBytes, &maps.ex, x0 - 4, y0 - 1, k, &bar[s], keep_l2);
         tma_load_3d_hint(q + 1 * Lay::kEBytes, &maps.ey, x0 - 4, y0 - 1, k, &bar[s], keep_l2);
         tma_load_3d_hint(q + 2 * Lay::kEBytes, &maps.ez, x0 - 4, y0 - 1, k, &bar[s], keep_l2);
@@ -159,7 +163,7 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
             tma_load_3d(h + 0 * Lay::kHBytes, &maps.hx, x0 - 4, y0 - 1, k, &bar[s]);
             tma_load_3d(h + 1 * Lay::kHBytes, &maps.hy, x0 - 4, y0 - 1, k, &bar[s]);
             tma_load_3d(h + 2 * Lay::kHBytes, &maps.hz, x0 - 4, y0 - 1, k, &bar[s]);
-            tma_load_3d(h + 3 * Lay::kHBytes, &maps.mat, x0, y0, k, &bar[s]);
+            if (!MATG) tma_load_3d(h + 3 * Lay::kHBytes, &maps.mat, x0, y0, k, &bar[s]);
         }
     };
     auto mat_of = [&](int s) -> uint8_t {
@@ -189,7 +193,7 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
     int issued = min(S, total);   // planes issued into the ring so far
     bool block_fail = false;
 
-    uint32_t c = valid ? (uint32_t)i + (uint32_t)nx * j + nxy * k0 : 0u;
+    uint32_t c = valid ? cell_place(a.g, i, j, k0) : 0u;
     // H^{n+1/2} of plane k0-1 at this cell (zero below the first plane)
     float hx_km1 = 0.0f, hy_km1 = 0.0f;
     if (valid && k0 > 0) {
@@ -226,7 +230,7 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
     // in a slab, on a low PEC wall or in the source's column (and on every
     // plane that a z slab, the k = 0 wall or a face term makes general);
     // elsewhere e_plain, without the tests of those cases.
-    const bool src_col = a.src.on && (uint32_t)a.src.cell % nxy == (uint32_t)i + (uint32_t)nx * j;
+    const bool src_col = a.src.on && (uint32_t)a.src.cell % nxy == (uint32_t)i + (uint32_t)a.g.px * j;
     const bool w_gen = w_pml || __any_sync(full, valid && (i == 0 || j == 0 || src_col));
     const bool w_pml_halo = __any_sync(full, pml_xy && halo && cell_in_xy_slab(a, hi, hj));
     const bool w_xy = __any_sync(full, face && valid && cells_on_xy_face(a.flux, i, 1, j));
@@ -235,8 +239,13 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
     const int own_n = (ty + 1) * Lay::kNX + tx + 1;
     constexpr int EW = Lay::kEBytes / 4, HW = Lay::kHBytes / 4, NN = Lay::kNW;
 
+    uint8_t m0 = 0, m1 = 0;   // MATG: the material of planes p and p + 1
+    if (MATG && valid) {
+        m0 = __ldg(f.mat + c);
+        if (planes > 1) m1 = __ldg(f.mat + c + nxy);
+    }
     bool fail = !mbar_wait_bounded(&bar[0], 0, kWaitLimit);
-    bool pg = valid && gain_on && (mat_of(0) & 0x80);
+    bool pg = valid && gain_on && ((MATG ? m0 : mat_of(0)) & 0x80);
     if (pg) prefetch_gain(0, c);
     cp_async_commit();
     // ring slots of planes p and p + 1, and the phase parity of plane p + 1
@@ -246,9 +255,11 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
         const int k = k0 + p;
         cp_async_wait_all();   // this plane's gain values (own thread's copies)
         fail |= !mbar_wait_bounded(&bar[s1], ph1, kWaitLimit);
+        uint8_t m2 = 0;
+        if (MATG && valid && p + 2 < planes) m2 = __ldg(f.mat + c + 2 * nxy);
         bool ng = false;
         if (p + 1 < planes) {
-            ng = valid && gain_on && (mat_of(s1) & 0x80);
+            ng = valid && gain_on && ((MATG ? m1 : mat_of(s1)) & 0x80);
             if (ng) prefetch_gain((p + 1) & 1, c + nxy);
         }
         cp_async_commit();
@@ -327,7 +338,7 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
             n1 = *gslot(b, 6);
             n2 = *gslot(b, 7);
             n3 = *gslot(b, 8);
-            lorentz_step(a.gain, c, n, E0[own_e], E0[EW + own_e], E0[2 * EW + own_e], n1, n2, jx,
+            lorentz_step(a.gain, cell_number(a.g, i, j, k), n, E0[own_e], E0[EW + own_e], E0[2 * EW + own_e], n1, n2, jx,
                          jy, jz, px, py, pz);
             __stcs(f.px + c, px);
             __stcs(f.py + c, py);
@@ -351,7 +362,7 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
             h.hz_j = hn[2 * NN + own_n - Lay::kNX];
             h.hx_k = hx_km1;
             h.hy_k = hy_km1;
-            const uint8_t m = mat_of(s);
+            const uint8_t m = MATG ? m0 : mat_of(s);
             const float ex0 = E0[own_e], ey0 = E0[EW + own_e], ez0 = E0[2 * EW + own_e];
             float ex1, ey1, ez1;
             if (gen) {
@@ -398,6 +409,8 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
             issued = p + S + 1;
         }
         pg = ng;
+        m0 = m1;
+        m1 = m2;
         c += nxy;
         s = s1;
         s1 = (s1 + 1 == S) ? 0 : s1 + 1;
@@ -420,26 +433,36 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
     finish_step(a, d.sample);
 }
 
-template <int BX, int BY>
-static void launch_fused(const StepArgs& a, const DevPing& d, int kz, const TmaFusedMaps& maps,
-                         cudaStream_t s) {
+template <int BX, int BY, bool MATG>
+static void launch_fused_as(const StepArgs& a, const DevPing& d, int kz, const TmaFusedMaps& maps,
+                            cudaStream_t s) {
     const int smem = FusedLayout<BX, BY>::smem_bytes(kTmaStages);
     static bool attr_set = false;   // per instantiation, once per process
     if (!attr_set) {
-        cudaFuncSetAttribute(k_step_fused<BX, BY, kTmaStages>,
+        cudaFuncSetAttribute(k_step_fused<BX, BY, kTmaStages, MATG>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         attr_set = true;
     }
     dim3 grid((a.g.nx + BX - 1) / BX, (a.g.ny + BY - 1) / BY, fused_z_blocks(a.g.nz, kz));
-    k_step_fused<BX, BY, kTmaStages><<<grid, dim3(BX, BY, 1), smem, s>>>(a, d, maps, kz);
+    k_step_fused<BX, BY, kTmaStages, MATG><<<grid, dim3(BX, BY, 1), smem, s>>>(a, d, maps, kz);
 }
+
+template <int BX, int BY>
+static void launch_fused(const StepArgs& a, const DevPing& d, int kz, const TmaFusedMaps& maps,
+                         cudaStream_t s) {
+    if (a.g.px % 16 == 0) launch_fused_as<BX, BY, false>(a, d, kz, maps, s);
+    else launch_fused_as<BX, BY, true>(a, d, kz, maps, s);
+}
+
+// Bulk tensor copies of the fields: rows of whole 16-byte words.
+bool fused_supported(const StepArgs& a) { return a.g.px % 4 == 0; }
 
 bool fused_tile_supported(int bx, int by) {
     return (bx == 32 || bx == 64) && (by == 4 || by == 8);
 }
 
 bool encode_fused(const StepArgs& a, int bx, int by, TmaFusedMaps* out) {
-    if (!tma_e_supported(a) || !fused_tile_supported(bx, by)) return false;
+    if (!fused_supported(a) || !fused_tile_supported(bx, by)) return false;
     const DevFields& f = a.f;
     const CUtensorMapDataType F32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     return encode_box(&out->ex, F32, f.ex, 4, a.g, bx + 8, by + 2) &&
@@ -448,7 +471,7 @@ bool encode_fused(const StepArgs& a, int bx, int by, TmaFusedMaps* out) {
            encode_box(&out->hx, F32, f.hx, 4, a.g, bx + 4, by + 1) &&
            encode_box(&out->hy, F32, f.hy, 4, a.g, bx + 4, by + 1) &&
            encode_box(&out->hz, F32, f.hz, 4, a.g, bx + 4, by + 1) &&
-           encode_box(&out->mat, CU_TENSOR_MAP_DATA_TYPE_UINT8, f.mat, 1, a.g, bx, by);
+           (a.g.px % 16 != 0 || encode_box(&out->mat, CU_TENSOR_MAP_DATA_TYPE_UINT8, f.mat, 1, a.g, bx, by));
 }
 
 void launch_fused_step(const StepArgs& a, const DevPing& d, const PassTune& t,

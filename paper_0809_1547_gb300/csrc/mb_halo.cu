@@ -23,9 +23,10 @@ struct HaloPlane {
     float* fields;   // the context's 15 arrays (P, J, n1..n3 from array 6)
     float* psx;      // x-slab CPML memories of the current copy (or null)
     float* psy;      // y-slab CPML memories of the current copy (or null)
-    int64_t N;
-    int64_t nxy;
+    int64_t N;       // cells of an array, rows px apart
+    int64_t nxy;     // cells of a packed plane (no padding)
     int nx, ny, nz, L2;
+    int px;
     int k;
 };
 
@@ -46,7 +47,8 @@ __device__ __forceinline__ float* halo_addr(const HaloPlane& h, int64_t q) {
         const int64_t seg = q / h.nxy;
         const int64_t r = q - seg * h.nxy;
         float* base = (seg < 6 ? h.eh : h.fields) + seg * h.N;
-        return base + (int64_t)h.k * h.nxy + r;
+        const int64_t j = r / h.nx;
+        return base + ((int64_t)h.k * h.ny + j) * h.px + (r - j * h.nx);
     }
     q -= a;
     const int64_t bx = (int64_t)h.ny * h.L2;
@@ -76,7 +78,8 @@ int halo_launch(mb_ctx* c, int k, float* buf, bool pack) {
     h.fields = c->d_fields;
     h.psx = mbi::psi_of(c, c->parity, 0);
     h.psy = mbi::psi_of(c, c->parity, 1);
-    h.N = c->ncell;
+    h.N = c->pcell;
+    h.px = c->px;
     h.nxy = (int64_t)c->nx * c->ny;
     h.nx = c->nx;
     h.ny = c->ny;

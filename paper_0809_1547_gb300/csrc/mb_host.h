@@ -171,6 +171,7 @@ struct TmaFusedMaps {
     CUtensorMap ex, ey, ez, hx, hy, hz, mat;
 };
 bool fused_tile_supported(int bx, int by);
+bool fused_supported(const StepArgs& a);
 bool encode_fused(const StepArgs& a, int bx, int by, TmaFusedMaps* out);
 void launch_fused_step(const StepArgs& a, const DevPing& d, const PassTune& t,
                        const TmaFusedMaps& maps, cudaStream_t s);
@@ -273,6 +274,11 @@ size_t gain_list_scratch(int64_t N);
 void launch_gain_count(const uint8_t* mat, int64_t N, uint32_t* scratch, cudaStream_t s);
 void launch_gain_scatter(const uint8_t* mat, int64_t N, const uint32_t* scratch, uint32_t* list,
                          cudaStream_t s);
+// The numbers (k n_y + j) n_x + i of the list's places, rows px apart.
+void launch_gain_numbers(const uint32_t* list, uint32_t n, int nx, int px, uint32_t* number, cudaStream_t s);
+// `count` rows of nx elements (1 or 4 bytes) from rows `from` elements apart
+// to rows `to` elements apart.
+void launch_rows(const void* src, int from, void* dst, int to, int nx, int64_t count, int esize, cudaStream_t s);
 // The material map on the device: the distinct eps_r values into keys
 // (kMatKeys entries, kNoKey where unused, filled as a prefix) with the first
 // cell of each into first (initialised to kNoKey; flags[0]: a value not
@@ -339,6 +345,9 @@ struct PointProbeHost {
 struct mb_ctx {
     int nx = 0, ny = 0, nz = 0;
     int64_t ncell = 0;
+    // rows of the device arrays are px cells apart (DevGrid); pcell = px ny nz
+    int px = 0;
+    int64_t pcell = 0;
     // z-window.  A context may hold one z-slab of a grid split along z
     // (mb_create_slab): local plane k is plane k + kz0 of the whole grid of
     // gnz planes; planes [own_lo, own_hi) are the slab's own, the others (at
@@ -364,7 +373,8 @@ struct mb_ctx {
     float* d_psi[3] = {nullptr, nullptr, nullptr};
     size_t psi_elems[3] = {0, 0, 0};
     float* d_coef = nullptr;           // CPML tables
-    uint32_t* d_glist = nullptr;       // gain cells, increasing order
+    uint32_t* d_glist = nullptr;       // places of the gain cells, increasing order
+    uint32_t* d_glist_num = nullptr;   // their numbers in the grid (padded rows only)
     uint32_t glist_count = 0;
     size_t glist_capacity = 0;
     uint32_t* d_glist_scratch = nullptr;   // per-chunk counters of the list build

@@ -62,29 +62,29 @@ __global__ void __launch_bounds__(256) k_face_dft(DevFaceProbes fp, DevFields f,
         float Ea = 0.f, Eb = 0.f, Ha = 0.f, Hb = 0.f;
         if (axis == 0) {        // x-face: points (j = ca, k = cb); (a, b) = (y, z)
             if (plane < g.nx) {
-                const int64_t c = plane + (int64_t)g.nx * ca + g.nxy * cb;
+                const int64_t c = plane + (int64_t)g.px * ca + g.nxy * cb;
                 Ea = f.ey[c]; Eb = f.ez[c];
             }
             if (plane >= 1) {
-                const int64_t c = (plane - 1) + (int64_t)g.nx * ca + g.nxy * cb;
+                const int64_t c = (plane - 1) + (int64_t)g.px * ca + g.nxy * cb;
                 Ha = f.hy[c]; Hb = f.hz[c];
             }
         } else if (axis == 1) { // y-face: points (i = ca, k = cb); fields (z, x)
             if (plane < g.ny) {
-                const int64_t c = ca + (int64_t)g.nx * plane + g.nxy * cb;
+                const int64_t c = ca + (int64_t)g.px * plane + g.nxy * cb;
                 Ea = f.ez[c]; Eb = f.ex[c];
             }
             if (plane >= 1) {
-                const int64_t c = ca + (int64_t)g.nx * (plane - 1) + g.nxy * cb;
+                const int64_t c = ca + (int64_t)g.px * (plane - 1) + g.nxy * cb;
                 Ha = f.hz[c]; Hb = f.hx[c];
             }
         } else {                // z-face: points (i = ca, j = cb); (a, b) = (x, y)
             if (plane < g.nz) {
-                const int64_t c = ca + (int64_t)g.nx * cb + g.nxy * plane;
+                const int64_t c = ca + (int64_t)g.px * cb + g.nxy * plane;
                 Ea = f.ex[c]; Eb = f.ey[c];
             }
             if (plane >= 1) {
-                const int64_t c = ca + (int64_t)g.nx * cb + g.nxy * (plane - 1);
+                const int64_t c = ca + (int64_t)g.px * cb + g.nxy * (plane - 1);
                 Ha = f.hx[c]; Hb = f.hy[c];
             }
         }
@@ -272,10 +272,10 @@ __global__ void k_plane_dft(DevPlaneProbe pp, DevFields f, DevGrid g, const long
         ph[kk] = make_double2(w.x, w.y);
     }
     __syncthreads();
-    const uint32_t nxy = g.nxy;
+    const uint32_t nxy = (uint32_t)g.nx * g.ny;   // (the sums have no padding)
     const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= nxy) return;
-    const uint32_t c = p + nxy * (uint32_t)pp.k;
+    const uint32_t c = cell_place(g, p % g.nx, p / g.nx, pp.k);
     const double e[3] = {(double)f.ex[c], (double)f.ey[c], (double)f.ez[c]};
     for (int kk = 0; kk < pp.nfreq; ++kk) {
         const double2 w = ph[kk];
@@ -293,8 +293,8 @@ __global__ void k_plane_dft(DevPlaneProbe pp, DevFields f, DevGrid g, const long
 // Energy density of plane z = k in J/m^3: u0 (eps_r |E|^2 + |H|^2) / 2.
 __global__ void k_plane_energy(DevFields f, DevGrid g, int k, const float* lut_eps, double u0, double* out) {
     const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= g.nxy) return;
-    const uint32_t c = p + g.nxy * (uint32_t)k;
+    if (p >= (uint32_t)g.nx * g.ny) return;
+    const uint32_t c = cell_place(g, p % g.nx, p / g.nx, k);
     const double eps = f.inv_eps ? 1.0 / (double)f.inv_eps[c] : (double)lut_eps[f.mat[c] & 0x7f];
     const double ex = f.ex[c], ey = f.ey[c], ez = f.ez[c];
     const double hx = f.hx[c], hy = f.hy[c], hz = f.hz[c];
@@ -303,13 +303,13 @@ __global__ void k_plane_energy(DevFields f, DevGrid g, int k, const float* lut_e
 
 void launch_plane_dft(const DevPlaneProbe& pp, const DevFields& f, const DevGrid& g,
                       const long long* ctr, double dt, cudaStream_t s) {
-    const unsigned blocks = (g.nxy + 255) / 256;
+    const unsigned blocks = ((unsigned)g.nx * g.ny + 255) / 256;
     k_plane_dft<<<blocks, 256, 0, s>>>(pp, f, g, ctr, dt);
 }
 
 void launch_plane_energy(const DevFields& f, const DevGrid& g, int k, const float* lut_eps, double u0,
                          double* out, cudaStream_t s) {
-    const unsigned blocks = (g.nxy + 255) / 256;
+    const unsigned blocks = ((unsigned)g.nx * g.ny + 255) / 256;
     k_plane_energy<<<blocks, 256, 0, s>>>(f, g, k, lut_eps, u0, out);
 }
 
@@ -480,6 +480,47 @@ void launch_gain_scatter(const uint8_t* mat, int64_t N, const uint32_t* scratch,
     const int nchunks = gain_chunks(N);
     if (nchunks == 0) return;
     k_gain_scatter<<<nchunks, kGainThreads, 0, s>>>(mat, N, scratch, list);
+}
+
+// The grid's numbers of the cells at the places in list (padded rows).
+__global__ void k_gain_numbers(const uint32_t* list, uint32_t n, uint32_t nx, uint32_t px, uint32_t* number) {
+    for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
+        const uint32_t r = list[q] / px;
+        number[q] = r * nx + (list[q] - r * px);
+    }
+}
+void launch_gain_numbers(const uint32_t* list, uint32_t n, int nx, int px, uint32_t* number, cudaStream_t s) {
+    k_gain_numbers<<<std::max(1u, std::min((n + 255) / 256, 4096u)), 256, 0, s>>>(list, n, nx, px, number);
+}
+
+// Rows between the padded and the packed layout: bound by memory; a warp
+// takes a row at a time, four loads of it in flight, so loads and stores are
+// whole lines but for the rows' ends.
+template <typename T>
+__global__ void __launch_bounds__(256) k_rows(const T* __restrict__ src, int from, T* __restrict__ dst, int to,
+                                              int nx, int64_t count) {
+    const int lane = threadIdx.x & 31;
+    const int64_t step = (int64_t)gridDim.x * 8;
+    for (int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); r < count; r += step) {
+        const T* a = src + r * from;
+        T* b = dst + r * to;
+        for (int i = lane; i < nx; i += 128) {
+            T v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (i + 32 * q < nx) v[q] = a[i + 32 * q];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (i + 32 * q < nx) b[i + 32 * q] = v[q];
+        }
+    }
+}
+void launch_rows(const void* src, int from, void* dst, int to, int nx, int64_t count, int esize, cudaStream_t s) {
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((count + 7) / 8, 152 * 64));
+    if (esize == 4)
+        k_rows<float><<<blocks, 256, 0, s>>>((const float*)src, from, (float*)dst, to, nx, count);
+    else
+        k_rows<uint8_t><<<blocks, 256, 0, s>>>((const uint8_t*)src, from, (uint8_t*)dst, to, nx, count);
 }
 
 // ------------------------------------------------------------ material map

@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(512) k_hg_3d(StepArgs a, HGLayout lay) {
     const int j = by * blockDim.y + threadIdx.y;
     const int k = bz * blockDim.z + threadIdx.z;
     if (i >= a.g.nx || j >= a.g.ny || k >= a.g.nz) return;
-    const uint32_t c = (uint32_t)i + (uint32_t)a.g.nx * j + a.g.nxy * k;
+    const uint32_t c = cell_place(a.g, i, j, k);
     const ENb e = load_e_nbrs(a, i, j, k, c);
     const int k0 = bz * blockDim.z;
     const bool pml = tile_in_xy_slab(a, bx * blockDim.x, blockDim.x, by * blockDim.y, blockDim.y) ||
@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(512, 2) k_e_3d(StepArgs a) {
                      plane_in_z_slab(a, k0 + blockDim.z - 1);
     float fl[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (valid) {
-        const uint32_t c = (uint32_t)i + (uint32_t)a.g.nx * j + a.g.nxy * k;
+        const uint32_t c = cell_place(a.g, i, j, k);
         const HNb h = load_h_nbrs(a, i, j, k, c);
         if (face) e_core<true, true, KEEP>(a, i, j, k, c, h, n, fl);
         else if (pml) e_core<false, true, KEEP>(a, i, j, k, c, h, n, fl);
@@ -124,15 +124,15 @@ __global__ void __launch_bounds__(256) k_hg_vec(StepArgs a, HGLayout lay, int kz
     const DevFields& f = a.f;
     const bool pml_xy = tile_in_xy_slab(a, 4 * bx * blockDim.x, 4 * blockDim.x, by * blockDim.y, blockDim.y);
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    uint32_t c = valid ? (uint32_t)i0 + (uint32_t)nx * j + nxy * k0 : 0u;
+    uint32_t c = valid ? (uint32_t)i0 + (uint32_t)a.g.px * j + nxy * k0 : 0u;
     float4 ex = valid ? ldg4(f.ex + c) : zero, ey = valid ? ldg4(f.ey + c) : zero;
     for (int k = k0; k < k1; ++k, c += nxy) {
         const bool zk = k + 1 < nz;
         const float4 ez = valid ? ldg4(f.ez + c) : zero;
-        const float4 exk = (valid && zk) ? ldg4(f.ex + c + nxy) : zero;
+        const float4 exk = (valid && zk) ? ldg4(f.ex + c + a.g.nxy) : zero;
         const float4 eyk = (valid && zk) ? ldg4(f.ey + c + nxy) : zero;
-        const float4 exj = (valid && yj) ? ldg4(f.ex + c + nx) : zero;
-        const float4 ezj = (valid && yj) ? ldg4(f.ez + c + nx) : zero;
+        const float4 exj = (valid && yj) ? ldg4(f.ex + c + a.g.px) : zero;
+        const float4 ezj = (valid && yj) ? ldg4(f.ez + c + a.g.px) : zero;
         float ey_n = __shfl_down_sync(full, ey.x, 1);
         float ez_n = __shfl_down_sync(full, ez.x, 1);
         const bool xn = i0 + 4 < nx;
@@ -212,15 +212,15 @@ __device__ __forceinline__ void e_vec_walk(const StepArgs& a, int i0, int j, int
     const DevFields& f = a.f;
     const bool gain_on = a.gain.on;
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    uint32_t c = valid ? (uint32_t)i0 + (uint32_t)nx * j + nxy * k0 : 0u;
-    float4 hxk = (valid && k0 > 0) ? ldg4(f.hx + c - nxy) : zero;
+    uint32_t c = valid ? (uint32_t)i0 + (uint32_t)a.g.px * j + nxy * k0 : 0u;
+    float4 hxk = (valid && k0 > 0) ? ldg4(f.hx + c - a.g.nxy) : zero;
     float4 hyk = (valid && k0 > 0) ? ldg4(f.hy + c - nxy) : zero;
     for (int k = k0; k < k1; ++k, c += nxy) {
         const float4 hx = valid ? ldg4(f.hx + c) : zero;
         const float4 hy = valid ? ldg4(f.hy + c) : zero;
         const float4 hz = valid ? ldg4(f.hz + c) : zero;
-        const float4 hxj = (valid && j > 0) ? ldg4(f.hx + c - nx) : zero;
-        const float4 hzj = (valid && j > 0) ? ldg4(f.hz + c - nx) : zero;
+        const float4 hxj = (valid && j > 0) ? ldg4(f.hx + c - a.g.px) : zero;
+        const float4 hzj = (valid && j > 0) ? ldg4(f.hz + c - a.g.px) : zero;
         float hy_p = __shfl_up_sync(full, hy.w, 1);
         float hz_p = __shfl_up_sync(full, hz.w, 1);
         if (lane == 0) {
@@ -355,10 +355,10 @@ __global__ void __launch_bounds__(BX * BY) k_e_tma(StepArgs a, const __grid_cons
     int issued = min(S, k1 - k0);   // planes issued into the ring so far
     bool block_fail = false;
 
-    uint32_t c = valid ? (uint32_t)i + (uint32_t)nx * j + nxy * k0 : 0u;
+    uint32_t c = valid ? (uint32_t)i + (uint32_t)a.g.px * j + nxy * k0 : 0u;
     float hx_km1 = 0.0f, hy_km1 = 0.0f;
     if (valid && k0 > 0) {
-        hx_km1 = __ldg(f.hx + c - nxy);
+        hx_km1 = __ldg(f.hx + c - a.g.nxy);
         hy_km1 = __ldg(f.hy + c - nxy);
     }
     bool fail = !mbar_wait_bounded(&bar[0], 0, kWaitLimit);
@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(BX * BY) k_hg_tma(StepArgs a, const __grid_con
     int issued = min(S, total);   // planes issued into the ring so far
     bool block_fail = false;
 
-    uint32_t c = valid ? (uint32_t)i + (uint32_t)nx * j + nxy * k0 : 0u;
+    uint32_t c = valid ? (uint32_t)i + (uint32_t)a.g.px * j + nxy * k0 : 0u;
     bool fail = !mbar_wait_bounded(&bar[0], 0, kWaitLimit);
     const int own = ty * (BX + 4) + tx;
     for (int p = 0; p < planes; ++p) {
@@ -657,7 +657,7 @@ bool encode_box(CUtensorMap* m, CUtensorMapDataType dt, const void* base, int es
     auto enc = tensor_map_encoder();
     if (!enc) return false;
     const cuuint64_t dims[3] = {(cuuint64_t)g.nx, (cuuint64_t)g.ny, (cuuint64_t)g.nz};
-    const cuuint64_t strides[2] = {(cuuint64_t)g.nx * esize, (cuuint64_t)g.nx * g.ny * esize};
+    const cuuint64_t strides[2] = {(cuuint64_t)g.px * esize, (cuuint64_t)g.nxy * esize};
     const cuuint32_t box[3] = {(cuuint32_t)bw, (cuuint32_t)bh, 1};
     const cuuint32_t estr[3] = {1, 1, 1};
     return enc(m, dt, 3, const_cast<void*>(base), dims, strides, box, estr,

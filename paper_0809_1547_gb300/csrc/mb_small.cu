@@ -99,8 +99,8 @@ enum : uint32_t {
 __device__ void small_probe(const SmallArgs& A, int p, unsigned base, long long n0, int* fail_s) {
     const DevPointProbes& pp = A.pp;
     const int64_t cell = pp.cell[p];
-    const int nx = A.a.g.nx, ny = A.a.g.ny;
-    const int gi = (int)(cell % nx), gj = (int)(cell / nx % ny), gk = (int)(cell / ((int64_t)nx * ny));
+    const int px = A.a.g.px, ny = A.a.g.ny;
+    const int gi = (int)(cell % px), gj = (int)(cell / px % ny), gk = (int)(cell / ((int64_t)px * ny));
     const int owner = gi / A.t.tx + A.t.bx * (gj / A.t.ty + A.t.by * (gk / A.t.tz));
     const int K = pp.nfreq, kk = threadIdx.x;
     double2 v[3];
@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_step_small(const __grid_co
                 i = r % lx; j = r / lx; k = -1;
             }
             const int gi = x0 + i, gj = y0 + j, gk = z0 + k;
-            const uint32_t c = (uint32_t)gi + (uint32_t)nx * gj + nxy * gk;
+            const uint32_t c = cell_place(a.g, gi, gj, gk);
             const int hp = ho + i + hy_ * j + hz_ * k;
             Hs[hp] = make_float4(f.hx[c], f.hy[c], f.hz[c], 0.f);
             uint32_t fl = 0;
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_step_small(const __grid_co
             const int ep = eo + i + ey_ * j + ez_ * k;
             uint32_t src = 0xffffffffu;
             if (gi >= 0 && gi < nx && gj >= 0 && gj < ny && gk >= 0 && gk < nz) {
-                const uint32_t c = (uint32_t)gi + (uint32_t)nx * gj + nxy * gk;
+                const uint32_t c = cell_place(a.g, gi, gj, gk);
                 Es[ep] = make_float4(f.ex[c], f.ey[c], f.ez[c], 0.f);
                 const int ob = gi / A.t.tx, oj = gj / A.t.ty, ok = gk / A.t.tz;
                 const int olx = min(A.t.tx, nx - ob * A.t.tx), oly = min(A.t.ty, ny - oj * A.t.ty);
@@ -318,8 +318,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_step_small(const __grid_co
         const Item first = decode(min(tid, nitems - 1));
         auto item = [&](int q) { return q == tid ? first : decode(q); };
         auto cell = [&](uint32_t pos) {
-            return (uint32_t)(x0 - 1) + (pos & 1023u) + (uint32_t)nx * ((uint32_t)(y0 - 1) + (pos >> 10 & 1023u)) +
-                   nxy * ((uint32_t)(z0 - 1) + (pos >> 20));
+            return cell_place(a.g, x0 - 1 + (int)(pos & 1023u), y0 - 1 + (int)(pos >> 10 & 1023u), z0 - 1 + (int)(pos >> 20));
         };
         // J^{n+1/2}, P^{n+1} of the own gain cells (time-n values of own cells only)
         auto lorentz = [&](long long n) {
@@ -330,7 +329,9 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_step_small(const __grid_co
                 const float4 e = Es[m.ep];
                 float4 j = Js[q];
                 const float2 nn = Ns[q];
-                lorentz_step(a.gain, cell(m.pos), n, e.x, e.y, e.z, nn.x, nn.y, j.x, j.y, j.z, p.x, p.y, p.z);
+                lorentz_step(a.gain, cell_number(a.g, x0 - 1 + (int)(m.pos & 1023u), y0 - 1 + (int)(m.pos >> 10 & 1023u),
+                                                 z0 - 1 + (int)(m.pos >> 20)),
+                             n, e.x, e.y, e.z, nn.x, nn.y, j.x, j.y, j.z, p.x, p.y, p.z);
                 Ps[q] = p;
                 Js[q] = j;
             }

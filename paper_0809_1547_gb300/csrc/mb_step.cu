@@ -31,7 +31,7 @@ mb::DevPing ping_of(const mb_ctx* c, const mb::StepArgs& a, int q) {
 // Allocates the second copy on first use.
 int ensure_second_copy(mb_ctx* c) {
     if (c->d_fields2) return MB_OK;
-    const size_t fb = sizeof(float) * 6 * (size_t)c->ncell;
+    const size_t fb = sizeof(float) * 6 * (size_t)c->pcell;
     cudaError_t e = inject_alloc_failure() ? cudaErrorMemoryAllocation
                                            : cudaMalloc((void**)&c->d_fields2, fb);
     for (int w = 0; w < 3 && e == cudaSuccess; ++w)
@@ -134,6 +134,16 @@ cudaError_t launch_small(mb_ctx* c, int p, int m, bool with_probes) {
     return mb::launch_step_small(A, c->stream);
 }
 
+int step_graphs(mb_ctx* c, int p, bool fused, bool chunk, bool one);
+
+// The shortest interval between samples of the face and plane probes.
+int sample_interval(const mb_ctx* c) {
+    int m = mb::kSmallMaxSteps;
+    if (c->face.on) m = std::min(m, c->face.every);
+    for (const mb::DevPlaneProbe& q : c->planes) m = std::min(m, q.every);
+    return m;
+}
+
 // n steps from copy p by small-grid launches, each ending where a face or a
 // plane probe samples next (point probes run inside); *p: the copy at the end.
 int step_small(mb_ctx* c, int n, int* p) {
@@ -150,14 +160,11 @@ int step_small(mb_ctx* c, int n, int* p) {
         } else {
             // too few steps for the launch's loading and storing of the state
             set_parity(c, *p);
-            const mb::DevPointProbes pp{(int)c->probes.size(), c->probe_nfreq, c->d_probe_cell, c->d_probe_omega,
-                                        c->d_probe_acc};
-            for (int r = 0; r < m; ++r) {
-                mb::launch_h_pass(c->args, c->tune_h, tma_for(c, c->tune_h), c->stream);
-                mb::launch_e_pass(c->args, c->tune_e, tma_for(c, c->tune_e), c->stream);
-                mb::launch_point_dft(pp, c->args.f, c->d_ctr, c->dt, c->stream);
-            }
-            c->launches += (int64_t)m * (pp.count ? 3 : 2);
+            if (int rc = step_graphs(c, *p, false, false, true)) return rc;
+            for (int r = 0; r < m; ++r) MB_CUDA(c, cudaGraphLaunch(c->graph_one[*p], c->stream));
+            c->launches += (int64_t)m * launches_per_step(c, false);
+            done += m;
+            continue;   // (its probes are in the graph)
         }
         done += m;
         const mb::StepArgs out = view_of(c, *p);
@@ -278,7 +285,7 @@ using namespace mbi;
 bool mb::hold_in_place(mb_ctx* c) {
     const bool on = c->use_fused;
     if (c->parity) {
-        const size_t N = (size_t)c->ncell;
+        const size_t N = (size_t)c->pcell;
         cudaMemcpyAsync(c->d_fields, c->d_fields2, sizeof(float) * 6 * N, cudaMemcpyDeviceToDevice, c->stream);
         for (int w = 0; w < 3; ++w)
             if (c->psi_elems[w])
@@ -348,8 +355,11 @@ int mb_step(mb_ctx* c, int n) {
     if (n < 0) return fail(c, MB_ERR_ARG, "negative step count");
     if (n == 0) return MB_OK;
     bool fused = fused_ready(c);
-    // calls of a few steps between read-outs: the two passes' graphs
-    if (fused && small_on(c) && n < c->tune_f.kz) fused = false;
+    // calls of a few steps between read-outs, or sampling planes that cut the
+    // steps into shorter runs than repay a launch: the two passes' graphs
+    // (42 x 38 x 44 with a plane probe at every step: 1.14 ms for 53 steps and
+    // their read-outs against 1.59 cut into single steps)
+    if (fused && small_on(c) && std::min(n, sample_interval(c)) < c->tune_f.kz) fused = false;
     if (fused && small_on(c)) {
         mb::join_probes(c);
         int q = c->parity;
@@ -494,29 +504,43 @@ int mb_autotune(mb_ctx* c) {
     float best_h = 1e30f, best_e = 1e30f;
     mb::PassTune bh = c->tune_h, be = c->tune_e;
     const int reps = c->ncell > 4000000 ? 2 : 6;
-    for (const mb::PassTune& t : cands) {
-        if (t.variant != mb::kVariant3D && t.kz > 2 * c->nz) continue;
-        if (t.variant == mb::kVariantTma && !tma_for(c, t)) continue;
-        for (int pass = 0; pass < 2; ++pass) {
-            if (pass == 0) mb::launch_h_pass(c->args, t, tma_for(c, t), c->stream);
-            else mb::launch_e_pass(c->args, t, tma_for(c, t), c->stream);
-            cudaEventRecord(e0, c->stream);
-            for (int r = 0; r < reps; ++r) {
-                if (pass == 0) mb::launch_h_pass(c->args, t, tma_for(c, t), c->stream);
-                else mb::launch_e_pass(c->args, t, tma_for(c, t), c->stream);
+    // every shape by a launch or two, then the four fastest again, longer and
+    // twice interleaved
+    const int coarse = c->ncell > 4000000 ? 1 : 2;
+    for (int pass = 0; pass < 2; ++pass) {
+        auto time_pass = [&](const mb::PassTune& t, int n) -> float {
+            const mb::TmaMaps* m = tma_for(c, t);
+            for (int r = -1; r < n; ++r) {   // (one untimed)
+                if (r == 0) cudaEventRecord(e0, c->stream);
+                if (pass == 0) mb::launch_h_pass(c->args, t, m, c->stream);
+                else mb::launch_e_pass(c->args, t, m, c->stream);
             }
             cudaEventRecord(e1, c->stream);
             cudaEventSynchronize(e1);
             float ms = 0;
             cudaEventElapsedTime(&ms, e0, e1);
-            if (pass == 0 && ms < best_h) { best_h = ms; bh = t; }
-            if (pass == 1 && ms < best_e) { best_e = ms; be = t; }
+            return ms;
+        };
+        std::vector<std::pair<float, mb::PassTune>> tp;
+        for (const mb::PassTune& t : cands) {
+            if (t.variant != mb::kVariant3D && t.kz > 2 * c->nz) continue;
+            if (t.variant == mb::kVariantTma && !tma_for(c, t)) continue;
+            tp.push_back({time_pass(t, coarse), t});
+        }
+        std::sort(tp.begin(), tp.end(), [](const auto& x, const auto& y) { return x.first < y.first; });
+        if (tp.size() > 4) tp.resize(4);
+        for (auto& q : tp) q.first = 1e30f;
+        for (int round = 0; round < 2; ++round)
+            for (auto& q : tp) q.first = std::min(q.first, time_pass(q.second, reps));
+        for (const auto& q : tp) {
+            if (pass == 0 && q.first < best_h) { best_h = q.first; bh = q.second; }
+            if (pass == 1 && q.first < best_e) { best_e = q.first; be = q.second; }
         }
     }
     // the single-pass step against the best pair of passes
     mb::PassTune bf = c->tune_f;
     float best_f = 1e30f;
-    const bool tma = mb::tma_e_supported(c->args);
+    const bool tma = mb::fused_supported(c->args);
     if (tma || small_ready(c)) ensure_second_copy(c);
     if (tma && c->d_fields2) {
         // current copy -> other copy, repeated (the other copy is scratch)
@@ -541,7 +565,7 @@ int mb_autotune(mb_ctx* c) {
             for (int kz : {8, 12, 16, 20, 24, 32, 48, 64}) {
                 const mb::PassTune t{mb::kVariantTma, b, kz};
                 if (kz > 2 * c->nz) continue;
-                tf.push_back({time_fused(t, reps), t});
+                tf.push_back({time_fused(t, coarse), t});
             }
         // the three fastest again, longer and twice interleaved (neighbouring
         // shapes often time within a percent of each other): the best minimum
@@ -609,8 +633,9 @@ int mb_autotune(mb_ctx* c) {
 int mb_get_single_pass(mb_ctx* c, int tune[4]) {
     if (int rc = check_ctx(c)) return rc;
     if (!tune) return fail(c, MB_ERR_ARG, "null output");
-    // the small-grid launch is the tuner's choice alone: reported as off
-    tune[0] = c->use_fused && !small_on(c) ? 1 : 0;
+    // the small-grid launch, and the single-pass step on rows that are not a
+    // multiple of 16 cells, are the tuner's choice alone: reported as off
+    tune[0] = c->use_fused && !small_on(c) && mb::tma_e_supported(c->args) ? 1 : 0;
     tune[1] = c->tune_f.block.x;
     tune[2] = c->tune_f.block.y;
     tune[3] = c->tune_f.kz;

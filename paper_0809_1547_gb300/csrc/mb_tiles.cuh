@@ -67,7 +67,8 @@ __device__ __forceinline__ void gain_block(const StepArgs& a, unsigned gidx, int
     for (int r = 0; r < PER; ++r) {
         if (!ok[r]) continue;
         const uint32_t c = cs[r];
-        lorentz_step(a.gain, c, n, ex[r], ey[r], ez[r], n1[r], n2[r], jx[r], jy[r], jz[r], px[r],
+        const uint32_t num = a.glist.number ? __ldg(a.glist.number + base + (uint32_t)(r * T)) : c;
+        lorentz_step(a.gain, num, n, ex[r], ey[r], ez[r], n1[r], n2[r], jx[r], jy[r], jz[r], px[r],
                      py[r], pz[r]);
         f.jx[c] = jx[r];
         f.jy[c] = jy[r];
@@ -125,9 +126,10 @@ __device__ __forceinline__ void h_tile_zmarch(const StepArgs& a, int bx, int by,
     const float* __restrict__ Ex = a.f.ex;
     const float* __restrict__ Ey = a.f.ey;
     const float* __restrict__ Ez = a.f.ez;
+    const int px = a.g.px;
     const bool xi = i + 1 < nx, yj = j + 1 < ny;
     const bool pml_xy = tile_in_xy_slab(a, bx * blockDim.x, blockDim.x, by * blockDim.y, blockDim.y);
-    uint32_t c = (uint32_t)i + (uint32_t)nx * j + nxy * k0;
+    uint32_t c = (uint32_t)i + (uint32_t)a.g.px * j + nxy * k0;
     float ex_c = __ldg(Ex + c), ey_c = __ldg(Ey + c);
     int k = k0;
     // two planes per iteration: all loads of both are issued before either update
@@ -139,20 +141,20 @@ __device__ __forceinline__ void h_tile_zmarch(const StepArgs& a, int bx, int by,
         e0.ez = __ldg(Ez + c);
         e0.ex_k1 = __ldg(Ex + c + nxy);
         e0.ey_k1 = __ldg(Ey + c + nxy);
-        e0.ex_j1 = yj ? __ldg(Ex + c + nx) : 0.0f;
+        e0.ex_j1 = yj ? __ldg(Ex + c + px) : 0.0f;
         e0.ey_i1 = xi ? __ldg(Ey + c + 1) : 0.0f;
         e0.ez_i1 = xi ? __ldg(Ez + c + 1) : 0.0f;
-        e0.ez_j1 = yj ? __ldg(Ez + c + nx) : 0.0f;
+        e0.ez_j1 = yj ? __ldg(Ez + c + px) : 0.0f;
         const uint32_t c1 = c + nxy;
         e1.ex = e0.ex_k1;
         e1.ey = e0.ey_k1;
         e1.ez = __ldg(Ez + c1);
         e1.ex_k1 = zk ? __ldg(Ex + c1 + nxy) : 0.0f;
         e1.ey_k1 = zk ? __ldg(Ey + c1 + nxy) : 0.0f;
-        e1.ex_j1 = yj ? __ldg(Ex + c1 + nx) : 0.0f;
+        e1.ex_j1 = yj ? __ldg(Ex + c1 + px) : 0.0f;
         e1.ey_i1 = xi ? __ldg(Ey + c1 + 1) : 0.0f;
         e1.ez_i1 = xi ? __ldg(Ez + c1 + 1) : 0.0f;
-        e1.ez_j1 = yj ? __ldg(Ez + c1 + nx) : 0.0f;
+        e1.ez_j1 = yj ? __ldg(Ez + c1 + px) : 0.0f;
         if (pml_xy || plane_in_z_slab(a, k)) h_core<true>(a, i, j, k, c, e0);
         else h_core<false>(a, i, j, k, c, e0);
         if (pml_xy || plane_in_z_slab(a, k + 1)) h_core<true>(a, i, j, k + 1, c1, e1);
@@ -168,10 +170,10 @@ __device__ __forceinline__ void h_tile_zmarch(const StepArgs& a, int bx, int by,
         e.ez = __ldg(Ez + c);
         e.ex_k1 = zk ? __ldg(Ex + c + nxy) : 0.0f;
         e.ey_k1 = zk ? __ldg(Ey + c + nxy) : 0.0f;
-        e.ex_j1 = yj ? __ldg(Ex + c + nx) : 0.0f;
+        e.ex_j1 = yj ? __ldg(Ex + c + px) : 0.0f;
         e.ey_i1 = xi ? __ldg(Ey + c + 1) : 0.0f;
         e.ez_i1 = xi ? __ldg(Ez + c + 1) : 0.0f;
-        e.ez_j1 = yj ? __ldg(Ez + c + nx) : 0.0f;
+        e.ez_j1 = yj ? __ldg(Ez + c + px) : 0.0f;
         if (pml_xy || plane_in_z_slab(a, k)) h_core<true>(a, i, j, k, c, e);
         else h_core<false>(a, i, j, k, c, e);
     }
@@ -219,12 +221,12 @@ __device__ __forceinline__ void finish_step(const StepArgs& a, long long* sample
 template <bool FACE, bool PML_XY, bool KEEP = false>
 __device__ __forceinline__ void e_walk(const StepArgs& a, int i, int j, int k0, int k1, long long n,
                                        float fl[6], bool w_xy = false) {
-    const int nx = a.g.nx;
+    const int px = a.g.px;
     const uint32_t nxy = a.g.nxy;
     const float* __restrict__ Hx = a.f.hx;
     const float* __restrict__ Hy = a.f.hy;
     const float* __restrict__ Hz = a.f.hz;
-    uint32_t c = (uint32_t)i + (uint32_t)nx * j + nxy * k0;
+    uint32_t c = (uint32_t)i + (uint32_t)a.g.px * j + nxy * k0;
     float hx_km1 = 0.0f, hy_km1 = 0.0f;
     if (k0 > 0) {
         hx_km1 = __ldg(Hx + c - nxy);
@@ -237,8 +239,8 @@ __device__ __forceinline__ void e_walk(const StepArgs& a, int i, int j, int k0, 
         h.hz = __ldg(Hz + c);
         h.hx_k = hx_km1;
         h.hy_k = hy_km1;
-        h.hx_j = (j > 0) ? __ldg(Hx + c - nx) : 0.0f;
-        h.hz_j = (j > 0) ? __ldg(Hz + c - nx) : 0.0f;
+        h.hx_j = (j > 0) ? __ldg(Hx + c - px) : 0.0f;
+        h.hz_j = (j > 0) ? __ldg(Hz + c - px) : 0.0f;
         h.hy_i = (i > 0) ? __ldg(Hy + c - 1) : 0.0f;
         h.hz_i = (i > 0) ? __ldg(Hz + c - 1) : 0.0f;
         if (FACE || PML_XY) e_core<FACE, true, KEEP>(a, i, j, k, c, h, n, fl,
