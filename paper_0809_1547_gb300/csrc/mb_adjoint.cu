@@ -508,36 +508,37 @@ __global__ void __launch_bounds__(256, 6) k_adj_e_point(AdjArgs a) {
 
 // Store slot of a segment's first state (the E pass keeps the others as it
 // computes them; this copy also serves the quad-vectorised E pass, which
-// does not): E (arrays 0..2) and J, n1..n3 (arrays 9..14) of
-// the field block, Hx and Hy of plane kp, and the step counter.  16-byte
-// moves when n_cells and the plane size are multiples of 4 (every array then
-// starts 16-byte aligned).  The stores are marked streaming (evict first), so
+// does not): E (arrays 0..2 of the field block F) and J, n1..n3 (gs), Hx and
+// Hy of plane kp, and the step counter.  E and H by 16-byte moves when n_cells
+// and the plane size are multiples of 4 (every array then starts 16-byte
+// aligned).  The stores are marked streaming (evict first), so
 // the segment store (gigabytes) does not push the recomputed state out of
 // L2; the reverse kernels read the stored states the same way.
-__global__ void k_keep(const float* __restrict__ F, float* __restrict__ dst, uint32_t n,
+__global__ void k_keep(const float* __restrict__ F, const float* __restrict__ gs, float* __restrict__ dst, uint32_t n,
                        uint32_t nxy, int kp, const long long* __restrict__ ctr,
                        long long* __restrict__ slot_n) {
     if (blockIdx.x == 0 && threadIdx.x == 0) *slot_n = *ctr;
-    const size_t n3 = 3 * (size_t)n, n6 = 6 * (size_t)n;
+    const size_t n3 = 3 * (size_t)n;
     const size_t t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     const float* hpx = F + 3 * (size_t)n + (size_t)nxy * kp;
     const float* hpy = F + 4 * (size_t)n + (size_t)nxy * kp;
     float* dp = dst + 9 * (size_t)n;
+    for (size_t t = t0; t < n; t += stride) {
+        const float* g = gs + gain_place((uint32_t)t);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) __stcs(dst + n3 + q * (size_t)n + t, g[q * kGainCells]);
+    }
     if ((n & 3u) == 0 && (nxy & 3u) == 0) {
         const float4* a = reinterpret_cast<const float4*>(F);
-        const float4* b = reinterpret_cast<const float4*>(F + 9 * (size_t)n);
         float4* d = reinterpret_cast<float4*>(dst);
         for (size_t t = t0; t < n3 / 4; t += stride) __stcs(d + t, a[t]);
-        for (size_t t = t0; t < n6 / 4; t += stride) __stcs(d + n3 / 4 + t, b[t]);
         for (size_t t = t0; t < nxy / 4; t += stride) {
             __stcs(reinterpret_cast<float4*>(dp) + t, reinterpret_cast<const float4*>(hpx)[t]);
             __stcs(reinterpret_cast<float4*>(dp + nxy) + t, reinterpret_cast<const float4*>(hpy)[t]);
         }
     } else {
-        const float* b = F + 9 * (size_t)n;
         for (size_t t = t0; t < n3; t += stride) __stcs(dst + t, F[t]);
-        for (size_t t = t0; t < n6; t += stride) __stcs(dst + n3 + t, b[t]);
         for (size_t t = t0; t < nxy; t += stride) {
             __stcs(dp + t, hpx[t]);
             __stcs(dp + nxy + t, hpy[t]);
@@ -644,7 +645,7 @@ extern "C" int mb_adjoint_energy_zface(mb_ctx* c, int n_steps, int ckpt_every, i
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int keep_blocks = (int)std::max<size_t>(1, std::min<size_t>((6 * N / 4 + 255) / 256, (size_t)sms * 8));
     auto keep = [&](int t) -> cudaError_t {
-        mb::k_keep<<<keep_blocks, 256, 0, c->stream>>>(F, store + slot * t, (uint32_t)N, (uint32_t)nxy,
+        mb::k_keep<<<keep_blocks, 256, 0, c->stream>>>(F, c->args.f.gs, store + slot * t, (uint32_t)N, (uint32_t)nxy,
                                                        zp - 1, c->d_ctr, slot_n + t);
         return cudaGetLastError();
     };

@@ -13,7 +13,6 @@
 #include <map>
 #include <memory>
 #include <mutex>
-#include <new>
 #include <thread>
 
 using mb::kC0;
@@ -99,12 +98,17 @@ std::pair<int, int> interior(int n, int L) {
 float* eh_of(const mb_ctx* c, int p) { return p ? c->d_fields2 : c->d_fields; }
 float* psi_of(const mb_ctx* c, int p, int w) { return p ? c->d_psi2[w] : c->d_psi[w]; }
 
-float* field_ptr(mb_ctx* c, int which) {
-    // layout: ex ey ez hx hy hz (current copy), px py pz jx jy jz n1 n2 n3
-    if (which < MB_EX || which > MB_N3 || which == MB_N0) return nullptr;
-    const int slot = which < MB_N0 ? which : which - 1;
-    if (slot < 6) return eh_of(c, c->parity) + (int64_t)slot * c->pcell;
-    return c->d_fields + (int64_t)slot * c->pcell;
+// Floats of d_fields before the gain blocks (whole 256 bytes).
+size_t gain_offset(const mb_ctx* c) { return (6 * (size_t)c->pcell + 63) / 64 * 64; }
+
+// An E or H array of the current copy.
+float* eh_ptr(mb_ctx* c, int which) { return eh_of(c, c->parity) + (int64_t)which * c->pcell; }
+
+// Where a field of P, J or the populations sits in the gain blocks.
+int gain_comp(int which) {
+    if (which <= MB_PZ) return mb::kPx + (which - MB_PX) * mb::kGainCells;
+    if (which <= MB_JZ) return mb::kJx + (which - MB_JX) * mb::kGainCells;
+    return mb::kN1 + (which - MB_N1) * mb::kGainCells;
 }
 
 // Points the step arguments' E, H and CPML memories at copy p.
@@ -140,11 +144,7 @@ void z_cpml_bounds(const mb_ctx* c, mb::DevCpml& m) {
 void build_args(mb_ctx* c) {
     mb::StepArgs& a = c->args;
     a.g = {c->nx, c->ny, c->nz, (uint32_t)c->px * (uint32_t)c->ny, (uint32_t)c->pcell, c->px};
-    float* F = c->d_fields;
-    const int64_t N = c->pcell;
-    a.f.px = F + 6 * N; a.f.py = F + 7 * N; a.f.pz = F + 8 * N;
-    a.f.jx = F + 9 * N; a.f.jy = F + 10 * N; a.f.jz = F + 11 * N;
-    a.f.n1 = F + 12 * N; a.f.n2 = F + 13 * N; a.f.n3 = F + 14 * N;
+    a.f.gs = c->d_fields + gain_offset(c);
     a.f.mat = c->d_mat;
     a.f.inv_eps = c->dense_eps ? c->d_inv_eps : nullptr;
     a.f.lut_inv_eps = c->d_lut;
@@ -274,7 +274,7 @@ int check_ctx(mb_ctx* c) {
 std::vector<StatePart> state_parts(mb_ctx* c) {
     std::vector<StatePart> v;
     v.push_back({eh_of(c, c->parity), sizeof(float) * 6 * (size_t)c->pcell, 6});
-    v.push_back({c->d_fields + 6 * c->pcell, sizeof(float) * 9 * (size_t)c->pcell, 9});
+    v.push_back({c->args.f.gs, sizeof(float) * mb::gain_floats(c->pcell), mb::kGainComps, true});
     for (int w = 0; w < 3; ++w)
         if (c->psi_elems[w]) v.push_back({psi_of(c, c->parity, w), sizeof(float) * c->psi_elems[w]});
     v.push_back({c->d_ctr, sizeof(long long) * 2});
@@ -294,71 +294,78 @@ size_t host_bytes(const mb_ctx* c, const StatePart& p) {
     return p.arrays ? sizeof(float) * (size_t)p.arrays * c->ncell : p.bytes;
 }
 
-// Padded rows are packed and spread by a kernel (a 2-D device copy of rows of
-// 157 floats measured 13 us more than the plain copy; the kernel as much as
-// it).  To and from the host they cross packed, an array at a time through
-// the material's upload buffer (2.7 M cells: a field read 1.7 ms as without
-// padding; packed on the host 2.7 ms); before a material is set, through a
-// host buffer, with zeros in the padding as the device's rows hold.
-cudaError_t rows_out(const mb_ctx* c, void* packed, const void* rows, size_t esize, int arrays, cudaMemcpyKind kind) {
+// The material's upload buffer (made here where no material is set yet).
+bool ensure_upload(mb_ctx* c) {
+    if (c->d_upload) return true;
+    const size_t bytes = 5 * (size_t)c->ncell + 16;
+    if (cudaMalloc((void**)&c->d_upload, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        c->d_upload = nullptr;
+        return false;
+    }
+    c->upload_bytes = bytes;
+    return true;
+}
+
+// Padded rows and the gain blocks are packed and spread by kernels (a 2-D
+// device copy of rows of 157 floats measured 13 us more than the plain copy;
+// the kernel as much as it).  To and from the host they cross packed, an array
+// at a time through the material's upload buffer (2.7 M cells: a field read
+// 1.7 ms as without padding; packed on the host 2.7 ms).
+cudaError_t rows_out(mb_ctx* c, void* packed, const void* rows, size_t esize, int arrays, cudaMemcpyKind kind) {
     if (c->px == c->nx)
         return cudaMemcpyAsync(packed, rows, esize * (size_t)arrays * c->ncell, kind, c->stream);
     const int64_t nrow = (int64_t)c->ny * c->nz;
-    const size_t to = esize * c->nx, from = esize * c->px;
+    const size_t to = esize * c->nx * nrow, from = esize * c->px * nrow;
     if (kind == cudaMemcpyDeviceToDevice) {
         mb::launch_rows(rows, c->px, packed, c->nx, c->nx, nrow * arrays, (int)esize, c->stream);
         return cudaGetLastError();
     }
-    if (c->upload_bytes >= to * nrow) {
-        for (int q = 0; q < arrays; ++q) {
-            mb::launch_rows((const char*)rows + from * nrow * q, c->px, c->d_upload, c->nx, c->nx, nrow, (int)esize,
-                            c->stream);
-            cudaError_t e = cudaMemcpyAsync((char*)packed + to * nrow * q, c->d_upload, to * nrow, kind, c->stream);
-            if (e != cudaSuccess) return e;
-        }
-        return cudaGetLastError();
-    }
-    std::unique_ptr<char[]> tmp(new (std::nothrow) char[from * nrow]);
-    if (!tmp) return cudaErrorMemoryAllocation;
+    if (!ensure_upload(c)) return cudaErrorMemoryAllocation;
     for (int q = 0; q < arrays; ++q) {
-        const char* src = (const char*)rows + from * nrow * q;
-        char* dst = (char*)packed + to * nrow * q;
-        cudaError_t e = cudaMemcpyAsync(tmp.get(), src, from * nrow, kind, c->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        mb::launch_rows((const char*)rows + from * q, c->px, c->d_upload, c->nx, c->nx, nrow, (int)esize, c->stream);
+        cudaError_t e = cudaMemcpyAsync((char*)packed + to * q, c->d_upload, to, kind, c->stream);
         if (e != cudaSuccess) return e;
-        for (int64_t r = 0; r < nrow; ++r) std::memcpy(dst + to * r, tmp.get() + from * r, to);
     }
-    return cudaSuccess;
+    return cudaGetLastError();
 }
-cudaError_t rows_in(const mb_ctx* c, void* rows, const void* packed, size_t esize, int arrays, cudaMemcpyKind kind) {
+cudaError_t rows_in(mb_ctx* c, void* rows, const void* packed, size_t esize, int arrays, cudaMemcpyKind kind) {
     if (c->px == c->nx)
         return cudaMemcpyAsync(rows, packed, esize * (size_t)arrays * c->ncell, kind, c->stream);
     const int64_t nrow = (int64_t)c->ny * c->nz;
-    const size_t to = esize * c->px, from = esize * c->nx;
+    const size_t to = esize * c->px * nrow, from = esize * c->nx * nrow;
     if (kind == cudaMemcpyDeviceToDevice) {
         mb::launch_rows(packed, c->nx, rows, c->px, c->nx, nrow * arrays, (int)esize, c->stream);
         return cudaGetLastError();
     }
-    if (c->upload_bytes >= from * nrow) {
-        for (int q = 0; q < arrays; ++q) {
-            cudaError_t e = cudaMemcpyAsync(c->d_upload, (const char*)packed + from * nrow * q, from * nrow, kind,
-                                            c->stream);
-            if (e != cudaSuccess) return e;
-            mb::launch_rows(c->d_upload, c->nx, (char*)rows + to * nrow * q, c->px, c->nx, nrow, (int)esize, c->stream);
-        }
-        return cudaGetLastError();
-    }
-    std::unique_ptr<char[]> tmp(new (std::nothrow) char[to * nrow]());
-    if (!tmp) return cudaErrorMemoryAllocation;
+    if (!ensure_upload(c)) return cudaErrorMemoryAllocation;
     for (int q = 0; q < arrays; ++q) {
-        const char* src = (const char*)packed + from * nrow * q;
-        for (int64_t r = 0; r < nrow; ++r) std::memcpy(tmp.get() + to * r, src + from * r, from);
-        cudaError_t e = cudaMemcpyAsync((char*)rows + to * nrow * q, tmp.get(), to * nrow, kind, c->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        cudaError_t e = cudaMemcpyAsync(c->d_upload, (const char*)packed + from * q, from, kind, c->stream);
         if (e != cudaSuccess) return e;
+        mb::launch_rows(c->d_upload, c->nx, (char*)rows + to * q, c->px, c->nx, nrow, (int)esize, c->stream);
     }
-    return cudaSuccess;
+    return cudaGetLastError();
 }
+cudaError_t field_out(mb_ctx* c, void* packed, int which, cudaMemcpyKind kind) {
+    if (which < MB_PX) return rows_out(c, packed, eh_ptr(c, which), 4, 1, kind);
+    const bool dev = kind == cudaMemcpyDeviceToDevice;
+    if (!dev && !ensure_upload(c)) return cudaErrorMemoryAllocation;
+    float* to = dev ? (float*)packed : (float*)c->d_upload;
+    mb::launch_gain_rows(c->args.f.gs, gain_comp(which), c->px, to, c->nx, (int64_t)c->ny * c->nz, true, c->stream);
+    if (!dev) cudaMemcpyAsync(packed, to, sizeof(float) * (size_t)c->ncell, kind, c->stream);
+    return cudaGetLastError();
+}
+cudaError_t field_in(mb_ctx* c, int which, const void* packed, cudaMemcpyKind kind) {
+    if (which < MB_PX) return rows_in(c, eh_ptr(c, which), packed, 4, 1, kind);
+    if (!ensure_upload(c)) return cudaErrorMemoryAllocation;
+    float* from = (float*)c->d_upload;
+    cudaError_t e = cudaMemcpyAsync(from, packed, sizeof(float) * (size_t)c->ncell, kind, c->stream);
+    if (e != cudaSuccess) return e;
+    mb::launch_gain_rows(c->args.f.gs, gain_comp(which), c->px, from, c->nx, (int64_t)c->ny * c->nz, false, c->stream);
+    return cudaGetLastError();
+}
+// The gain fields in blob order.
+constexpr int kGainFields[9] = {MB_PX, MB_PY, MB_PZ, MB_JX, MB_JY, MB_JZ, MB_N1, MB_N2, MB_N3};
 
 // Tensor maps for a TMA tuning over the current copy (encoded once per tile
 // shape and copy), else nullptr.
@@ -758,7 +765,8 @@ static int create_ctx(mb_ctx** out, const int grid[3], int gnz, int kz0, int own
         return MB_OK;
     };
     int rc;
-    rc = alloc((void**)&c->d_fields, sizeof(float) * 15 * (size_t)c->pcell);
+    const size_t field_bytes = sizeof(float) * (gain_offset(c) + mb::gain_floats(c->pcell));
+    rc = alloc((void**)&c->d_fields, field_bytes);
     if (rc) return bail(rc);
     if ((rc = alloc((void**)&c->d_mat, (size_t)c->pcell))) return bail(rc);
     if ((rc = alloc((void**)&c->d_lut, sizeof(float) * 256))) return bail(rc);
@@ -808,7 +816,7 @@ static int create_ctx(mb_ctx** out, const int grid[3], int gnz, int kz0, int own
     } while (0)
     MB_CREATE_CUDA(cudaMemcpy(c->d_coef, coef.data(), sizeof(float) * ncoef, cudaMemcpyHostToDevice));
     MB_CREATE_CUDA(cudaMemcpy(c->d_lut, lut.data(), sizeof(float) * 256, cudaMemcpyHostToDevice));
-    MB_CREATE_CUDA(cudaMemset(c->d_fields, 0, sizeof(float) * 15 * (size_t)c->pcell));
+    MB_CREATE_CUDA(cudaMemset(c->d_fields, 0, field_bytes));
     MB_CREATE_CUDA(cudaMemset(c->d_mat, 0, (size_t)c->pcell));
     for (int w = 0; w < 3; ++w)
         if (c->psi_elems[w]) MB_CREATE_CUDA(cudaMemset(c->d_psi[w], 0, sizeof(float) * c->psi_elems[w]));
@@ -1036,7 +1044,7 @@ int mb_set_material(mb_ctx* c, const float* eps_map, const uint8_t* gain_mask, d
     c->W_p = pump;
     c->glist_count = (uint32_t)n_gain;
     // reset P, J and the populations (N0 = N_a, n1 = n2 = n3 = 0)
-    MB_CUDA(c, cudaMemsetAsync(c->d_fields + 6 * c->pcell, 0, sizeof(float) * 9 * (size_t)c->pcell, c->stream));
+    MB_CUDA(c, cudaMemsetAsync(c->args.f.gs, 0, sizeof(float) * mb::gain_floats(c->pcell), c->stream));
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
     c->have_material = true;
     build_args(c);
@@ -1450,8 +1458,7 @@ int mb_energy(mb_ctx* c, double* out_U, double* out_flux6) {
     const int64_t off = (int64_t)c->own_lo * c->px * c->ny;   // (padding: zero fields)
     const int64_t own = (int64_t)(c->own_hi - c->own_lo) * c->px * c->ny;
     mb::DevFields f = c->args.f;
-    for (float** q : {&f.ex, &f.ey, &f.ez, &f.hx, &f.hy, &f.hz, &f.px, &f.py, &f.pz, &f.jx, &f.jy,
-                      &f.jz, &f.n1, &f.n2, &f.n3})
+    for (float** q : {&f.ex, &f.ey, &f.ez, &f.hx, &f.hy, &f.hz})
         *q += off;
     f.mat += off;
     if (f.inv_eps) f.inv_eps += off;
@@ -1519,9 +1526,9 @@ int mb_get_field(mb_ctx* c, int which, float* host_out) {
     if (which == MB_N0) {
         std::vector<float> a((size_t)N), b((size_t)N), d((size_t)N);
         std::vector<uint8_t> m((size_t)N, 0);
-        MB_CUDA(c, rows_out(c, a.data(), field_ptr(c, MB_N1), 4, 1, cudaMemcpyDeviceToHost));
-        MB_CUDA(c, rows_out(c, b.data(), field_ptr(c, MB_N2), 4, 1, cudaMemcpyDeviceToHost));
-        MB_CUDA(c, rows_out(c, d.data(), field_ptr(c, MB_N3), 4, 1, cudaMemcpyDeviceToHost));
+        MB_CUDA(c, field_out(c, a.data(), MB_N1, cudaMemcpyDeviceToHost));
+        MB_CUDA(c, field_out(c, b.data(), MB_N2, cudaMemcpyDeviceToHost));
+        MB_CUDA(c, field_out(c, d.data(), MB_N3, cudaMemcpyDeviceToHost));
         if (c->have_material)
             MB_CUDA(c, rows_out(c, m.data(), c->d_mat, 1, 1, cudaMemcpyDeviceToHost));
         MB_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -1529,7 +1536,7 @@ int mb_get_field(mb_ctx* c, int which, float* host_out) {
             host_out[q] = (m[q] & 0x80) ? (float)(c->N_a * (1.0 - (double)a[q] - (double)b[q] - (double)d[q])) : 0.0f;
         return MB_OK;
     }
-    MB_CUDA(c, rows_out(c, tmp.data(), field_ptr(c, which), 4, 1, cudaMemcpyDeviceToHost));
+    MB_CUDA(c, field_out(c, tmp.data(), which, cudaMemcpyDeviceToHost));
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
     const double s = field_scale(c, which);
     for (int64_t q = 0; q < N; ++q) host_out[q] = (float)(s * (double)tmp[q]);
@@ -1546,7 +1553,7 @@ int mb_set_field(mb_ctx* c, int which, const float* host_in) {
     std::vector<float> tmp((size_t)N);
     for (int64_t q = 0; q < N; ++q) tmp[q] = (float)(s * (double)host_in[q]);
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
-    MB_CUDA(c, rows_in(c, field_ptr(c, which), tmp.data(), 4, 1, cudaMemcpyHostToDevice));
+    MB_CUDA(c, field_in(c, which, tmp.data(), cudaMemcpyHostToDevice));
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
     return MB_OK;
 }
@@ -1555,7 +1562,7 @@ int mb_get_field_device(mb_ctx* c, int which, float* dev_out, double* scale) {
     if (int rc = check_ctx(c)) return rc;
     if (!dev_out || which < 0 || which >= MB_NUM_FIELDS || which == MB_N0)
         return fail(c, MB_ERR_ARG, "bad field id (N0 is not stored) or null output");
-    MB_CUDA(c, rows_out(c, dev_out, field_ptr(c, which), 4, 1, cudaMemcpyDeviceToDevice));
+    MB_CUDA(c, field_out(c, dev_out, which, cudaMemcpyDeviceToDevice));
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
     if (scale) *scale = field_scale(c, which);
     return MB_OK;
@@ -1577,7 +1584,10 @@ int mb_save_state(mb_ctx* c, void* host_blob, size_t* bytes) {
     std::memcpy(o, hdr, sizeof(hdr));
     o += sizeof(hdr);
     for (auto& p : parts) {
-        if (p.arrays) MB_CUDA(c, rows_out(c, o, p.ptr, 4, p.arrays, cudaMemcpyDeviceToHost));
+        if (p.gain)
+            for (int q = 0; q < 9; ++q)
+                MB_CUDA(c, field_out(c, o + sizeof(float) * (size_t)c->ncell * q, kGainFields[q], cudaMemcpyDeviceToHost));
+        else if (p.arrays) MB_CUDA(c, rows_out(c, o, p.ptr, 4, p.arrays, cudaMemcpyDeviceToHost));
         else MB_CUDA(c, cudaMemcpyAsync(o, p.ptr, p.bytes, cudaMemcpyDeviceToHost, c->stream));
         o += host_bytes(c, p);
     }
@@ -1598,7 +1608,10 @@ int mb_load_state(mb_ctx* c, const void* host_blob, size_t bytes) {
     const char* o = (const char*)host_blob + 4 * sizeof(int64_t);
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
     for (auto& p : parts) {
-        if (p.arrays) MB_CUDA(c, rows_in(c, p.ptr, o, 4, p.arrays, cudaMemcpyHostToDevice));
+        if (p.gain)
+            for (int q = 0; q < 9; ++q)
+                MB_CUDA(c, field_in(c, kGainFields[q], o + sizeof(float) * (size_t)c->ncell * q, cudaMemcpyHostToDevice));
+        else if (p.arrays) MB_CUDA(c, rows_in(c, p.ptr, o, 4, p.arrays, cudaMemcpyHostToDevice));
         else MB_CUDA(c, cudaMemcpyAsync(p.ptr, o, p.bytes, cudaMemcpyHostToDevice, c->stream));
         o += host_bytes(c, p);
     }

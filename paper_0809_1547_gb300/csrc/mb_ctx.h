@@ -60,14 +60,22 @@ void point_args_at(mb::StepArgs& a, const mb_ctx* c, int p);
 struct StatePart {
     void* ptr;
     size_t bytes;     // on the device
-    int arrays = 0;   // grid arrays of floats among them (rows px apart; a host blob holds n_x of each row)
+    // how many grid arrays of floats it holds (0: none), which a host blob
+    // holds packed, n_x of each row: E and H (gain false), or P, J, n1..n3
+    int arrays = 0;
+    bool gain = false;
 };
 size_t host_bytes(const mb_ctx* c, const StatePart& p);
 
 // Copies of `arrays` consecutive grid arrays of esize-byte elements between
-// the device's rows and a packed buffer (host or device).
-cudaError_t rows_out(const mb_ctx* c, void* packed, const void* rows, size_t esize, int arrays, cudaMemcpyKind kind);
-cudaError_t rows_in(const mb_ctx* c, void* rows, const void* packed, size_t esize, int arrays, cudaMemcpyKind kind);
+// the device's rows and a packed buffer (host or device), and of a field by
+// its id.
+cudaError_t rows_out(mb_ctx* c, void* packed, const void* rows, size_t esize, int arrays, cudaMemcpyKind kind);
+cudaError_t rows_in(mb_ctx* c, void* rows, const void* packed, size_t esize, int arrays, cudaMemcpyKind kind);
+cudaError_t field_out(mb_ctx* c, void* packed, int which, cudaMemcpyKind kind);
+cudaError_t field_in(mb_ctx* c, int which, const void* packed, cudaMemcpyKind kind);
+// P, J and the populations: the context's blocks of them and their floats.
+size_t gain_offset(const mb_ctx* c);
 std::vector<StatePart> state_parts(mb_ctx* c);
 
 // Tensor maps of the two-pass TMA launches over the current copy, else nullptr.

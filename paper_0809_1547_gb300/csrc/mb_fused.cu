@@ -170,16 +170,16 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
         return (smem + s * Lay::kStage + 3 * Lay::kEBytes + 3 * Lay::kHBytes)[tcell];
     };
     auto gslot = [&](int b, int q) -> float* { return gbuf + (b * 9 + q) * T + tid; };
-    auto prefetch_gain = [&](int b, uint32_t cc) {
-        cp_async_4(gslot(b, 0), f.px + cc);
-        cp_async_4(gslot(b, 1), f.py + cc);
-        cp_async_4(gslot(b, 2), f.pz + cc);
-        cp_async_4(gslot(b, 3), f.jx + cc);
-        cp_async_4(gslot(b, 4), f.jy + cc);
-        cp_async_4(gslot(b, 5), f.jz + cc);
-        cp_async_4(gslot(b, 6), f.n1 + cc);
-        cp_async_4(gslot(b, 7), f.n2 + cc);
-        cp_async_4(gslot(b, 8), f.n3 + cc);
+    auto prefetch_gain = [&](int b, const float* g) {
+        cp_async_4(gslot(b, 0), g + kPx);
+        cp_async_4(gslot(b, 1), g + kPy);
+        cp_async_4(gslot(b, 2), g + kPz);
+        cp_async_4(gslot(b, 3), g + kJx);
+        cp_async_4(gslot(b, 4), g + kJy);
+        cp_async_4(gslot(b, 5), g + kJz);
+        cp_async_4(gslot(b, 6), g + kN1);
+        cp_async_4(gslot(b, 7), g + kN2);
+        cp_async_4(gslot(b, 8), g + kN3);
     };
 
     if (tid == 0) {
@@ -246,7 +246,8 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
     }
     bool fail = !mbar_wait_bounded(&bar[0], 0, kWaitLimit);
     bool pg = valid && gain_on && ((MATG ? m0 : mat_of(0)) & 0x80);
-    if (pg) prefetch_gain(0, c);
+    float* g0 = f.gs + gain_place(c);   // the cell's gain block, plane p
+    if (pg) prefetch_gain(0, g0);
     cp_async_commit();
     // ring slots of planes p and p + 1, and the phase parity of plane p + 1
     int s = 0, s1 = 1 % S;
@@ -258,9 +259,10 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
         uint8_t m2 = 0;
         if (MATG && valid && p + 2 < planes) m2 = __ldg(f.mat + c + 2 * nxy);
         bool ng = false;
+        float* g1 = f.gs + gain_place(c + nxy);   // (plane p + 1; used where ng)
         if (p + 1 < planes) {
             ng = valid && gain_on && ((MATG ? m1 : mat_of(s1)) & 0x80);
-            if (ng) prefetch_gain((p + 1) & 1, c + nxy);
+            if (ng) prefetch_gain((p + 1) & 1, g1);
         }
         cp_async_commit();
         const float* E0 = reinterpret_cast<const float*>(smem + s * Lay::kStage);
@@ -340,12 +342,12 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
             n3 = *gslot(b, 8);
             lorentz_step(a.gain, cell_number(a.g, i, j, k), n, E0[own_e], E0[EW + own_e], E0[2 * EW + own_e], n1, n2, jx,
                          jy, jz, px, py, pz);
-            __stcs(f.px + c, px);
-            __stcs(f.py + c, py);
-            __stcs(f.pz + c, pz);
-            __stcs(f.jx + c, jx);
-            __stcs(f.jy + c, jy);
-            __stcs(f.jz + c, jz);
+            __stcs(g0 + kPx, px);
+            __stcs(g0 + kPy, py);
+            __stcs(g0 + kPz, pz);
+            __stcs(g0 + kJx, jx);
+            __stcs(g0 + kJy, jy);
+            __stcs(g0 + kJz, jz);
         }
         __syncthreads();   // the H tile is complete
 
@@ -379,9 +381,9 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
             __stcs(d.ey + c, ey1);
             __stcs(d.ez + c, ez1);
             if (pg) {
-                __stcs(f.n1 + c, n1);
-                __stcs(f.n2 + c, n2);
-                __stcs(f.n3 + c, n3);
+                __stcs(g0 + kN1, n1);
+                __stcs(g0 + kN2, n2);
+                __stcs(g0 + kN3, n3);
             }
             hx_km1 = hx;
             hy_km1 = hy;
@@ -409,6 +411,7 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
             issued = p + S + 1;
         }
         pg = ng;
+        g0 = g1;
         m0 = m1;
         m1 = m2;
         c += nxy;

@@ -20,7 +20,7 @@ namespace {
 // One plane of a context's state, at local plane k of the current copy.
 struct HaloPlane {
     float* eh;       // E, H of the current copy (6 arrays of N floats)
-    float* fields;   // the context's 15 arrays (P, J, n1..n3 from array 6)
+    float* gs;       // P, J, n1..n3
     float* psx;      // x-slab CPML memories of the current copy (or null)
     float* psy;      // y-slab CPML memories of the current copy (or null)
     int64_t N;       // cells of an array, rows px apart
@@ -46,9 +46,11 @@ __device__ __forceinline__ float* halo_addr(const HaloPlane& h, int64_t q) {
     if (q < a) {
         const int64_t seg = q / h.nxy;
         const int64_t r = q - seg * h.nxy;
-        float* base = (seg < 6 ? h.eh : h.fields) + seg * h.N;
         const int64_t j = r / h.nx;
-        return base + ((int64_t)h.k * h.ny + j) * h.px + (r - j * h.nx);
+        const int64_t c = ((int64_t)h.k * h.ny + j) * h.px + (r - j * h.nx);
+        if (seg < 6) return h.eh + seg * h.N + c;
+        // (P, J, n1..n3 in the plane's order)
+        return h.gs + mb::gain_place((uint32_t)c) + (seg < 9 ? mb::kPx + (seg - 6) * mb::kGainCells : (seg - 9) * mb::kGainCells);
     }
     q -= a;
     const int64_t bx = (int64_t)h.ny * h.L2;
@@ -75,7 +77,7 @@ __global__ void k_halo(HaloPlane h, float* buf, int64_t total) {
 int halo_launch(mb_ctx* c, int k, float* buf, bool pack) {
     HaloPlane h;
     h.eh = mbi::eh_of(c, c->parity);
-    h.fields = c->d_fields;
+    h.gs = c->args.f.gs;
     h.psx = mbi::psi_of(c, c->parity, 0);
     h.psy = mbi::psi_of(c, c->parity, 1);
     h.N = c->pcell;

@@ -279,6 +279,9 @@ void launch_gain_numbers(const uint32_t* list, uint32_t n, int nx, int px, uint3
 // `count` rows of nx elements (1 or 4 bytes) from rows `from` elements apart
 // to rows `to` elements apart.
 void launch_rows(const void* src, int from, void* dst, int to, int nx, int64_t count, int esize, cudaStream_t s);
+// Component comp (kJx, ..) of the cells of `count` rows of nx between the gain
+// blocks (rows px cells apart) and a packed device array.
+void launch_gain_rows(float* gs, int comp, int px, float* packed, int nx, int64_t count, bool out, cudaStream_t s);
 // The material map on the device: the distinct eps_r values into keys
 // (kMatKeys entries, kNoKey where unused, filled as a prefix) with the first
 // cell of each into first (initialised to kNoKey; flags[0]: a value not
@@ -366,7 +369,7 @@ struct mb_ctx {
     double E0 = 0, eta0 = 0, S = 0;
 
     // device memory
-    float* d_fields = nullptr;         // 15 arrays of ncell floats
+    float* d_fields = nullptr;         // 6 arrays of pcell floats (E, H), then the gain blocks
     uint8_t* d_mat = nullptr;
     float* d_inv_eps = nullptr;        // dense 1/eps_r (only when > 128 materials)
     float* d_lut = nullptr;            // [0..127]: 1/eps_r, [128..255]: eps_r

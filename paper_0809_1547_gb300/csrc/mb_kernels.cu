@@ -523,6 +523,39 @@ void launch_rows(const void* src, int from, void* dst, int to, int nx, int64_t c
         k_rows<uint8_t><<<blocks, 256, 0, s>>>((const uint8_t*)src, from, (uint8_t*)dst, to, nx, count);
 }
 
+// One component of P, J or the populations (its place comp floats into the
+// blocks) to (OUT) or from the packed array, a row a warp.
+template <bool OUT>
+__global__ void __launch_bounds__(256) k_gain_rows(float* __restrict__ gs, int comp, int px, float* __restrict__ packed,
+                                                   int nx, int64_t count) {
+    const int lane = threadIdx.x & 31;
+    const int64_t step = (int64_t)gridDim.x * 8;
+    for (int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); r < count; r += step) {
+        float* b = packed + r * nx;
+        for (int i = lane; i < nx; i += 128) {
+            float v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int x = i + 32 * q;
+                if (x < nx) v[q] = OUT ? gs[gain_place((uint32_t)(r * px + x)) + comp] : b[x];
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int x = i + 32 * q;
+                if (x < nx) {
+                    if (OUT) b[x] = v[q];
+                    else gs[gain_place((uint32_t)(r * px + x)) + comp] = v[q];
+                }
+            }
+        }
+    }
+}
+void launch_gain_rows(float* gs, int comp, int px, float* packed, int nx, int64_t count, bool out, cudaStream_t s) {
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((count + 7) / 8, 152 * 64));
+    if (out) k_gain_rows<true><<<blocks, 256, 0, s>>>(gs, comp, px, packed, nx, count);
+    else k_gain_rows<false><<<blocks, 256, 0, s>>>(gs, comp, px, packed, nx, count);
+}
+
 // ------------------------------------------------------------ material map
 // The eps_r map's distinct values (bit patterns) into a table of kMatKeys
 // entries by compare-and-swap on the first free slot, so the table fills as

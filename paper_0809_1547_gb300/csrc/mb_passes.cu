@@ -232,9 +232,10 @@ __device__ __forceinline__ void e_vec_walk(const StepArgs& a, int i0, int j, int
             const uint32_t m4 = __ldg(reinterpret_cast<const uint32_t*>(f.mat + c));
             const bool any_gain = gain_on && (m4 & 0x80808080u);
             float4 jx = zero, jy = zero, jz = zero, n1 = zero, n2 = zero, n3 = zero;
+            float* g = f.gs + gain_place(c);   // (the quad's four cells share a block)
             if (any_gain) {
-                jx = ld4(f.jx + c); jy = ld4(f.jy + c); jz = ld4(f.jz + c);
-                n1 = ld4(f.n1 + c); n2 = ld4(f.n2 + c); n3 = ld4(f.n3 + c);
+                jx = ld4(g + kJx); jy = ld4(g + kJy); jz = ld4(g + kJz);
+                n1 = ld4(g + kN1); n2 = ld4(g + kN2); n3 = ld4(g + kN3);
             }
             float4 ex1, ey1, ez1;
             if (FACE && plane_has_flux(a.flux, true, w_xy, k))
@@ -250,9 +251,9 @@ __device__ __forceinline__ void e_vec_walk(const StepArgs& a, int i0, int j, int
             st4(f.ey + c, ey1);
             st4(f.ez + c, ez1);
             if (any_gain) {
-                st4(f.n1 + c, n1);
-                st4(f.n2 + c, n2);
-                st4(f.n3 + c, n3);
+                st4(g + kN1, n1);
+                st4(g + kN2, n2);
+                st4(g + kN3, n3);
             }
         }
         hxk = hx;
@@ -336,12 +337,13 @@ __global__ void __launch_bounds__(BX * BY) k_e_tma(StepArgs a, const __grid_cons
     // J and n1..n3 of a gain cell, one plane ahead, into buffer b (no registers held)
     auto gslot = [&](int b, int q) -> float* { return gbuf + (b * 6 + q) * (BX * BY) + tid; };
     auto prefetch_gain = [&](int b, uint32_t cc) {
-        cp_async_4(gslot(b, 0), f.jx + cc);
-        cp_async_4(gslot(b, 1), f.jy + cc);
-        cp_async_4(gslot(b, 2), f.jz + cc);
-        cp_async_4(gslot(b, 3), f.n1 + cc);
-        cp_async_4(gslot(b, 4), f.n2 + cc);
-        cp_async_4(gslot(b, 5), f.n3 + cc);
+        const float* g = f.gs + gain_place(cc);
+        cp_async_4(gslot(b, 0), g + kJx);
+        cp_async_4(gslot(b, 1), g + kJy);
+        cp_async_4(gslot(b, 2), g + kJz);
+        cp_async_4(gslot(b, 3), g + kN1);
+        cp_async_4(gslot(b, 4), g + kN2);
+        cp_async_4(gslot(b, 5), g + kN3);
     };
 
     if (tid == 0) {

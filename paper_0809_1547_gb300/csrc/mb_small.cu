@@ -255,9 +255,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_step_small(const __grid_co
                 const uint8_t m = f.mat[c];
                 const float ie = f.inv_eps ? f.inv_eps[c] : f.lut_inv_eps[m & 0x7f];
                 const bool g = a.gain.on && (m & 0x80);
-                Ps[q] = make_float4(f.px[c], f.py[c], f.pz[c], g ? -ie : ie);
-                Js[q] = make_float4(f.jx[c], f.jy[c], f.jz[c], f.n3[c]);
-                Ns[q] = make_float2(f.n1[c], f.n2[c]);
+                const float* gs = f.gs + gain_place(c);
+                Ps[q] = make_float4(gs[kPx], gs[kPy], gs[kPz], g ? -ie : ie);
+                Js[q] = make_float4(gs[kJx], gs[kJy], gs[kJz], gs[kN3]);
+                Ns[q] = make_float2(gs[kN1], gs[kN2]);
             }
             items[q] = make_uint2((uint32_t)(i + 1) | (uint32_t)(j + 1) << 10 | (uint32_t)(k + 1) << 20, fl);
         }
@@ -518,15 +519,16 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_step_small(const __grid_co
             if (p4.w < 0.0f) {
                 const float4 j4 = Js[q];
                 const float2 nn = Ns[q];
-                f.px[c] = p4.x;
-                f.py[c] = p4.y;
-                f.pz[c] = p4.z;
-                f.jx[c] = j4.x;
-                f.jy[c] = j4.y;
-                f.jz[c] = j4.z;
-                f.n1[c] = nn.x;
-                f.n2[c] = nn.y;
-                f.n3[c] = j4.w;
+                float* gs = f.gs + gain_place(c);
+                gs[kPx] = p4.x;
+                gs[kPy] = p4.y;
+                gs[kPz] = p4.z;
+                gs[kJx] = j4.x;
+                gs[kJy] = j4.y;
+                gs[kJz] = j4.z;
+                gs[kN1] = nn.x;
+                gs[kN2] = nn.y;
+                gs[kN3] = j4.w;
             }
             if (m.fl & kInX) {
                 const uint32_t p = qx(gi, gj, gk);

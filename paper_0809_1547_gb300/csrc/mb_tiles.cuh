@@ -54,14 +54,15 @@ __device__ __forceinline__ void gain_block(const StepArgs& a, unsigned gidx, int
         ex[r] = __ldg(f.ex + c);
         ey[r] = __ldg(f.ey + c);
         ez[r] = __ldg(f.ez + c);
-        n1[r] = f.n1[c];
-        n2[r] = f.n2[c];
-        px[r] = f.px[c];
-        py[r] = f.py[c];
-        pz[r] = f.pz[c];
-        jx[r] = f.jx[c];
-        jy[r] = f.jy[c];
-        jz[r] = f.jz[c];
+        const float* g = f.gs + gain_place(c);
+        n1[r] = g[kN1];
+        n2[r] = g[kN2];
+        px[r] = g[kPx];
+        py[r] = g[kPy];
+        pz[r] = g[kPz];
+        jx[r] = g[kJx];
+        jy[r] = g[kJy];
+        jz[r] = g[kJz];
     }
 #pragma unroll
     for (int r = 0; r < PER; ++r) {
@@ -70,12 +71,13 @@ __device__ __forceinline__ void gain_block(const StepArgs& a, unsigned gidx, int
         const uint32_t num = a.glist.number ? __ldg(a.glist.number + base + (uint32_t)(r * T)) : c;
         lorentz_step(a.gain, num, n, ex[r], ey[r], ez[r], n1[r], n2[r], jx[r], jy[r], jz[r], px[r],
                      py[r], pz[r]);
-        f.jx[c] = jx[r];
-        f.jy[c] = jy[r];
-        f.jz[c] = jz[r];
-        f.px[c] = px[r];
-        f.py[c] = py[r];
-        f.pz[c] = pz[r];
+        float* g = f.gs + gain_place(c);
+        g[kJx] = jx[r];
+        g[kJy] = jy[r];
+        g[kJz] = jz[r];
+        g[kPx] = px[r];
+        g[kPy] = py[r];
+        g[kPz] = pz[r];
     }
 }
 
