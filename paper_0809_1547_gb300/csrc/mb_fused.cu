@@ -7,20 +7,30 @@
 // One thread streams, S - 1 planes ahead, each plane's E (with a one-cell
 // halo on every side), H^{n-1/2} (with its -x/-y halo) and material tile from
 // the source copy into an S-slot shared-memory ring (cp.async.bulk.tensor on
-// mbarriers).  Plane k then takes four steps:
+// mbarriers, the three components of E and of H in one copy each).  Plane k
+// then takes three steps:
 //   1. H^{n+1/2} of the tile's own cells (E of planes k and k+1), written to
 //      the destination copy and to a shared tile; threads of the first warps
 //      also compute H^{n+1/2} of the row j = y0-1 and the column i = x0-1,
 //      which the E update of the tile's edge cells needs (the neighbouring
 //      tiles compute the same values from the same inputs, bit for bit);
 //   2. for gain cells, J^{n+1/2} and P^{n+1} (E^n from the ring, P, J and the
-//      populations prefetched one plane ahead with cp.async), in place;
+//      populations prefetched with cp.async since the plane before), in place;
 //   3. after a block barrier, E^{n+1} from the shared H tile and the own H of
 //      plane k-1 (registers), the populations N^{n+1}, and in blocks that
 //      hold face cells of the flux box their outward Poynting terms (summed
 //      per warp and plane into shared partials, added to the FP64 face slots
-//      once per block);
-//   4. a barrier frees the ring slot for plane k + S.
+//      once per block).
+// Step 3 reads nothing of the ring (a cell's E^n and material stay in
+// registers), so that one barrier also frees the plane's slot, which the copy
+// of plane k + S then fills; and with two H tiles in turn it is the only
+// barrier of a plane: a warp may run a plane's step 3 and the next one's steps
+// 1 and 2 while others still compute step 3.  With a second barrier, a second
+// buffer of gain values and a copy per component 0.643 ms per 320^3 launch
+// (passive 0.423, 192^3 0.167), with one barrier and one buffer 0.638 (0.420,
+// 0.162), with one copy per three components as well 0.622 (0.383, 0.156): the
+// copies are issued by a single thread, whose warp the others wait for, and
+// the smaller ring lets a ninth block of 32 x 4 onto an SM.
 // The first plane of a block needs H^{n+1/2} of plane k0-1 at its own cells:
 // recomputed from the source copy (never written: the block below owns it).
 // Because no block writes what another reads, the launch needs no ordering
@@ -41,17 +51,17 @@ struct FusedLayout {
     static constexpr int kEX = BX + 8, kEY = BY + 2;   // E box from (x0-4, y0-1)
     static constexpr int kHX = BX + 4, kHY = BY + 1;   // H box from (x0-4, y0-1)
     static constexpr int kEW = kEX * kEY, kHW = kHX * kHY, kMW = BX * BY;
-    static constexpr int kEBytes = (kEW * 4 + 127) / 128 * 128;
-    static constexpr int kHBytes = (kHW * 4 + 127) / 128 * 128;
+    static constexpr int kEBytes = (3 * kEW * 4 + 127) / 128 * 128;
+    static constexpr int kHBytes = (3 * kHW * 4 + 127) / 128 * 128;
     static constexpr int kMBytes = (kMW + 127) / 128 * 128;
-    static constexpr int kStage = 3 * kEBytes + 3 * kHBytes + kMBytes;
+    static constexpr int kStage = kEBytes + kHBytes + kMBytes;
     static constexpr int kTxE = 3 * kEW * 4;                  // top stage: E only
     static constexpr int kTx = kTxE + 3 * kHW * 4 + kMW;
-    // H^{n+1/2} of the tile with its -x/-y halo: [3][BY+1][BX+1]
+    // H^{n+1/2} of the tile with its -x/-y halo: two of [3][BY+1][BX+1]
     static constexpr int kNX = BX + 1, kNW = (BX + 1) * (BY + 1);
-    static constexpr int kNBytes = (3 * kNW * 4 + 127) / 128 * 128;
-    // P, J, n1..n3 of gain cells, two planes (cp.async double buffer)
-    static constexpr int kGBytes = 2 * 9 * kMW * 4;
+    static constexpr int kNBytes = (6 * kNW * 4 + 127) / 128 * 128;
+    // P, J, n1..n3 of gain cells (each thread its own cell's)
+    static constexpr int kGBytes = 9 * kMW * 4;
     static constexpr int smem_bytes(int stages) {
         return stages * kStage + kGBytes + kNBytes + 64 + 128;
     }
@@ -113,7 +123,7 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
     __shared__ float wfl[6][NW];   // per-warp face-flux partials
     unsigned char* smem = align_smem(smem_raw);
     float* gbuf = reinterpret_cast<float*>(smem + S * Lay::kStage);
-    float* hn = reinterpret_cast<float*>(smem + S * Lay::kStage + Lay::kGBytes);
+    float* hn2 = reinterpret_cast<float*>(smem + S * Lay::kStage + Lay::kGBytes);
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + S * Lay::kStage + Lay::kGBytes + Lay::kNBytes);
     static_assert(BX % 8 == 0 && BY % 4 == 0, "x-edge tiles map warps onto 8 x 4 cells");
     const int tid = threadIdx.x + BX * threadIdx.y;
@@ -155,31 +165,26 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
         unsigned char* q = smem + s * Lay::kStage;
         const int k = k0 + p;
         mbar_arrive_expect_tx(&bar[s], p < planes ? Lay::kTx - (MATG ? Lay::kMW : 0) : Lay::kTxE);
-        tma_load_3d_hint(q + 0 * Lay::kEBytes, &maps.ex, x0 - 4, y0 - 1, k, &bar[s], keep_l2);
-        tma_load_3d_hint(q + 1 * Lay::kEBytes, &maps.ey, x0 - 4, y0 - 1, k, &bar[s], keep_l2);
-        tma_load_3d_hint(q + 2 * Lay::kEBytes, &maps.ez, x0 - 4, y0 - 1, k, &bar[s], keep_l2);
+        tma_load_4d_hint(q, &maps.e, x0 - 4, y0 - 1, k, 0, &bar[s], keep_l2);
         if (p < planes) {
-            unsigned char* h = q + 3 * Lay::kEBytes;
-            tma_load_3d(h + 0 * Lay::kHBytes, &maps.hx, x0 - 4, y0 - 1, k, &bar[s]);
-            tma_load_3d(h + 1 * Lay::kHBytes, &maps.hy, x0 - 4, y0 - 1, k, &bar[s]);
-            tma_load_3d(h + 2 * Lay::kHBytes, &maps.hz, x0 - 4, y0 - 1, k, &bar[s]);
-            if (!MATG) tma_load_3d(h + 3 * Lay::kHBytes, &maps.mat, x0, y0, k, &bar[s]);
+            tma_load_4d(q + Lay::kEBytes, &maps.h, x0 - 4, y0 - 1, k, 0, &bar[s]);
+            if (!MATG) tma_load_3d(q + Lay::kEBytes + Lay::kHBytes, &maps.mat, x0, y0, k, &bar[s]);
         }
     };
     auto mat_of = [&](int s) -> uint8_t {
-        return (smem + s * Lay::kStage + 3 * Lay::kEBytes + 3 * Lay::kHBytes)[tcell];
+        return (smem + s * Lay::kStage + Lay::kEBytes + Lay::kHBytes)[tcell];
     };
-    auto gslot = [&](int b, int q) -> float* { return gbuf + (b * 9 + q) * T + tid; };
-    auto prefetch_gain = [&](int b, const float* g) {
-        cp_async_4(gslot(b, 0), g + kPx);
-        cp_async_4(gslot(b, 1), g + kPy);
-        cp_async_4(gslot(b, 2), g + kPz);
-        cp_async_4(gslot(b, 3), g + kJx);
-        cp_async_4(gslot(b, 4), g + kJy);
-        cp_async_4(gslot(b, 5), g + kJz);
-        cp_async_4(gslot(b, 6), g + kN1);
-        cp_async_4(gslot(b, 7), g + kN2);
-        cp_async_4(gslot(b, 8), g + kN3);
+    auto gslot = [&](int q) -> float* { return gbuf + q * T + tid; };
+    auto prefetch_gain = [&](const float* g) {
+        cp_async_4(gslot(0), g + kPx);
+        cp_async_4(gslot(1), g + kPy);
+        cp_async_4(gslot(2), g + kPz);
+        cp_async_4(gslot(3), g + kJx);
+        cp_async_4(gslot(4), g + kJy);
+        cp_async_4(gslot(5), g + kJz);
+        cp_async_4(gslot(6), g + kN1);
+        cp_async_4(gslot(7), g + kN2);
+        cp_async_4(gslot(8), g + kN3);
     };
 
     if (tid == 0) {
@@ -237,37 +242,31 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
     const int own_e = (ty + 1) * Lay::kEX + tx + 4;
     const int own_h = (ty + 1) * Lay::kHX + tx + 4;
     const int own_n = (ty + 1) * Lay::kNX + tx + 1;
-    constexpr int EW = Lay::kEBytes / 4, HW = Lay::kHBytes / 4, NN = Lay::kNW;
+    constexpr int EW = Lay::kEW, HW = Lay::kHW, NN = Lay::kNW;
 
-    uint8_t m0 = 0, m1 = 0;   // MATG: the material of planes p and p + 1
+    uint8_t m0 = 0, m1 = 0;   // the material of planes p and p + 1
     if (MATG && valid) {
         m0 = __ldg(f.mat + c);
         if (planes > 1) m1 = __ldg(f.mat + c + nxy);
     }
     bool fail = !mbar_wait_bounded(&bar[0], 0, kWaitLimit);
-    bool pg = valid && gain_on && ((MATG ? m0 : mat_of(0)) & 0x80);
-    float* g0 = f.gs + gain_place(c);   // the cell's gain block, plane p
-    if (pg) prefetch_gain(0, g0);
+    if (!MATG) m0 = mat_of(0);
+    bool pg = valid && gain_on && (m0 & 0x80);
+    if (pg) prefetch_gain(f.gs + gain_place(c));
     cp_async_commit();
     // ring slots of planes p and p + 1, and the phase parity of plane p + 1
     int s = 0, s1 = 1 % S;
     uint32_t ph1 = (1 / S) & 1;
     for (int p = 0; p < planes; ++p) {
         const int k = k0 + p;
-        cp_async_wait_all();   // this plane's gain values (own thread's copies)
         fail |= !mbar_wait_bounded(&bar[s1], ph1, kWaitLimit);
         uint8_t m2 = 0;
         if (MATG && valid && p + 2 < planes) m2 = __ldg(f.mat + c + 2 * nxy);
-        bool ng = false;
-        float* g1 = f.gs + gain_place(c + nxy);   // (plane p + 1; used where ng)
-        if (p + 1 < planes) {
-            ng = valid && gain_on && ((MATG ? m1 : mat_of(s1)) & 0x80);
-            if (ng) prefetch_gain((p + 1) & 1, g1);
-        }
-        cp_async_commit();
+        if (!MATG) m1 = mat_of(s1);
+        const bool ng = p + 1 < planes && valid && gain_on && (m1 & 0x80);
         const float* E0 = reinterpret_cast<const float*>(smem + s * Lay::kStage);
         const float* E1 = reinterpret_cast<const float*>(smem + s1 * Lay::kStage);
-        const float* H0 = reinterpret_cast<const float*>(smem + s * Lay::kStage + 3 * Lay::kEBytes);
+        const float* H0 = reinterpret_cast<const float*>(smem + s * Lay::kStage + Lay::kEBytes);
         const bool zpml = plane_in_z_slab(a, k);
         const bool pml = w_pml || zpml, pml_h = w_pml_halo || zpml;
         const bool fk = plane_has_flux(a.flux, face, w_xy, k);
@@ -279,11 +278,13 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
         // what the ring holds.
         // 1. H^{n+1/2}: own cell, then the halo row / column
         float hx = 0.0f, hy = 0.0f, hz = 0.0f;
+        const float ex0 = E0[own_e], ey0 = E0[EW + own_e], ez0 = E0[2 * EW + own_e];
+        float* hn = hn2 + (p & 1) * 3 * NN;
         if (valid) {
             ENb e;
-            e.ex = E0[own_e];
-            e.ey = E0[EW + own_e];
-            e.ez = E0[2 * EW + own_e];
+            e.ex = ex0;
+            e.ey = ey0;
+            e.ez = ez0;
             e.ex_j1 = E0[own_e + Lay::kEX];
             e.ez_j1 = E0[2 * EW + own_e + Lay::kEX];
             e.ey_i1 = E0[EW + own_e + 1];
@@ -330,26 +331,35 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
         }
 
         // 2. J^{n+1/2}, P^{n+1} of a gain cell (time-n state only)
-        const int b = p & 1;
         float jx = 0.f, jy = 0.f, jz = 0.f, n1 = 0.f, n2 = 0.f, n3 = 0.f;
         if (pg) {
-            float px = *gslot(b, 0), py = *gslot(b, 1), pz = *gslot(b, 2);
-            jx = *gslot(b, 3);
-            jy = *gslot(b, 4);
-            jz = *gslot(b, 5);
-            n1 = *gslot(b, 6);
-            n2 = *gslot(b, 7);
-            n3 = *gslot(b, 8);
-            lorentz_step(a.gain, cell_number(a.g, i, j, k), n, E0[own_e], E0[EW + own_e], E0[2 * EW + own_e], n1, n2, jx,
+            cp_async_wait_all();   // own thread's copies
+            float px = *gslot(0), py = *gslot(1), pz = *gslot(2);
+            jx = *gslot(3);
+            jy = *gslot(4);
+            jz = *gslot(5);
+            n1 = *gslot(6);
+            n2 = *gslot(7);
+            n3 = *gslot(8);
+            lorentz_step(a.gain, cell_number(a.g, i, j, k), n, ex0, ey0, ez0, n1, n2, jx,
                          jy, jz, px, py, pz);
-            __stcs(g0 + kPx, px);
-            __stcs(g0 + kPy, py);
-            __stcs(g0 + kPz, pz);
-            __stcs(g0 + kJx, jx);
-            __stcs(g0 + kJy, jy);
-            __stcs(g0 + kJz, jz);
+            float* g = f.gs + gain_place(c);
+            __stcs(g + kPx, px);
+            __stcs(g + kPy, py);
+            __stcs(g + kPz, pz);
+            __stcs(g + kJx, jx);
+            __stcs(g + kJy, jy);
+            __stcs(g + kJz, jz);
         }
-        __syncthreads();   // the H tile is complete
+        // the plane's H tile is complete, its ring slot free
+        block_fail = __syncthreads_or(fail);
+        if (block_fail) break;   // issue nothing more; drained below
+        if (p + S < total) {
+            if (tid == T - 32) issue(s, p + S);   // (not of the warps with the halo cells)
+            issued = p + S + 1;
+        }
+        if (ng) prefetch_gain(f.gs + gain_place(c + nxy));
+        cp_async_commit();
 
         // 3. E^{n+1}, N^{n+1}, face flux
         float fl[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -364,8 +374,7 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
             h.hz_j = hn[2 * NN + own_n - Lay::kNX];
             h.hx_k = hx_km1;
             h.hy_k = hy_km1;
-            const uint8_t m = MATG ? m0 : mat_of(s);
-            const float ex0 = E0[own_e], ey0 = E0[EW + own_e], ez0 = E0[2 * EW + own_e];
+            const uint8_t m = m0;
             float ex1, ey1, ez1;
             if (gen) {
                 e_compute_to<true, true>(a, i, j, k, c, h, m, ex0, ey0, ez0, pg, jx, jy, jz, n1, n2, n3, n, fl,
@@ -381,9 +390,10 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
             __stcs(d.ey + c, ey1);
             __stcs(d.ez + c, ez1);
             if (pg) {
-                __stcs(g0 + kN1, n1);
-                __stcs(g0 + kN2, n2);
-                __stcs(g0 + kN3, n3);
+                float* g = f.gs + gain_place(c);
+                __stcs(g + kN1, n1);
+                __stcs(g + kN2, n2);
+                __stcs(g + kN3, n3);
             }
             hx_km1 = hx;
             hy_km1 = hy;
@@ -402,16 +412,7 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
                 }
             }
         }
-        // ring slot s and the H tile are free again; the barrier also ORs the
-        // threads' wait verdicts, so every thread sees the same block_fail
-        block_fail = __syncthreads_or(fail);
-        if (block_fail) break;   // issue nothing more; drained below
-        if (p + S < total) {
-            if (tid == 0) issue(s, p + S);
-            issued = p + S + 1;
-        }
         pg = ng;
-        g0 = g1;
         m0 = m1;
         m1 = m2;
         c += nxy;
@@ -467,13 +468,7 @@ bool fused_tile_supported(int bx, int by) {
 bool encode_fused(const StepArgs& a, int bx, int by, TmaFusedMaps* out) {
     if (!fused_supported(a) || !fused_tile_supported(bx, by)) return false;
     const DevFields& f = a.f;
-    const CUtensorMapDataType F32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
-    return encode_box(&out->ex, F32, f.ex, 4, a.g, bx + 8, by + 2) &&
-           encode_box(&out->ey, F32, f.ey, 4, a.g, bx + 8, by + 2) &&
-           encode_box(&out->ez, F32, f.ez, 4, a.g, bx + 8, by + 2) &&
-           encode_box(&out->hx, F32, f.hx, 4, a.g, bx + 4, by + 1) &&
-           encode_box(&out->hy, F32, f.hy, 4, a.g, bx + 4, by + 1) &&
-           encode_box(&out->hz, F32, f.hz, 4, a.g, bx + 4, by + 1) &&
+    return encode_boxes(&out->e, f.ex, a.g, bx + 8, by + 2) && encode_boxes(&out->h, f.hx, a.g, bx + 4, by + 1) &&
            (a.g.px % 16 != 0 || encode_box(&out->mat, CU_TENSOR_MAP_DATA_TYPE_UINT8, f.mat, 1, a.g, bx, by));
 }
 

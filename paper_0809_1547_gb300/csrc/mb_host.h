@@ -160,6 +160,7 @@ bool encode_tma(const StepArgs& a, int bx, int by, TmaMaps* out);
 // (bw, bh, 1) box, zero fill beyond the array.
 bool encode_box(CUtensorMap* m, CUtensorMapDataType dt, const void* base, int esize,
                 const DevGrid& g, int bw, int bh);
+bool encode_boxes(CUtensorMap* m, const float* base, const DevGrid& g, int bw, int bh);
 
 // Single-pass step (H half-step, Lorentz update, E / population update in
 // one launch) reading one copy of E / H / CPML memories and writing the
@@ -168,7 +169,7 @@ bool encode_box(CUtensorMap* m, CUtensorMapDataType dt, const void* base, int es
 // (x0-4, y0-1)), H with its -x/-y halo ((bx+4) x (by+1) from (x0-4, y0-1))
 // and the material byte (bx x by).
 struct TmaFusedMaps {
-    CUtensorMap ex, ey, ez, hx, hy, hz, mat;
+    CUtensorMap e, h, mat;   // (three components at once; the material byte)
 };
 bool fused_tile_supported(int bx, int by);
 bool fused_supported(const StepArgs& a);
