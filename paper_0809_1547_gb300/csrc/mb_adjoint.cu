@@ -305,9 +305,21 @@ __device__ __forceinline__ WCoef w_plain(float S, float ux, float uy, float uz) 
     return w;
 }
 
+// The thread's cell in a block of 32 x 8.  In blocks that hold x-CPML columns
+// (or neighbours of them) a warp covers 8 columns x 4 rows, so that the slab's
+// columns fill whole warps and the others take the coefficients without the
+// memories; elsewhere a warp covers one row.  True: 8 x 4.
+__device__ __forceinline__ bool adj_cell(const AdjArgs& a, int& i, int& j) {
+    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 8;
+    const bool edge = a.L > 0 && (x0 <= a.L || x0 + 32 >= a.g.nx - a.L);
+    i = x0 + (edge ? 8 * (threadIdx.y & 3) + (threadIdx.x & 7) : threadIdx.x);
+    j = y0 + (edge ? 4 * (threadIdx.y >> 2) + (threadIdx.x >> 3) : threadIdx.y);
+    return edge;
+}
+
 __global__ void __launch_bounds__(256) k_adj_h(AdjArgs a) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y * blockDim.y + threadIdx.y;
+    int i, j;
+    adj_cell(a, i, j);
     const int k = blockIdx.z;
     const int nx = a.g.nx, ny = a.g.ny, nz = a.g.nz, L = a.L;
     const bool valid = i < nx && j < ny;
@@ -492,8 +504,8 @@ __global__ void __launch_bounds__(256) k_adj_e(AdjArgs a) {
 // registers (6 blocks per SM, a few spilled bytes): the launch is latency
 // bound, and the added warps gain more than the spills cost.
 __global__ void __launch_bounds__(256, 6) k_adj_e_point(AdjArgs a) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y * blockDim.y + threadIdx.y;
+    int i, j;
+    const bool edge = adj_cell(a, i, j);
     const int k = blockIdx.z;
     const bool valid = i < a.g.nx && j < a.g.ny;
     const bool pml = __any_sync(0xffffffffu, valid && near_slab_lo(a, i, j, k));
@@ -501,6 +513,15 @@ __global__ void __launch_bounds__(256, 6) k_adj_e_point(AdjArgs a) {
     if (valid) adj_e_gather(a, i, j, k, cell_place(a.g, i, j, k), pml, lx, ly, lz);
     float obj, gw;
     adj_point_cell(a, i, j, k, valid, lx, ly, lz, obj, gw);
+    if (edge) {   // the sums by rows all the same
+        __shared__ float so[256], sg[256];
+        const int at = (i - (int)blockIdx.x * 32) + 32 * (j - (int)blockIdx.y * 8), me = threadIdx.x + 32 * threadIdx.y;
+        so[at] = obj;
+        sg[at] = gw;
+        __syncthreads();
+        obj = so[me];
+        gw = sg[me];
+    }
     const unsigned slot = block_slot();
     warp_acc(a.acc, obj, slot);
     warp_acc(a.acc + kAccSlots, gw, slot);
