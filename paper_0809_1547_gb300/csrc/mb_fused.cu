@@ -107,12 +107,51 @@ __device__ __forceinline__ void e_plain(float S, const HNb& h, float ie, float e
     ez1 = fmaf(ie, fmaf(S, cz, -jz), ez0);
 }
 
+__device__ __forceinline__ void prefetch_l2(const float* p) {
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
+// One warp brings the lines of the CPML memories that a block's cells of plane
+// k read (all four arrays of each slab axis the tile or the plane touches)
+// into L2; lane = 8 f + row.  The slabs are latency: 192^3 without gain takes
+// 76 us a launch without a CPML and took 117 with 21 % more instructions, each
+// cell having asked for its own values into L1 half a plane ahead (from HBM
+// that is too late, and the requests were a fifth of the slabs' instructions).
+// Two planes ahead and a line at a time: 113 us, 144^3 69.1 -> 65.3 (with gain
+// 83.3 -> 79.7), 320^3 383 -> 375 (622 -> 623); no request at all: 119, 70.1, 394.
+template <int BX, int BY>
+__device__ __forceinline__ void prefetch_psi_tile(const StepArgs& a, int x0, int y0, int k) {
+    const int nx = a.g.nx, ny = a.g.ny, nz = a.g.nz, L = a.pml.L, L2 = 2 * L;
+    const int lane = threadIdx.x & 31;
+    const uint32_t f = lane >> 3;
+    const int j = y0 + (lane & 7);
+    if ((lane & 7) >= BY || j >= ny) return;
+    const int xe = min(x0 + BX, nx) - 1;
+    if (plane_in_z_slab(a, k)) {
+        const uint32_t s = (k < a.pml.zlo) ? k : k - a.pml.zhi + a.pml.zs;
+        const float* q = a.pml.psz + ((size_t)(f * a.pml.zn + s) * ny + j) * nx;
+        for (int x = x0; x < xe; x += 32) prefetch_l2(q + x);
+        prefetch_l2(q + xe);
+    }
+    if (j < L || j >= ny - L) {
+        const float* q = a.pml.psy + ((size_t)(f * nz + k) * L2 + slab_index(j, ny, L)) * nx;
+        for (int x = x0; x < xe; x += 32) prefetch_l2(q + x);
+        prefetch_l2(q + xe);
+    }
+    const float* q = a.pml.psx + ((size_t)(f * nz + k) * ny + j) * L2;
+    if (x0 < L) prefetch_l2(q);
+    if (xe >= nx - L) prefetch_l2(q + L);
+}
+
 // MATG: the material bytes come by plain loads two planes ahead, kept in
 // registers, instead of with the tensor copies (whose byte rows must be
 // multiples of 16: n_x = 320, 448, ...; every other n_x has rows of a
 // multiple of 4 cells only).
+// 32 x 4: 56 registers, so that nine blocks fit an SM as their shared memory
+// does (64 registers and eight blocks: 448^3 1.69 ms, 320^3 0.627; nine: 1.68
+// and 0.623; the larger tiles lose 2 % under a bound).
 template <int BX, int BY, int S, bool MATG>
-__global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
+__global__ void __launch_bounds__(BX * BY, BX * BY == 128 ? 9 : 0) k_step_fused(StepArgs a, DevPing d,
                                                         const __grid_constant__ TmaFusedMaps maps,
                                                         int kz) {
     using Lay = FusedLayout<BX, BY>;
@@ -195,6 +234,12 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
     __syncthreads();
     if (tid == 0)
         for (int s = 0; s < S && s < total; ++s) issue(s, s);
+    // the CPML memories of a block that holds slab cells come into L2 two
+    // planes ahead, asked for by a warp without halo cells
+    const bool pf = a.pml.L > 0 && (tid >> 5) == 2;
+    if (pf)
+        for (int q = 0; q < 2 && q < planes; ++q)
+            if (pml_xy || plane_in_z_slab(a, k0 + q)) prefetch_psi_tile<BX, BY>(a, x0, y0, k0 + q);
     int issued = min(S, total);   // planes issued into the ring so far
     bool block_fail = false;
 
@@ -299,8 +344,6 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
             __stcs(d.hx + c, hx);
             __stcs(d.hy + c, hy);
             __stcs(d.hz + c, hz);
-            // the CPML memories the E update reads after the barrier
-            if (pml) prefetch_psi(a, i, j, k, 0);
         }
         hn[own_n] = hx;
         hn[NN + own_n] = hy;
@@ -358,6 +401,7 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
             if (tid == T - 32) issue(s, p + S);   // (not of the warps with the halo cells)
             issued = p + S + 1;
         }
+        if (pf && p + 2 < planes && (pml_xy || plane_in_z_slab(a, k + 2))) prefetch_psi_tile<BX, BY>(a, x0, y0, k + 2);
         if (ng) prefetch_gain(f.gs + gain_place(c + nxy));
         cp_async_commit();
 
@@ -397,8 +441,6 @@ __global__ void __launch_bounds__(BX * BY) k_step_fused(StepArgs a, DevPing d,
             }
             hx_km1 = hx;
             hy_km1 = hy;
-            // the CPML memories the next plane's H update reads
-            if (p + 1 < planes && (w_pml || plane_in_z_slab(a, k + 1))) prefetch_psi(a, i, j, k + 1, 2);
         }
         if (fk) {
             // this plane's flux terms: warp sums, added to the warp's partials
