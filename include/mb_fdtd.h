@@ -336,6 +336,11 @@ int mb_launch_stats(mb_ctx* ctx, int* per_step, int64_t* total);
  * switches the injection off.  Process-wide. */
 void mb_debug_fail_alloc(int n);
 
+/* Test hook: the device memory of these allocations starts filled with this
+ * byte (0..255; 0xff: NaNs), as memory used before may be; -1: as it comes.
+ * Process-wide. */
+void mb_debug_fill_alloc(int byte);
+
 /* Device bytes the context holds. */
 int mb_device_bytes(mb_ctx* ctx, size_t* bytes);
 

@@ -99,6 +99,7 @@ _SIGS = [
     ("mb_set_tuning", C.c_int, [_P, C.POINTER(C.c_int), C.POINTER(C.c_int)]),
     ("mb_flux_async", C.c_int, [_P, _P]),
     ("mb_debug_fail_alloc", None, [C.c_int]),
+    ("mb_debug_fill_alloc", None, [C.c_int]),
     ("mb_get_single_pass", C.c_int, [_P, C.POINTER(C.c_int)]),
     ("mb_set_single_pass", C.c_int, [_P, C.POINTER(C.c_int)]),
     ("mb_launch_stats", C.c_int, [_P, C.POINTER(C.c_int), C.POINTER(C.c_int64)]),
@@ -300,6 +301,11 @@ def mb_flux_async(h, out_ptr: int):
 def mb_debug_fail_alloc(n: int):
     """Test hook: make the n-th device allocation from now on fail (n < 0: off)."""
     load_library().mb_debug_fail_alloc(int(n))
+
+
+def mb_debug_fill_alloc(byte: int):
+    """Test hook: device allocations start filled with this byte (< 0: off)."""
+    load_library().mb_debug_fill_alloc(int(byte))
 
 
 def mb_host_tables(grid, dx, dt, params: mb_params | None = None, N_a=0.0, pump=0.0):

@@ -24,15 +24,20 @@ using mb::kQe;
 namespace mbi {
 
 thread_local std::string g_err;
-// allocations left before an injected failure (-1: none)
-std::atomic<int> g_fail_alloc_after{-1};
+// allocations left before an injected failure (-1: none), and the byte new
+// allocations are filled with (-1: left as they come)
+std::atomic<int> g_fail_alloc_after{-1}, g_fill_alloc{-1};
 
-bool inject_alloc_failure() {
+cudaError_t device_malloc(void** p, size_t bytes) {
     int v = g_fail_alloc_after.load();
-    while (v >= 0) {
-        if (g_fail_alloc_after.compare_exchange_weak(v, v - 1)) return v == 0;
+    while (v >= 0 && !g_fail_alloc_after.compare_exchange_weak(v, v - 1)) {}
+    cudaError_t e = v == 0 ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+    const int fill = g_fill_alloc.load();
+    if (e == cudaSuccess && fill >= 0) {
+        cudaMemset(*p, fill, bytes);
+        e = cudaDeviceSynchronize();
     }
-    return false;
+    return e;
 }
 
 int fail(mb_ctx* ctx, int code, const std::string& msg) {
@@ -756,7 +761,7 @@ static int create_ctx(mb_ctx** out, const int grid[3], int gnz, int kz0, int own
     }
     auto alloc = [&](void** ptr, size_t bytes) -> int {
         if (bytes == 0) { *ptr = nullptr; return MB_OK; }
-        cudaError_t ae = inject_alloc_failure() ? cudaErrorMemoryAllocation : cudaMalloc(ptr, bytes);
+        cudaError_t ae = device_malloc(ptr, bytes);
         if (ae != cudaSuccess) {
             cudaGetLastError();
             return fail(nullptr, MB_ERR_OOM, "cudaMalloc of " + std::to_string(bytes) + " bytes failed");
@@ -1621,6 +1626,8 @@ int mb_load_state(mb_ctx* c, const void* host_blob, size_t bytes) {
 }
 
 void mb_debug_fail_alloc(int n) { g_fail_alloc_after.store(n < 0 ? -1 : n); }
+
+void mb_debug_fill_alloc(int byte) { g_fill_alloc.store(byte < 0 ? -1 : byte & 0xff); }
 
 int mb_device_bytes(mb_ctx* c, size_t* bytes) {
     if (int rc = check_ctx(c)) return rc;

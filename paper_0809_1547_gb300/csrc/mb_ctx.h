@@ -25,9 +25,8 @@ struct NvtxRange {
     NvtxRange& operator=(const NvtxRange&) = delete;
 };
 
-// Allocation-failure injection for tests (mb_debug_fail_alloc): true when
-// the next device allocation of a context should fail.
-bool inject_alloc_failure();
+// cudaMalloc under the test hooks (mb_debug_fail_alloc, mb_debug_fill_alloc).
+cudaError_t device_malloc(void** p, size_t bytes);
 
 // Records msg as the context's (and the thread's) last error; returns code.
 int fail(mb_ctx* ctx, int code, const std::string& msg);

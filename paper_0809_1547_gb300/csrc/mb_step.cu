@@ -28,14 +28,15 @@ mb::DevPing ping_of(const mb_ctx* c, const mb::StepArgs& a, int q) {
                        mb::PsiOut{a.pml.psx, a.pml.psy, a.pml.psz}, c->d_ctr + 2 + q};
 }
 
-// Allocates the second copy on first use.
+// Allocates the second copy on first use.  Steps write its cells only: the
+// places past n_x of padded rows, which the energy sums run over, are zeroed here.
 int ensure_second_copy(mb_ctx* c) {
     if (c->d_fields2) return MB_OK;
     const size_t fb = sizeof(float) * 6 * (size_t)c->pcell;
-    cudaError_t e = inject_alloc_failure() ? cudaErrorMemoryAllocation
-                                           : cudaMalloc((void**)&c->d_fields2, fb);
+    cudaError_t e = device_malloc((void**)&c->d_fields2, fb);
     for (int w = 0; w < 3 && e == cudaSuccess; ++w)
-        if (c->psi_elems[w]) e = cudaMalloc((void**)&c->d_psi2[w], sizeof(float) * c->psi_elems[w]);
+        if (c->psi_elems[w]) e = device_malloc((void**)&c->d_psi2[w], sizeof(float) * c->psi_elems[w]);
+    if (e == cudaSuccess && c->px != c->nx) e = cudaMemsetAsync(c->d_fields2, 0, fb, c->stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
         cudaFree(c->d_fields2);
@@ -101,8 +102,8 @@ bool small_ready(mb_ctx* c) {
     }
     const mb::SmallTile& t = c->small;
     const size_t xb = sizeof(float4) * 2 * (size_t)(t.bx * t.by * t.bz) * (t.tx * t.ty * t.tz);
-    if (cudaMalloc((void**)&c->d_small_x, xb) != cudaSuccess ||
-        cudaMalloc((void**)&c->d_small, sizeof(unsigned) * kSmallWords) != cudaSuccess) {
+    if (device_malloc((void**)&c->d_small_x, xb) != cudaSuccess ||
+        device_malloc((void**)&c->d_small, sizeof(unsigned) * kSmallWords) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(c->d_small_x);
         c->d_small_x = nullptr;
