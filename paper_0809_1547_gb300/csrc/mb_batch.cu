@@ -24,6 +24,9 @@ struct mb_batch {
     unsigned long long* d_tick = nullptr;
     int* d_err = nullptr;
     long long* d_ctr = nullptr;
+    // the copy of its state that each instance's device arguments point at
+    // (its own single-pass or small-grid steps change copies)
+    std::vector<const float*> at;
     int n1 = 0, n2 = 0;
     dim3 block{32, 4, 1};
     int kz = 16;
@@ -100,6 +103,7 @@ int rebuild(mb_batch* b) {
     std::vector<mb::DevPointProbes> probes;
     std::vector<int> tiles;
     std::vector<int4> items1, items2;
+    b->at.clear();
     const int threads = (int)(b->block.x * b->block.y);
     const int gq = threads * mb::kBatchGainPerThread;
     for (int q = 0; q < B; ++q) {
@@ -108,6 +112,7 @@ int rebuild(mb_batch* b) {
         if (c->face.on || !c->planes.empty())
             return bfail(b, MB_ERR_STATE, "face and plane probes are not advanced inside a batch");
         args.push_back(c->args);
+        b->at.push_back(c->args.f.ex);
         probes.push_back({(int)c->probes.size(), c->probe_nfreq, c->d_probe_cell, c->d_probe_omega,
                           c->d_probe_acc});
         const int gx = (c->nx + b->block.x - 1) / b->block.x;
@@ -294,6 +299,8 @@ int mb_batch_step(mb_batch* b, int n) {
     if (!b || n < 0) return bfail(b, MB_ERR_ARG, "bad batch step arguments");
     if (n == 0) return MB_OK;
     if (int rc = check_lockstep(b)) return rc;
+    if (b->mode == MB_BATCH_PERSISTENT && !b->dirty)
+        for (size_t q = 0; q < b->inst.size(); ++q) b->dirty = b->dirty || b->at[q] != b->inst[q]->args.f.ex;
     if (b->dirty)
         if (int rc = rebuild(b)) return rc;
     if (b->mode == MB_BATCH_CONCURRENT) {
