@@ -543,7 +543,7 @@ int mb_selftest_bounded_waits(int which, int limit, int* gave_up);
  * for each eigenvalue E[q] > 1 (bound states exist above threshold), on
  * n_grid points tau_i = -L + i h, i = 1..n_grid, h = 2L/(n_grid + 1),
  * L = sqrt(E) + 8, phi(+-L) = 0, second-order differences, solved in FP64 on
- * the GPU by Newton's method (one thread per eigenvalue).  Outputs (host
+ * the GPU by Newton's method (a thread block per eigenvalue).  Outputs (host
  * arrays of nE doubles): w_phi[q], the standard deviation of |phi~|^2 in the
  * frequency Omega / 2 pi, and p_phi[q] = |phi~(0)|^2 / (4 pi^2), with phi~
  * the Fourier transform of phi — the normalised spectral waist and peak of

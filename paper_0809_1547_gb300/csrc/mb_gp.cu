@@ -8,7 +8,7 @@
 // in FP64.  Newton starts from the larger of the Thomas-Fermi profile
 // sqrt(max(E - tau^2, 0)) and the first-order solution near threshold
 // 2^{1/4} sqrt(E - 1) exp(-tau^2 / 2) and stops when the residual is below
-// 1e-12 max(1, E) or stagnates at rounding level; a result whose
+// 1e-13 max(1, E) or stagnates at rounding level; a result whose
 // residual stays above 1e-9 max(1, E), or that collapses towards the trivial
 // solution phi = 0, is reported as not converged.
 #include "mb_host.h"
@@ -64,11 +64,19 @@ __device__ __forceinline__ unsigned long long abs_bits(double x) {
 // a tridiagonal system of one row per thread, solved by parallel cyclic
 // reduction; back-substitution gives the rest.
 //
+// The residual takes phi'' from differences of neighbours, which are exact
+// (their ratio is below 2 where phi matters), so that what is left of its
+// rounding is of the size of phi'' and not of phi / h^2: with the sum of the
+// neighbours against 2 phi the features at n = 2047 were off by up to 2e-11
+// (p_phi; the tridiagonal solve in order of the points 1e-13), with the
+// differences by 2e-14 (against extended precision, 1.05 <= E <= 60).
+//
 // The serial form (one thread per eigenvalue walking its n points through
 // global memory, three dependent passes and two divisions per point and
 // iteration) took 35 ms for 200 eigenvalues at n = 2047 (8 warps busy on the
-// whole GPU); this takes 0.5 ms, 0.36 ms for one eigenvalue.  This form is bound by the FP64 pipe (2 operations per cycle
-// and SM here): about 27 FP64 operations per point and iteration plus the
+// whole GPU); this takes 0.55 ms, 0.32 ms for one eigenvalue.  This form is
+// bound by the FP64 pipe (2 operations per cycle and SM here): about 29 FP64
+// operations per point and iteration plus the
 // cyclic reduction's ~170 per thread.  128 threads put one warp on each of
 // an SM's four schedulers, which the pipe's rate already fills: 64 threads took
 // 0.45 ms for one eigenvalue and 1.6 against 1.0 ms for 64 at n = 8191, 256
@@ -93,7 +101,7 @@ __global__ void __launch_bounds__(kGpThreads) k_gp_solve(const double* Es, int n
     const double ih2 = 1.0 / (h * h);
     const double off = -ih2;
     const double amp = pow(2.0, 0.25) * sqrt(E - 1.0);
-    const double d0 = 2.0 * ih2 - E;
+    const double d0 = 2.0 * ih2;
     const int i0 = t * m;
     const int mine = min(m, max(0, n - i0));   // points of the grid among the thread's m
     for (int i = 0; i < m; ++i) {
@@ -104,7 +112,7 @@ __global__ void __launch_bounds__(kGpThreads) k_gp_solve(const double* Es, int n
     // phi of the point before the thread's first and after its last
     auto left = [&]() { return t > 0 ? phi[(size_t)(m - 1) * T - 1] : 0.0; };
     auto right = [&]() { return t < T - 1 ? phi[1] : 0.0; };
-    const double tol = 1e-12 * fmax(1.0, E), accept = 1e-9 * fmax(1.0, E);
+    const double tol = 1e-13 * fmax(1.0, E), accept = 1e-9 * fmax(1.0, E);
     double rprev = 0.0;
     int ok = 0;
     for (int it = 0;; ++it) {
@@ -112,18 +120,19 @@ __global__ void __launch_bounds__(kGpThreads) k_gp_solve(const double* Es, int n
         __syncthreads();
         unsigned long long rm = 0;
         {
-            double l = left(), c = phi[0];
+            double c = phi[0], dl = c - left();
             const double after = right();
             for (int i = 0; i < mine; ++i) {
                 const double r = i + 1 < m ? phi[(size_t)(i + 1) * T] : after;
                 const double tau = fma(h, (double)(i0 + i + 1), -L);
                 const double p2 = c * c;
-                const double g = fma(tau, tau, d0) + p2;
-                const double f = fma(c, g, off * (l + r));
+                const double g = fma(tau, tau, -E) + p2;
+                const double dr = r - c;
+                const double f = fma(c, g, off * (dr - dl));
                 ff[(size_t)i * T] = f;
-                bb[(size_t)i * T] = fma(2.0, p2, g);
+                bb[(size_t)i * T] = fma(2.0, p2, g) + d0;
                 rm = max(rm, abs_bits(f));
-                l = c;
+                dl = dr;
                 c = r;
             }
         }
@@ -234,13 +243,14 @@ __global__ void __launch_bounds__(kGpThreads) k_gp_solve(const double* Es, int n
             rprev = 0.0;
             __syncthreads();
             unsigned long long r2 = 0;
-            double l = left(), c = phi[0];
+            double c = phi[0], dl = c - left();
             const double after = right();
             for (int i = 0; i < mine; ++i) {
                 const double r = i + 1 < m ? phi[(size_t)(i + 1) * T] : after;
                 const double tau = fma(h, (double)(i0 + i + 1), -L);
-                r2 = max(r2, abs_bits(fma(c, fma(tau, tau, d0) + c * c, off * (l + r))));
-                l = c;
+                const double dr = r - c;
+                r2 = max(r2, abs_bits(fma(c, fma(tau, tau, -E) + c * c, off * (dr - dl))));
+                dl = dr;
                 c = r;
             }
             ok = __longlong_as_double((long long)block_max(r2, redu)) < accept;
