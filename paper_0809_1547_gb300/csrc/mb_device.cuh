@@ -313,34 +313,42 @@ __device__ __forceinline__ HNb load_h_nbrs(const StepArgs& a, int i, int j, int 
     return h;
 }
 
-// Sum of non-negative terms in FP32 as an unevaluated pair, for the energy
-// sums: a term w x (exact as product and error) or x is added with TwoSum
-// (Knuth), so the pair carries about 48 bits through the few hundred terms of
-// a thread before it goes over to FP64.  In FP64 throughout the sum was bound
-// by that pipe (six operations per cell at 2 per cycle and SM: 41 us for
-// 160^3 cells, 0.34 ms for 320^3, three times the reads' time).  Terms whose
-// product or error leaves FP32's normal range are added in FP64.
-struct PairSum {
-    float h = 0.0f, l = 0.0f;
+// x added to h + l + m: TwoSum (Knuth) into h, its error into l the same way,
+// and that one's error into m, which then carries bits 72 places below h's
+// first.  FP32 operations where an FP64 addition would wait for that pipe.
+__device__ __forceinline__ void add_expansion(float x, float& h, float& l, float& m) {
+    float t = h + x, b = t - h;
+    const float e = (h - (t - b)) + (x - b);
+    h = t;
+    t = l + e;
+    b = t - l;
+    m += (l - (t - b)) + (e - b);
+    l = t;
+}
+
+// Sum of non-negative terms in FP32 as an unevaluated sum of three, for the
+// energy sums: the terms w x (as product and its exact error) and x go in
+// without loss of what an FP64 sum would keep, and it goes over to FP64 once
+// per thread.  In FP64 throughout the sum was bound by that pipe (six
+// operations per cell at 2 per cycle and SM: 41 us for 160^3 cells, 0.34 ms
+// for 320^3, three times the reads' time).  Terms whose product or error
+// leaves FP32's normal range, or whose sum might, are added in FP64.
+struct EnergySum {
+    float h = 0.0f, l = 0.0f, m = 0.0f;
     double big = 0.0;
-    __device__ __forceinline__ void add(float x) {
-        const float t = h + x, b = t - h;
-        l += (h - (t - b)) + (x - b);
-        h = t;
-    }
     // w |E|^2 + |H|^2 of a cell
     __device__ __forceinline__ void cell(float w, float e2, float h2) {
         const float lo = fminf(e2 > 0.0f ? e2 : 1.0f, h2 > 0.0f ? h2 : 1.0f);
-        if (lo < 1e-27f || !(fmaxf(e2, h2) < 1e33f) || !(w < 1e4f)) {
+        if (lo < 1e-27f || !(fmaxf(e2, h2) < 1e29f) || !(w >= 1e-3f && w < 1e4f)) {
             big += (double)w * (double)e2 + (double)h2;
         } else {
             const float p = w * e2;
-            l += fmaf(w, e2, -p);
-            add(p);
-            add(h2);
+            add_expansion(p, h, l, m);
+            add_expansion(h2, h, l, m);
+            add_expansion(fmaf(w, e2, -p), h, l, m);
         }
     }
-    __device__ __forceinline__ double value() const { return big + ((double)h + (double)l); }
+    __device__ __forceinline__ double value() const { return big + ((double)h + ((double)l + (double)m)); }
 };
 
 // ------------------------------------------------------------- H half-step

@@ -134,7 +134,7 @@ template <bool VEC>
 __global__ void __launch_bounds__(256) k_energy_partial(DevFields f, int64_t ncell,
                                                         const float* lut_eps, double* partial,
                                                         int* nonfinite) {
-    PairSum acc;
+    EnergySum acc;
     double dense = 0.0;   // a dense map holds 1/eps_r: its cells divide in FP64
     bool bad = false;
     auto one = [&](float ex, float ey, float ez, float hx, float hy, float hz, uint8_t m, int64_t c) {

@@ -68,7 +68,7 @@ bool current_context_id(unsigned long long* id) {
     return get_id(ctx, id) == CUDA_SUCCESS;
 }
 
-// Pass 1: block b sums w |E|^2 + |H|^2 over cells [b C, (b+1) C) (PairSum per
+// Pass 1: block b sums w |E|^2 + |H|^2 over cells [b C, (b+1) C) (EnergySum per
 // thread, FP64 across threads).
 __global__ void __launch_bounds__(kNoAllocThreads)
 k_energy_partial_static(const float* ex, const float* ey, const float* ez, const float* hx,
@@ -76,7 +76,7 @@ k_energy_partial_static(const float* ex, const float* ey, const float* ez, const
                         NoAllocScratch* scratch) {
     const int64_t begin = blockIdx.x * kNoAllocCellsPerBlock;
     const int64_t end = begin + kNoAllocCellsPerBlock < ncell ? begin + kNoAllocCellsPerBlock : ncell;
-    mb::PairSum sum;
+    mb::EnergySum sum;
     bool bad = false;
     for (int64_t c = begin + threadIdx.x; c < end; c += kNoAllocThreads) {
         const float e2 = ex[c] * ex[c] + ey[c] * ey[c] + ez[c] * ez[c];
