@@ -130,7 +130,7 @@ __device__ void small_probe(const SmallArgs& A, int p, unsigned base, long long 
 __global__ void __launch_bounds__(kSmallThreads, 1) k_step_small(const __grid_constant__ SmallArgs A) {
     extern __shared__ float4 sm[];
     __shared__ int fail_s;
-    __shared__ float2 flux_s[6][kSmallThreads / 32];   // per-warp face-flux sums (value, error)
+    __shared__ float3 flux_s[6][kSmallThreads / 32];   // per-warp face-flux sums (add_expansion)
     __shared__ uint32_t pcell[kSmallMaxProbes];
     const StepArgs& a = A.a;
     const DevFields& f = a.f;
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_step_small(const __grid_co
     const unsigned base = *A.base;
     const int nblk = A.t.bx * A.t.by * A.t.bz;
     if (tid == 0) fail_s = 0;
-    for (int q = tid; q < 6 * (kSmallThreads / 32); q += T) (&flux_s[0][0])[q] = make_float2(0.f, 0.f);
+    for (int q = tid; q < 6 * (kSmallThreads / 32); q += T) (&flux_s[0][0])[q] = make_float3(0.f, 0.f, 0.f);
     if (tid < A.pp.count) pcell[tid] = (uint32_t)A.pp.cell[tid];
     __syncthreads();
     if ((int)blockIdx.x >= nblk) {
@@ -472,8 +472,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_step_small(const __grid_co
             if (svc == 31) st_release(A.flags + kSmallFlagStride * blockIdx.x, base + s + 1);   // (cumulative over the barrier)
             if (face && __any_sync(0xffffffffu, on_face)) {
                 // face flux, while the flags travel: warp sums, added to the
-                // warp's running sums as unevaluated pairs (TwoSum; an FP64
-                // addition costs about a microsecond of latency here)
+                // warp's running sums in three FP32 parts, more bits than FP64
+                // holds (an FP64 addition costs about a microsecond of latency here)
 #pragma unroll
                 for (int w = 0; w < 6; ++w) {
                     float v = fl[w];
@@ -481,9 +481,9 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_step_small(const __grid_co
 #pragma unroll
                         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
                         if ((tid & 31) == 0) {
-                            const float2 h = flux_s[w][tid >> 5];
-                            const float t = h.x + v, b = t - h.x;
-                            flux_s[w][tid >> 5] = make_float2(t, h.y + ((h.x - (t - b)) + (v - b)));
+                            float3 p = flux_s[w][tid >> 5];
+                            add_expansion(v, p.x, p.y, p.z);
+                            flux_s[w][tid >> 5] = p;
                         }
                     }
                 }
@@ -554,7 +554,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_step_small(const __grid_co
         }
         if (tid < 6) {
             double v = 0.0;
-            for (int w = 0; w < (T >> 5); ++w) v += (double)flux_s[tid][w].x + (double)flux_s[tid][w].y;
+            for (int w = 0; w < (T >> 5); ++w) v += (double)flux_s[tid][w].x + ((double)flux_s[tid][w].y + (double)flux_s[tid][w].z);
             if (v != 0.0) atomicAdd(a.flux.acc + tid * kFluxSlots + blockIdx.x % kFluxSlots, v);
         }
     }
