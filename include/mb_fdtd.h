@@ -330,10 +330,10 @@ int mb_set_single_pass(mb_ctx* ctx, const int tune[4]);
 /* Kernel launches queued per step by mb_step, and in total so far. */
 int mb_launch_stats(mb_ctx* ctx, int* per_step, int64_t* total);
 
-/* Test hook: the n-th device allocation made by mb_create or by the
- * single-pass step's second copy from now on (n = 0: the next one) fails as
- * if the device were out of memory (MB_ERR_OOM, nothing leaked); n < 0
- * switches the injection off.  Process-wide. */
+/* Test hook: the n-th device allocation made by mb_create, by the
+ * single-pass step's second copy or by the adjoint from now on (n = 0: the
+ * next one) fails as if the device were out of memory (MB_ERR_OOM, nothing
+ * leaked); n < 0 switches the injection off.  Process-wide. */
 void mb_debug_fail_alloc(int n);
 
 /* Test hook: the device memory of these allocations starts filled with this
@@ -512,7 +512,7 @@ int mb_halo_unpack(mb_ctx* ctx, int side, const void* d_buf);
  * The context advances n_steps exactly as mb_step would (probes and flux
  * included); then a reverse-time discrete adjoint of the FP32 step runs back
  * over the window.  Forward checkpoints are kept every ckpt_every steps
- * (<= 0: 200); each segment is recomputed and its states stored (48 bytes
+ * (<= 0: 200); each segment is recomputed and its states stored (36 bytes
  * per cell per step) before its reverse sweep.  Noise and sources are held
  * fixed: the gradient is that of the realization with this seed.
  *   d_grad_eps  device array of n_cells floats (x fastest) or NULL:

@@ -21,7 +21,7 @@
 //   R2 (like the H pass, forward differences of mu): lambda_H, psi_H memories;
 //   R3 (like the E pass, backward differences of lambda_H): lambda_E.
 // The three use the forward states x^n and x^{n+1} kept by the segment store.
-#include "mb_host.h"
+#include "mb_ctx.h"
 
 #include <nvtx3/nvToolsExt.h>
 
@@ -608,13 +608,6 @@ int afail(mb_ctx* c, int code, const std::string& msg) {
 
 }  // namespace
 
-void mb::adjoint_release(mb_ctx* c) {
-    if (c->d_adj_ws) cudaFree(c->d_adj_ws);
-    c->d_adj_ws = nullptr;
-    c->dev_bytes -= c->adj_ws_bytes;
-    c->adj_ws_bytes = 0;
-}
-
 extern "C" int mb_adjoint_energy_zface(mb_ctx* c, int n_steps, int ckpt_every, int z_plane,
                                        float* d_grad_eps, double* grad_pump, double* J_out) {
     if (!c) {
@@ -639,6 +632,7 @@ extern "C" int mb_adjoint_energy_zface(mb_ctx* c, int n_steps, int ckpt_every, i
     const bool was_single_pass = mb::hold_in_place(c);
 
     int rc = MB_OK;
+    char* ws = nullptr;   // all of the call's device memory, cut into the following
     char* ckpt = nullptr;
     float* store = nullptr;
     float* adj = nullptr;
@@ -717,25 +711,19 @@ extern "C" int mb_adjoint_energy_zface(mb_ctx* c, int n_steps, int ckpt_every, i
     };
 
     {
-        // one block of device memory for all of it, kept in the context for
-        // the next call where it is at most a sixteenth of the device's memory
-        // (allocating and freeing 8.6 GB took 3.5 ms of a 72 ms call)
+        // one block of device memory for all of it, freed before the call
+        // returns: a caller may count on that memory between its calls
         const size_t part[6] = {sb * (nseg + 1), sizeof(float) * slot * (K + 1), sizeof(float) * (18 * N + psi_total),
                                 sizeof(double) * N, sizeof(double) * 2 * mb::kAccSlots, sizeof(long long) * (K + 1)};
         size_t at[7] = {0};
         for (int q = 0; q < 6; ++q) at[q + 1] = at[q] + (part[q] + 255) / 256 * 256;
-        if (c->adj_ws_bytes < at[6]) {
-            mb::adjoint_release(c);
-            MB_ACUDA(c, cudaMalloc((void**)&c->d_adj_ws, at[6]));
-            c->adj_ws_bytes = at[6];
-            c->dev_bytes += at[6];
-        }
-        ckpt = c->d_adj_ws + at[0];
-        store = reinterpret_cast<float*>(c->d_adj_ws + at[1]);
-        adj = reinterpret_cast<float*>(c->d_adj_ws + at[2]);
-        geps = reinterpret_cast<double*>(c->d_adj_ws + at[3]);
-        acc = reinterpret_cast<double*>(c->d_adj_ws + at[4]);
-        slot_n = reinterpret_cast<long long*>(c->d_adj_ws + at[5]);
+        MB_ACUDA(c, mbi::device_malloc((void**)&ws, at[6]));
+        ckpt = ws + at[0];
+        store = reinterpret_cast<float*>(ws + at[1]);
+        adj = reinterpret_cast<float*>(ws + at[2]);
+        geps = reinterpret_cast<double*>(ws + at[3]);
+        acc = reinterpret_cast<double*>(ws + at[4]);
+        slot_n = reinterpret_cast<long long*>(ws + at[5]);
     }
 
     // forward sweep: a checkpoint at the start of every segment but the last,
@@ -920,10 +908,7 @@ extern "C" int mb_adjoint_energy_zface(mb_ctx* c, int n_steps, int ckpt_every, i
 done:
     if (c->stream) cudaStreamSynchronize(c->stream);
     if (seg_graph) cudaGraphExecDestroy(seg_graph);
-    {
-        size_t free_b = 0, total_b = 0;
-        if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || c->adj_ws_bytes > total_b / 16) mb::adjoint_release(c);
-    }
+    if (ws) cudaFree(ws);
     mb::restore_single_pass(c, was_single_pass);
     return rc;
 }

@@ -892,7 +892,6 @@ int mb_destroy(mb_ctx* c) {
         cudaStreamSynchronize(c->stream);
     }
     drop_graphs(c);
-    mb::adjoint_release(c);
     void* bufs[] = {c->d_fields, c->d_mat, c->d_inv_eps, c->d_lut, c->d_psi[0], c->d_psi[1],
                     c->d_psi[2], c->d_coef, c->d_ctr, c->d_flux, c->d_partial, c->d_energy,
                     c->d_nonfinite, c->d_probe_cell, c->d_probe_omega, c->d_probe_acc,

@@ -319,9 +319,6 @@ void restore_single_pass(mb_ctx* c, bool on);
 // running on the second stream (event waits only; never blocks the host).
 void join_probes(mb_ctx* c);
 
-// Frees the adjoint's device memory kept in the context.
-void adjoint_release(mb_ctx* c);
-
 // d/dW_p of the reduced population propagator (g, G, mk of DevGain).
 void gain_pump_derivative(const mb_ctx* c, float dg[3], float dG[3][3], float dmk[3]);
 
@@ -446,9 +443,6 @@ struct mb_ctx {
     bool use_fused = false;
     mb::PassTune tune_f{mb::kVariantTma, dim3(32, 8, 1), 32};
     float* d_fields2 = nullptr;        // second copy of E, H (6 arrays)
-    // the adjoint's device memory, kept between calls (mb_adjoint.cu)
-    char* d_adj_ws = nullptr;
-    size_t adj_ws_bytes = 0;
     // the small-grid launch: its boxes (bx = 0: not available), and the flag
     // words, step base and probe samples on the device
     mb::SmallTile small{0, 0, 0, 0, 0, 0};
