@@ -293,9 +293,9 @@ int mb_load_state(mb_ctx* ctx, const void* host_blob, size_t bytes);
  * around the trials) and keep the fastest: block shapes of the two field
  * passes, the single-pass step, and on small grids (up to about 60^3 cells)
  * a launch that advances up to 64 steps with the state in shared memory,
- * used for calls of enough steps; mb_get_single_pass reports that one as
- * off.  All give the same bits (the face-flux sums to FP32 rounding).  The
- * choice is cached per grid shape for the process. */
+ * used for calls of enough steps (mb_get_step_launch tells which).  All
+ * give the same bits (the face-flux sums to FP32 rounding).  The choice is
+ * cached per grid shape for the process. */
 int mb_autotune(mb_ctx* ctx);
 
 /* Launch shape of the H pass and of the E pass, as {variant, bx, by, bz}:
@@ -322,10 +322,28 @@ int mb_set_tuning(mb_ctx* ctx, const int tune_h[4], const int tune_e[4]);
  * the two-pass step's bit for bit (the face-flux sums agree to the FP32
  * rounding of their partial sums).  tune = {on (0 or 1), bx, by, kz}: tiles of bx x by columns
  * (32x4, 32x8, 64x4 or 64x8) walking kz planes; needs n_x a multiple of 16.
- * mb_autotune selects it when it is the faster.  Errors: MB_ERR_ARG (bad
- * tile or grid), MB_ERR_OOM (second copy). */
+ * mb_autotune selects it when it is the faster.  Where it selects a launch
+ * that this switch does not cover (this step on rows of another length, many
+ * steps a launch), the answer is {0, bx, by, -kz}, and setting that answer,
+ * here or on another context, selects that launch again where the grid takes
+ * it; {0, .., kz >= 0} is off.  Errors: MB_ERR_ARG (bad tile or grid),
+ * MB_ERR_OOM (second copy). */
 int mb_get_single_pass(mb_ctx* ctx, int tune[4]);
 int mb_set_single_pass(mb_ctx* ctx, const int tune[4]);
+
+/* The launch that mb_step takes, whatever selected it, as {kind, bx, by, kz}:
+ * MB_LAUNCH_TWO_PASSES (the other values are ignored), MB_LAUNCH_SINGLE_PASS
+ * (as above, on any rows of a multiple of 4 cells, or padded to one: n_x
+ * within a sixteenth of the next multiple, where memory was left for it) or
+ * MB_LAUNCH_MANY_STEPS (small grids with up to 4 point probes of 1024 bins:
+ * up to 64 steps a launch, for calls of at least kz steps; bx and by are 0).
+ * Errors of the setter: MB_ERR_ARG (a launch that the grid does not take),
+ * MB_ERR_OOM; the launch is then as before. */
+#define MB_LAUNCH_TWO_PASSES 0
+#define MB_LAUNCH_SINGLE_PASS 1
+#define MB_LAUNCH_MANY_STEPS 2
+int mb_get_step_launch(mb_ctx* ctx, int launch[4]);
+int mb_set_step_launch(mb_ctx* ctx, const int launch[4]);
 
 /* Kernel launches queued per step by mb_step, and in total so far. */
 int mb_launch_stats(mb_ctx* ctx, int* per_step, int64_t* total);

@@ -19,6 +19,7 @@ LIB_PATH = os.path.join(_PKG, "libmbfdtd.so")
 MB_OK, MB_ERR_ARG, MB_ERR_COURANT, MB_ERR_OOM, MB_ERR_MATERIALS = 0, -1, -2, -3, -4
 MB_ERR_TIMEOUT, MB_ERR_NONFINITE, MB_ERR_CUDA, MB_ERR_STATE = -5, -6, -7, -8
 MB_BATCH_PERSISTENT, MB_BATCH_CONCURRENT = 0, 1
+MB_LAUNCH_TWO_PASSES, MB_LAUNCH_SINGLE_PASS, MB_LAUNCH_MANY_STEPS = 0, 1, 2
 ERROR_NAMES = {MB_ERR_ARG: "MB_ERR_ARG", MB_ERR_COURANT: "MB_ERR_COURANT", MB_ERR_OOM: "MB_ERR_OOM",
                MB_ERR_MATERIALS: "MB_ERR_MATERIALS", MB_ERR_TIMEOUT: "MB_ERR_TIMEOUT",
                MB_ERR_NONFINITE: "MB_ERR_NONFINITE", MB_ERR_CUDA: "MB_ERR_CUDA",
@@ -102,6 +103,8 @@ _SIGS = [
     ("mb_debug_fill_alloc", None, [C.c_int]),
     ("mb_get_single_pass", C.c_int, [_P, C.POINTER(C.c_int)]),
     ("mb_set_single_pass", C.c_int, [_P, C.POINTER(C.c_int)]),
+    ("mb_get_step_launch", C.c_int, [_P, C.POINTER(C.c_int)]),
+    ("mb_set_step_launch", C.c_int, [_P, C.POINTER(C.c_int)]),
     ("mb_launch_stats", C.c_int, [_P, C.POINTER(C.c_int), C.POINTER(C.c_int64)]),
     ("mb_device_bytes", C.c_int, [_P, C.POINTER(C.c_size_t)]),
     ("mb_philox4x32_10", C.c_int, [_P, _P, _P, C.c_int]),
@@ -469,8 +472,20 @@ def mb_set_tuning(h, tune_h, tune_e):
     _check(load_library().mb_set_tuning(h, (C.c_int * 4)(*tune_h), (C.c_int * 4)(*tune_e)), h)
 
 
+def mb_get_step_launch(h):
+    """(kind, bx, by, kz) of the launch mb_step takes (MB_LAUNCH_*)."""
+    t = (C.c_int * 4)()
+    _check(load_library().mb_get_step_launch(h, t), h)
+    return tuple(t)
+
+
+def mb_set_step_launch(h, launch):
+    _check(load_library().mb_set_step_launch(h, (C.c_int * 4)(*launch)), h)
+
+
 def mb_get_single_pass(h):
-    """(on, bx, by, kz) of the single-pass step."""
+    """(on, bx, by, kz) of the single-pass step; on = 0 and kz < 0: another
+    launch, selected by the tuner (mb_get_step_launch)."""
     t = (C.c_int * 4)()
     _check(load_library().mb_get_single_pass(h, t), h)
     return tuple(t)
@@ -781,8 +796,17 @@ class MBSimulation:
     def set_tuning(self, tune_h, tune_e):
         mb_set_tuning(self._h, tune_h, tune_e)
 
+    def step_launch(self):
+        """(kind, bx, by, kz) of the launch that step takes: kind 0 two passes, 1 the
+        single-pass step, 2 many steps of a small grid (calls of kz steps or more)."""
+        return mb_get_step_launch(self._h)
+
+    def set_step_launch(self, launch):
+        mb_set_step_launch(self._h, launch)
+
     def single_pass(self):
-        """(on, bx, by, kz) of the single-pass step."""
+        """(on, bx, by, kz) of the single-pass step; on = 0 and kz < 0: another
+        launch that the tuner selected (:meth:`step_launch`)."""
         return mb_get_single_pass(self._h)
 
     def set_single_pass(self, tune):

@@ -92,8 +92,11 @@ constexpr size_t kSmallWords = mb::kSmallFlagWords + 1 + 3 * (size_t)mb::kSmallM
 // The boxes of the small-grid launch and its device words (flags, step base,
 // probe samples), made on first use; false where the grid is too large for
 // it or holds more point probes than it advances.
+bool small_takes_probes(const mb_ctx* c) {
+    return (int)c->probes.size() <= mb::kSmallMaxProbes && c->probe_nfreq <= mb::kSmallMaxBins;
+}
 bool small_ready(mb_ctx* c) {
-    if ((int)c->probes.size() > mb::kSmallMaxProbes || c->probe_nfreq > mb::kSmallMaxBins) return false;
+    if (!small_takes_probes(c)) return false;
     if (c->d_small) return true;
     if (!c->small.bx) {
         int sms = 0;
@@ -632,15 +635,62 @@ int mb_autotune(mb_ctx* c) {
     return MB_OK;
 }
 
-int mb_get_single_pass(mb_ctx* c, int tune[4]) {
+int mb_get_step_launch(mb_ctx* c, int launch[4]) {
     if (int rc = check_ctx(c)) return rc;
-    if (!tune) return fail(c, MB_ERR_ARG, "null output");
-    // the small-grid launch, and the single-pass step on rows that are not a
-    // multiple of 16 cells, are the tuner's choice alone: reported as off
-    tune[0] = c->use_fused && !small_on(c) && mb::tma_e_supported(c->args) ? 1 : 0;
-    tune[1] = c->tune_f.block.x;
-    tune[2] = c->tune_f.block.y;
-    tune[3] = c->tune_f.kz;
+    if (!launch) return fail(c, MB_ERR_ARG, "null output");
+    const bool small = small_on(c);
+    launch[0] = !c->use_fused ? MB_LAUNCH_TWO_PASSES : small ? MB_LAUNCH_MANY_STEPS : MB_LAUNCH_SINGLE_PASS;
+    launch[1] = small ? 0 : (int)c->tune_f.block.x;
+    launch[2] = small ? 0 : (int)c->tune_f.block.y;
+    launch[3] = c->tune_f.kz;
+    return MB_OK;
+}
+
+int mb_set_step_launch(mb_ctx* c, const int launch[4]) {
+    if (int rc = check_ctx(c)) return rc;
+    if (!launch) return fail(c, MB_ERR_ARG, "null input");
+    mb::PassTune t{mb::kVariantTma, dim3(32, 8, 1), launch[3]};
+    switch (launch[0]) {
+        case MB_LAUNCH_TWO_PASSES:
+            c->use_fused = false;
+            drop_graphs(c);
+            return MB_OK;
+        case MB_LAUNCH_SINGLE_PASS:
+            if (!mb::fused_tile_supported(launch[1], launch[2]) || launch[3] < 1)
+                return fail(c, MB_ERR_ARG, "single-pass tiles are 32x4, 32x8, 64x4 or 64x8, kz >= 1");
+            if (!mb::fused_supported(c->args))
+                return fail(c, MB_ERR_ARG, "the single-pass step needs rows of a multiple of 4 cells or padded to one");
+            t.block = dim3(launch[1], launch[2], 1);
+            break;
+        case MB_LAUNCH_MANY_STEPS:
+            if (launch[3] < 1 || launch[3] > mb::kSmallMaxSteps)
+                return fail(c, MB_ERR_ARG, "many steps a launch: calls of 1 to 64 steps and more");
+            if (!small_takes_probes(c))
+                return fail(c, MB_ERR_ARG, "more point probes or bins than many steps a launch advance");
+            t.variant = mb::kVariantSmall;
+            if (!small_ready(c))
+                return c->small.bx ? fail(c, MB_ERR_OOM, "allocation for the launch of many steps failed")
+                                   : fail(c, MB_ERR_ARG, "the grid is too large for many steps a launch");
+            break;
+        default:
+            return fail(c, MB_ERR_ARG, "the launch must be 0 (two passes), 1 (single pass) or 2 (many steps)");
+    }
+    if (int rc = ensure_second_copy(c)) return rc;
+    if (!fused_maps_for(c, t)) return fail(c, MB_ERR_ARG, "tensor maps of the single-pass step cannot be encoded");
+    c->tune_f = t;
+    c->use_fused = true;
+    drop_graphs(c);
+    return MB_OK;
+}
+
+int mb_get_single_pass(mb_ctx* c, int tune[4]) {
+    if (int rc = mb_get_step_launch(c, tune)) return rc;
+    // a launch outside this switch: off, with kz negated, so that
+    // mb_set_single_pass of the answer gives the same launch again
+    if (tune[0] && (tune[0] != MB_LAUNCH_SINGLE_PASS || !mb::tma_e_supported(c->args))) {
+        tune[0] = 0;
+        tune[3] = -tune[3];
+    }
     return MB_OK;
 }
 
@@ -648,22 +698,17 @@ int mb_set_single_pass(mb_ctx* c, const int tune[4]) {
     if (int rc = check_ctx(c)) return rc;
     if (!tune) return fail(c, MB_ERR_ARG, "null input");
     if (tune[0] != 0 && tune[0] != 1) return fail(c, MB_ERR_ARG, "tune[0] must be 0 or 1");
-    if (tune[0] == 0) {
-        c->use_fused = false;
-        drop_graphs(c);
-        return MB_OK;
-    }
-    if (!mb::fused_tile_supported(tune[1], tune[2]) || tune[3] < 1)
-        return fail(c, MB_ERR_ARG, "single-pass tiles are 32x4, 32x8, 64x4 or 64x8, kz >= 1");
-    if (!mb::tma_e_supported(c->args))
+    if (tune[0] == 1 && !mb::tma_e_supported(c->args) && mb::fused_tile_supported(tune[1], tune[2]) && tune[3] >= 1)
         return fail(c, MB_ERR_ARG, "the single-pass step needs n_x % 16 == 0");
-    if (int rc = ensure_second_copy(c)) return rc;
-    const mb::PassTune t{mb::kVariantTma, dim3(tune[1], tune[2], 1), tune[3]};
-    if (!fused_maps_for(c, t)) return fail(c, MB_ERR_ARG, "tensor maps of the single-pass step cannot be encoded");
-    c->tune_f = t;
-    c->use_fused = true;
-    drop_graphs(c);
-    return MB_OK;
+    int launch[4] = {tune[0], tune[1], tune[2], tune[3]};
+    if (tune[0] == 0 && tune[3] < 0) {   // an answer of mb_get_single_pass, from this grid or from another
+        launch[0] = tune[1] ? MB_LAUNCH_SINGLE_PASS : MB_LAUNCH_MANY_STEPS;
+        launch[3] = -tune[3];
+        if (mb_set_step_launch(c, launch) == MB_OK) return MB_OK;
+        c->err.clear();
+        launch[0] = MB_LAUNCH_TWO_PASSES;
+    }
+    return mb_set_step_launch(c, launch);
 }
 
 int mb_get_tuning(mb_ctx* c, int tune_h[4], int tune_e[4]) {
