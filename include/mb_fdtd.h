@@ -111,7 +111,9 @@ const char* mb_last_error(const mb_ctx* ctx);
  * rate W_p (1/s) from N0 to N3, constant in time.  Resets P, J and the
  * populations; fields and probes are kept.  With <= 128 distinct eps values
  * the map is stored as a uint8 material id per cell, otherwise as a dense
- * FP32 1/eps_r map.  Errors: MB_ERR_ARG, MB_ERR_MATERIALS. */
+ * FP32 1/eps_r map.  Errors: MB_ERR_ARG, MB_ERR_MATERIALS, MB_ERR_OOM (the
+ * material is then the one before, or, where the list of gain cells has no
+ * memory, none: vacuum, as after mb_create). */
 int mb_set_material(mb_ctx* ctx, const float* eps_map, const uint8_t* gain_mask,
                     double N_a, double pump);
 
@@ -349,7 +351,8 @@ int mb_set_step_launch(mb_ctx* ctx, const int launch[4]);
 int mb_launch_stats(mb_ctx* ctx, int* per_step, int64_t* total);
 
 /* Test hook: the n-th device allocation made by mb_create, by the
- * single-pass step's second copy or by the adjoint from now on (n = 0: the
+ * single-pass step's second copy, by the adjoint, for the gain list or for
+ * face probes from now on (n = 0: the
  * next one) fails as if the device were out of memory (MB_ERR_OOM, nothing
  * leaked); n < 0 switches the injection off.  Process-wide. */
 void mb_debug_fail_alloc(int n);

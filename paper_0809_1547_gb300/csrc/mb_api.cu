@@ -1024,16 +1024,38 @@ int mb_set_material(mb_ctx* c, const float* eps_map, const uint8_t* gain_mask, d
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
     const size_t n_gain = n_gain32;
     if (n_gain > c->glist_capacity || !c->d_glist) {
-        if (c->d_glist) {
+        auto free_lists = [&]() {
             cudaFree(c->d_glist);
             cudaFree(c->d_glist_num);
-            c->dev_bytes -= sizeof(uint32_t) * c->glist_capacity * (rows ? 2 : 1);
             c->d_glist = c->d_glist_num = nullptr;
-        }
+        };
+        free_lists();
+        c->dev_bytes -= sizeof(uint32_t) * c->glist_capacity * (rows ? 2 : 1);
+        c->glist_capacity = 0;
         const size_t cap = n_gain ? n_gain : 1;
-        cudaError_t e = cudaMalloc((void**)&c->d_glist, sizeof(uint32_t) * cap);
-        if (e == cudaSuccess && rows) e = cudaMalloc((void**)&c->d_glist_num, sizeof(uint32_t) * cap);
-        if (e != cudaSuccess) { cudaGetLastError(); return fail(c, MB_ERR_OOM, "gain list allocation failed"); }
+        cudaError_t e = device_malloc((void**)&c->d_glist, sizeof(uint32_t) * cap);
+        if (e == cudaSuccess && rows) e = device_malloc((void**)&c->d_glist_num, sizeof(uint32_t) * cap);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            free_lists();
+            // the material bytes are the new map's already, the old lists are
+            // gone: as mb_create left the context, without a material
+            std::fill(lut.begin(), lut.end(), 1.0f);
+            c->h_lut_eps.assign(128, 1.0f);
+            c->n_lut = 128;
+            c->h_lut_ie[0] = c->h_lut_ie[1] = 1.0f;
+            c->dense_eps = c->have_material = false;
+            c->N_a = c->W_p = 0.0;
+            c->glist_count = 0;
+            cudaMemsetAsync(c->d_mat, 0, (size_t)c->pcell, c->stream);
+            cudaMemcpyAsync(c->d_lut, lut.data(), sizeof(float) * 256, cudaMemcpyHostToDevice, c->stream);
+            cudaMemsetAsync(c->args.f.gs, 0, sizeof(float) * mb::gain_floats(c->pcell), c->stream);
+            cudaStreamSynchronize(c->stream);
+            build_args(c);
+            gain_coefficients(c);
+            drop_graphs(c);
+            return fail(c, MB_ERR_OOM, "gain list allocation failed");
+        }
         c->glist_capacity = cap;
         c->dev_bytes += sizeof(uint32_t) * cap * (rows ? 2 : 1);
     }
