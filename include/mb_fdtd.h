@@ -134,7 +134,8 @@ int mb_add_point_probe(mb_ctx* ctx, const int ijk[3], int n_freq,
  * at t_{n+1}) and H (half a cell outside, at t_{n+1/2}) are accumulated into
  * running DFTs every `every` steps (1 <= n_freq <= 4096): FP32 sums over 16
  * consecutive accumulations, each added into FP64 sums on the device (the
- * spectrum reads both).  Replaces earlier face probes. */
+ * spectrum reads both).  Replaces earlier face probes (on an error there
+ * are none). */
 int mb_add_face_probes(mb_ctx* ctx, int stride, int every, int n_freq,
                        double lam_min, double lam_max);
 

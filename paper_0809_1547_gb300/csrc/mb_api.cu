@@ -1147,7 +1147,8 @@ int mb_add_face_probes(mb_ctx* c, int stride, int every, int n_freq, double lam_
     if (c->d_face_acc32) { cudaFree(c->d_face_acc32); c->d_face_acc32 = nullptr; }
     if (c->d_face_omega) { cudaFree(c->d_face_omega); c->d_face_omega = nullptr; }
     if (c->d_face_spec) { cudaFree(c->d_face_spec); c->d_face_spec = nullptr; }
-    mb::DevFaceProbes& F = c->face;
+    drop_graphs(c);   // (they hold the old sums)
+    mb::DevFaceProbes& F = c->face;   // off until its memory is there
     std::memset(&F, 0, sizeof(F));
     const int n3[3] = {c->nx, c->ny, c->nz};
     const int L = c->p.npml;
@@ -1192,7 +1193,6 @@ int mb_add_face_probes(mb_ctx* c, int stride, int every, int n_freq, double lam_
         F.offset[face] = (int)off;
         off += (int64_t)na * nb;
     }
-    F.on = 1;
     F.stride = stride;
     F.every = every;
     F.nfreq = n_freq;
@@ -1205,18 +1205,18 @@ int mb_add_face_probes(mb_ctx* c, int stride, int every, int n_freq, double lam_
         c->face_lam.push_back(lam);
         om.push_back(2.0 * kPi * kC0 / lam);
     }
-    MB_CUDA(c, cudaMalloc((void**)&c->d_face_omega, sizeof(double) * n_freq));
+    MB_CUDA(c, device_malloc((void**)&c->d_face_omega, sizeof(double) * n_freq));
     MB_CUDA(c, cudaMemcpy(c->d_face_omega, om.data(), sizeof(double) * n_freq, cudaMemcpyHostToDevice));
     const size_t accn = 4 * (size_t)off * n_freq;
-    MB_CUDA(c, cudaMalloc((void**)&c->d_face_acc, sizeof(double2) * (accn ? accn : 1)));
+    MB_CUDA(c, device_malloc((void**)&c->d_face_acc, sizeof(double2) * (accn ? accn : 1)));
     MB_CUDA(c, cudaMemset(c->d_face_acc, 0, sizeof(double2) * (accn ? accn : 1)));
-    MB_CUDA(c, cudaMalloc((void**)&c->d_face_acc32, sizeof(float2) * (accn ? accn : 1)));
+    MB_CUDA(c, device_malloc((void**)&c->d_face_acc32, sizeof(float2) * (accn ? accn : 1)));
     MB_CUDA(c, cudaMemset(c->d_face_acc32, 0, sizeof(float2) * (accn ? accn : 1)));
-    MB_CUDA(c, cudaMalloc((void**)&c->d_face_spec, sizeof(double) * (mb::kFaceSpecChunks + 1) * (size_t)n_freq));
+    MB_CUDA(c, device_malloc((void**)&c->d_face_spec, sizeof(double) * (mb::kFaceSpecChunks + 1) * (size_t)n_freq));
     F.omega = c->d_face_omega;
     F.acc = c->d_face_acc;
     F.acc32 = c->d_face_acc32;
-    drop_graphs(c);
+    F.on = 1;
     return MB_OK;
 }
 
