@@ -351,11 +351,12 @@ int mb_set_step_launch(mb_ctx* ctx, const int launch[4]);
 /* Kernel launches queued per step by mb_step, and in total so far. */
 int mb_launch_stats(mb_ctx* ctx, int* per_step, int64_t* total);
 
-/* Test hook: the n-th device allocation made by mb_create, by the
- * single-pass step's second copy, by the adjoint, for the gain list or for
- * face probes from now on (n = 0: the
- * next one) fails as if the device were out of memory (MB_ERR_OOM, nothing
- * leaked); n < 0 switches the injection off.  Process-wide. */
+/* Test hook: the n-th device allocation from now on (n = 0: the next one)
+ * made by mb_create, by the single-pass step's second copy, by the adjoint,
+ * for the gain list, for face probes, or for fields read and written before
+ * a material is set (which then cross through host memory) fails as if the
+ * device were out of memory (MB_ERR_OOM, nothing leaked); n < 0 switches the
+ * injection off.  Process-wide. */
 void mb_debug_fail_alloc(int n);
 
 /* Test hook: the device memory of these allocations starts filled with this

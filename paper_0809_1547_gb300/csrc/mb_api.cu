@@ -299,24 +299,45 @@ size_t host_bytes(const mb_ctx* c, const StatePart& p) {
     return p.arrays ? sizeof(float) * (size_t)p.arrays * c->ncell : p.bytes;
 }
 
-// The material's upload buffer (made here where no material is set yet).
-bool ensure_upload(mb_ctx* c) {
-    if (c->d_upload) return true;
+// Where fields cross packed between host and device, an array at a time: the
+// material's upload buffer (made here where no material is set yet) or, where
+// the device has no memory left for it, page-locked host memory, which the
+// kernels reach as well; null where neither can be had.
+uint8_t* staging(mb_ctx* c) {
+    if (c->d_upload) return c->d_upload;
     const size_t bytes = 5 * (size_t)c->ncell + 16;
-    if (cudaMalloc((void**)&c->d_upload, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        c->d_upload = nullptr;
-        return false;
+    if (device_malloc((void**)&c->d_upload, bytes) == cudaSuccess) {
+        c->upload_bytes = bytes;
+        return c->d_upload;
     }
-    c->upload_bytes = bytes;
-    return true;
+    cudaGetLastError();
+    c->d_upload = nullptr;
+    if (!c->h_stage && cudaMallocHost((void**)&c->h_stage, sizeof(float) * (size_t)c->ncell) != cudaSuccess) {
+        cudaGetLastError();
+        c->h_stage = nullptr;
+    }
+    return c->h_stage;
+}
+// bytes between the staging memory and the host, after and before the
+// kernels around it.
+cudaError_t stage_out(mb_ctx* c, void* host, const uint8_t* stage, size_t bytes) {
+    if (stage != c->h_stage) return cudaMemcpyAsync(host, stage, bytes, cudaMemcpyDeviceToHost, c->stream);
+    const cudaError_t e = cudaStreamSynchronize(c->stream);
+    if (e == cudaSuccess) std::memcpy(host, stage, bytes);
+    return e;
+}
+cudaError_t stage_in(mb_ctx* c, uint8_t* stage, const void* host, size_t bytes) {
+    if (stage != c->h_stage) return cudaMemcpyAsync(stage, host, bytes, cudaMemcpyHostToDevice, c->stream);
+    const cudaError_t e = cudaStreamSynchronize(c->stream);
+    if (e == cudaSuccess) std::memcpy(stage, host, bytes);
+    return e;
 }
 
 // Padded rows and the gain blocks are packed and spread by kernels (a 2-D
 // device copy of rows of 157 floats measured 13 us more than the plain copy;
 // the kernel as much as it).  To and from the host they cross packed, an array
-// at a time through the material's upload buffer (2.7 M cells: a field read
-// 1.7 ms as without padding; packed on the host 2.7 ms).
+// at a time through the staging memory (2.7 M cells: a field read 1.7 ms as
+// without padding; packed on the host 2.7 ms).
 cudaError_t rows_out(mb_ctx* c, void* packed, const void* rows, size_t esize, int arrays, cudaMemcpyKind kind) {
     if (c->px == c->nx)
         return cudaMemcpyAsync(packed, rows, esize * (size_t)arrays * c->ncell, kind, c->stream);
@@ -326,10 +347,11 @@ cudaError_t rows_out(mb_ctx* c, void* packed, const void* rows, size_t esize, in
         mb::launch_rows(rows, c->px, packed, c->nx, c->nx, nrow * arrays, (int)esize, c->stream);
         return cudaGetLastError();
     }
-    if (!ensure_upload(c)) return cudaErrorMemoryAllocation;
+    uint8_t* stage = staging(c);
+    if (!stage) return cudaErrorMemoryAllocation;
     for (int q = 0; q < arrays; ++q) {
-        mb::launch_rows((const char*)rows + from * q, c->px, c->d_upload, c->nx, c->nx, nrow, (int)esize, c->stream);
-        cudaError_t e = cudaMemcpyAsync((char*)packed + to * q, c->d_upload, to, kind, c->stream);
+        mb::launch_rows((const char*)rows + from * q, c->px, stage, c->nx, c->nx, nrow, (int)esize, c->stream);
+        cudaError_t e = stage_out(c, (char*)packed + to * q, stage, to);
         if (e != cudaSuccess) return e;
     }
     return cudaGetLastError();
@@ -343,30 +365,33 @@ cudaError_t rows_in(mb_ctx* c, void* rows, const void* packed, size_t esize, int
         mb::launch_rows(packed, c->nx, rows, c->px, c->nx, nrow * arrays, (int)esize, c->stream);
         return cudaGetLastError();
     }
-    if (!ensure_upload(c)) return cudaErrorMemoryAllocation;
+    uint8_t* stage = staging(c);
+    if (!stage) return cudaErrorMemoryAllocation;
     for (int q = 0; q < arrays; ++q) {
-        cudaError_t e = cudaMemcpyAsync(c->d_upload, (const char*)packed + from * q, from, kind, c->stream);
+        cudaError_t e = stage_in(c, stage, (const char*)packed + from * q, from);
         if (e != cudaSuccess) return e;
-        mb::launch_rows(c->d_upload, c->nx, (char*)rows + to * q, c->px, c->nx, nrow, (int)esize, c->stream);
+        mb::launch_rows(stage, c->nx, (char*)rows + to * q, c->px, c->nx, nrow, (int)esize, c->stream);
     }
     return cudaGetLastError();
 }
 cudaError_t field_out(mb_ctx* c, void* packed, int which, cudaMemcpyKind kind) {
     if (which < MB_PX) return rows_out(c, packed, eh_ptr(c, which), 4, 1, kind);
     const bool dev = kind == cudaMemcpyDeviceToDevice;
-    if (!dev && !ensure_upload(c)) return cudaErrorMemoryAllocation;
-    float* to = dev ? (float*)packed : (float*)c->d_upload;
-    mb::launch_gain_rows(c->args.f.gs, gain_comp(which), c->px, to, c->nx, (int64_t)c->ny * c->nz, true, c->stream);
-    if (!dev) cudaMemcpyAsync(packed, to, sizeof(float) * (size_t)c->ncell, kind, c->stream);
-    return cudaGetLastError();
+    uint8_t* stage = dev ? nullptr : staging(c);
+    if (!dev && !stage) return cudaErrorMemoryAllocation;
+    mb::launch_gain_rows(c->args.f.gs, gain_comp(which), c->px, dev ? (float*)packed : (float*)stage, c->nx,
+                         (int64_t)c->ny * c->nz, true, c->stream);
+    const cudaError_t e = dev ? cudaSuccess : stage_out(c, packed, stage, sizeof(float) * (size_t)c->ncell);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 cudaError_t field_in(mb_ctx* c, int which, const void* packed, cudaMemcpyKind kind) {
     if (which < MB_PX) return rows_in(c, eh_ptr(c, which), packed, 4, 1, kind);
-    if (!ensure_upload(c)) return cudaErrorMemoryAllocation;
-    float* from = (float*)c->d_upload;
-    cudaError_t e = cudaMemcpyAsync(from, packed, sizeof(float) * (size_t)c->ncell, kind, c->stream);
+    uint8_t* stage = staging(c);
+    if (!stage) return cudaErrorMemoryAllocation;
+    cudaError_t e = stage_in(c, stage, packed, sizeof(float) * (size_t)c->ncell);
     if (e != cudaSuccess) return e;
-    mb::launch_gain_rows(c->args.f.gs, gain_comp(which), c->px, from, c->nx, (int64_t)c->ny * c->nz, false, c->stream);
+    mb::launch_gain_rows(c->args.f.gs, gain_comp(which), c->px, (float*)stage, c->nx, (int64_t)c->ny * c->nz, false,
+                         c->stream);
     return cudaGetLastError();
 }
 // The gain fields in blob order.
@@ -901,6 +926,7 @@ int mb_destroy(mb_ctx* c) {
                     c->d_small_x};
     for (void* b : bufs)
         if (b) cudaFree(b);
+    if (c->h_stage) cudaFreeHost(c->h_stage);
     for (const mb::DevPlaneProbe& q : c->planes) {
         cudaFree(const_cast<double*>(q.omega));
         cudaFree(q.acc);

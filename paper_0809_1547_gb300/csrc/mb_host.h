@@ -419,6 +419,7 @@ struct mb_ctx {
     // (5 bytes per cell), the table of distinct values and two flags
     uint8_t* d_upload = nullptr;
     size_t upload_bytes = 0;
+    uint8_t* h_stage = nullptr;        // page-locked, made where a field read finds no device memory
     uint32_t* d_keys = nullptr;
     size_t keys_bytes = 0;
     std::vector<float> h_lut_eps;      // eps_r per material id
