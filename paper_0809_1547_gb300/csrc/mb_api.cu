@@ -394,6 +394,31 @@ cudaError_t field_in(mb_ctx* c, int which, const void* packed, cudaMemcpyKind ki
                          c->stream);
     return cudaGetLastError();
 }
+// Can a kernel of this context store `bytes` of floats at p: memory of its own
+// device, aligned, inside one allocation?  A copy takes any address and turns
+// a bad one into an error; a store there would fault.
+bool kernel_writes(const mb_ctx* c, const float* p, size_t bytes) {
+    using RangeFn = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+    static const RangeFn range = []() -> RangeFn {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            return (RangeFn)f;
+        cudaGetLastError();
+        return nullptr;
+    }();
+    cudaPointerAttributes at{};
+    if (!range || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    return (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) && at.device == c->device &&
+           (uintptr_t)p % sizeof(float) == 0 && range(&base, &size, (CUdeviceptr)p) == CUDA_SUCCESS &&
+           (CUdeviceptr)p + bytes <= base + size;
+}
 // The gain fields in blob order.
 constexpr int kGainFields[9] = {MB_PX, MB_PY, MB_PZ, MB_JX, MB_JY, MB_JZ, MB_N1, MB_N2, MB_N3};
 
@@ -1614,7 +1639,16 @@ int mb_get_field_device(mb_ctx* c, int which, float* dev_out, double* scale) {
     if (int rc = check_ctx(c)) return rc;
     if (!dev_out || which < 0 || which >= MB_NUM_FIELDS || which == MB_N0)
         return fail(c, MB_ERR_ARG, "bad field id (N0 is not stored) or null output");
-    MB_CUDA(c, field_out(c, dev_out, which, cudaMemcpyDeviceToDevice));
+    const size_t bytes = sizeof(float) * (size_t)c->ncell;
+    if ((which < MB_PX && c->px == c->nx) || kernel_writes(c, dev_out, bytes)) {
+        MB_CUDA(c, field_out(c, dev_out, which, cudaMemcpyDeviceToDevice));
+    } else {
+        uint8_t* stage = staging(c);
+        if (!stage) return fail(c, MB_ERR_OOM, "no memory for the packed field");
+        MB_CUDA(c, field_out(c, stage, which, cudaMemcpyDeviceToDevice));
+        MB_CUDA(c, cudaMemcpyAsync(dev_out, stage, bytes,
+                                   stage == c->h_stage ? cudaMemcpyDefault : cudaMemcpyDeviceToDevice, c->stream));
+    }
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
     if (scale) *scale = field_scale(c, which);
     return MB_OK;
