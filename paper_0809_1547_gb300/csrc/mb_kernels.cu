@@ -523,8 +523,17 @@ void launch_rows(const void* src, int from, void* dst, int to, int nx, int64_t c
         k_rows<uint8_t><<<blocks, 256, 0, s>>>((const uint8_t*)src, from, (uint8_t*)dst, to, nx, count);
 }
 
+// A load that asks L2 for 64 bytes around the address instead of the 128 that
+// a plain load brings from HBM here.
+__device__ __forceinline__ float load_64(const float* p) {
+    float v;
+    asm volatile("ld.global.L2::64B.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
 // One component of P, J or the populations (its place comp floats into the
-// blocks) to (OUT) or from the packed array, a row a warp.
+// blocks) to (OUT) or from the packed array, a row a warp.  Bound by memory:
+// a block's eight values are 32 bytes of 288, of which HBM reads 64 at least,
+// so a read moves 1.5 times the bytes of a copy; a plain load moved 2.5 times.
 template <bool OUT>
 __global__ void __launch_bounds__(256) k_gain_rows(float* __restrict__ gs, int comp, int px, float* __restrict__ packed,
                                                    int nx, int64_t count) {
@@ -537,7 +546,7 @@ __global__ void __launch_bounds__(256) k_gain_rows(float* __restrict__ gs, int c
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int x = i + 32 * q;
-                if (x < nx) v[q] = OUT ? gs[gain_place((uint32_t)(r * px + x)) + comp] : b[x];
+                if (x < nx) v[q] = OUT ? load_64(gs + gain_place((uint32_t)(r * px + x)) + comp) : b[x];
             }
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
