@@ -110,9 +110,13 @@ __device__ void small_probe(const SmallArgs& A, int p, unsigned base, long long 
         for (int c = 0; c < 3; ++c) v[c] = pp.acc[((int64_t)p * 3 + c) * K + kk];
     }
     for (int s = 0; s < A.nsteps; ++s) {
-        if (threadIdx.x == 0 && !wait_flag(A.flags + kSmallFlagStride * owner, base + s + 1)) *fail_s = 1;
-        __syncthreads();
-        if (*fail_s) break;
+        // the barrier carries the verdict: a flag in shared memory could be set
+        // for step s + 1 while a slower warp still reads it for step s
+        const bool late = threadIdx.x == 0 && !wait_flag(A.flags + kSmallFlagStride * owner, base + s + 1);
+        if (__syncthreads_or(late)) {
+            if (late) *fail_s = 1;
+            break;
+        }
         if (kk < K) {
             const float* e = A.samples + ((size_t)s * pp.count + p) * 3;
             const float2 ph = phase_f32(w, (double)(n0 + s + 1) * A.dt);
