@@ -355,8 +355,9 @@ int mb_launch_stats(mb_ctx* ctx, int* per_step, int64_t* total);
  * made by mb_create, by the single-pass step's second copy, by the adjoint,
  * for the gain list, for face probes, or for fields read and written before
  * a material is set (which then cross through host memory) fails as if the
- * device were out of memory (MB_ERR_OOM, nothing leaked); n < 0 switches the
- * injection off.  Process-wide. */
+ * device were out of memory (MB_ERR_OOM, nothing leaked); on a grid whose rows
+ * mb_create would pad, its first is the look at the memory left, and the rows
+ * are then not padded; n < 0 switches the injection off.  Process-wide. */
 void mb_debug_fail_alloc(int n);
 
 /* Test hook: the device memory of these allocations starts filled with this

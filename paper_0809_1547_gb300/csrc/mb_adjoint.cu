@@ -581,9 +581,9 @@ __global__ void k_adj_out(const double* geps, float* out, uint32_t n, uint32_t n
 
 namespace {
 
-// Launch shapes of the recomputation per grid shape and CPML depth.
+// Launch shapes of the recomputation per grid shape, row length and CPML depth.
 std::mutex g_shape_mu;
-std::map<std::tuple<int, int, int, int>, std::pair<mb::PassTune, mb::PassTune>> g_shapes;
+std::map<mbi::TuneKey, std::pair<mb::PassTune, mb::PassTune>> g_shapes;
 
 struct NvtxScope {
     explicit NvtxScope(const char* name) { nvtxRangePushA(name); }
@@ -741,7 +741,7 @@ extern "C" int mb_adjoint_energy_zface(mb_ctx* c, int n_steps, int ckpt_every, i
         th = te_r = mb::PassTune{mb::kVariant3D, dim3(64, 4, 1), 1};
         have_shape = true;
     }
-    const auto shape_key = std::make_tuple(c->nx, c->ny, c->nz, c->p.npml);
+    const mbi::TuneKey shape_key = mbi::tune_key(c);
     if (!have_shape) {
         std::lock_guard<std::mutex> lk(g_shape_mu);
         const auto it = g_shapes.find(shape_key);

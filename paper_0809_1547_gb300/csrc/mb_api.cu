@@ -28,10 +28,14 @@ thread_local std::string g_err;
 // allocations are filled with (-1: left as they come)
 std::atomic<int> g_fail_alloc_after{-1}, g_fill_alloc{-1};
 
-cudaError_t device_malloc(void** p, size_t bytes) {
+static bool inject_alloc_failure() {
     int v = g_fail_alloc_after.load();
     while (v >= 0 && !g_fail_alloc_after.compare_exchange_weak(v, v - 1)) {}
-    cudaError_t e = v == 0 ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+    return v == 0;
+}
+
+cudaError_t device_malloc(void** p, size_t bytes) {
+    cudaError_t e = inject_alloc_failure() ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
     const int fill = g_fill_alloc.load();
     if (e == cudaSuccess && fill >= 0) {
         cudaMemset(*p, fill, bytes);
@@ -480,7 +484,7 @@ void drop_graphs(mb_ctx* c) {
 }
 
 std::mutex g_tune_mu;
-std::map<std::tuple<int, int, int, int>, TuneSet> g_tune_cache;
+std::map<TuneKey, TuneSet> g_tune_cache;
 
 }  // namespace mbi
 
@@ -775,12 +779,12 @@ static int create_ctx(mb_ctx** out, const int grid[3], int gnz, int kz0, int own
     c->px = c->nx;
     // rows of whole 16-byte words, which the single-pass step's tensor maps
     // need (139^3: 95.6 us a step against 103 for the two passes), where the
-    // added cells are few (at most a sixteenth; below 48 cells a row they may
-    // be more) and memory for that step's second copy of the state is left
+    // added cells are at most a sixteenth of the row (every n_x of 48 and more,
+    // some below) and memory for that step's second copy of the state is left
     const int px = (c->nx + 3) / 4 * 4;
     const int64_t pcell = (int64_t)px * c->ny * c->nz;
     size_t mem_free = 0, mem_total = 0;
-    if (px != c->nx && (px - c->nx) * 16 <= c->nx && pcell < (int64_t(1) << 32) &&
+    if (px != c->nx && (px - c->nx) * 16 <= c->nx && pcell < (int64_t(1) << 32) && !inject_alloc_failure() &&
         cudaMemGetInfo(&mem_free, &mem_total) == cudaSuccess && 2 * sizeof(float) * 15 * (size_t)pcell <= mem_free)
         c->px = px;
     c->pcell = (int64_t)c->px * c->ny * c->nz;
@@ -885,7 +889,7 @@ static int create_ctx(mb_ctx** out, const int grid[3], int gnz, int kz0, int own
     gain_coefficients(c);
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
-        auto it = g_tune_cache.find({c->nx, c->ny, c->nz, L});
+        auto it = g_tune_cache.find(tune_key(c));
         if (it != g_tune_cache.end()) {
             c->tune_h = it->second.h;
             c->tune_e = it->second.e;

@@ -418,13 +418,13 @@ int mb_batch_autotune(mb_batch* b) {
     // single-pass instance ends in the copy it started from.
     int rc = MB_OK;
     {
-        std::map<std::tuple<int, int, int>, mb_ctx*> tuned;   // one trial set per grid shape
+        std::map<std::tuple<int, int, int, int>, mb_ctx*> tuned;   // one trial set per grid shape and row length
         for (mb_ctx* c : b->inst) {
             if (rc) break;
-            auto it = tuned.find({c->nx, c->ny, c->nz});
+            auto it = tuned.find({c->nx, c->ny, c->nz, c->px});
             if (it == tuned.end()) {
                 if ((rc = mb_autotune(c))) rc = bfail(b, rc, mb_last_error(c));
-                tuned[{c->nx, c->ny, c->nz}] = c;
+                tuned[{c->nx, c->ny, c->nz, c->px}] = c;
             } else {
                 const mb_ctx* t = it->second;
                 c->tune_h = t->tune_h;

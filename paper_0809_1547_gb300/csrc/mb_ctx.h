@@ -90,12 +90,15 @@ bool has_probes(const mb_ctx* c);
 int launches_per_step(const mb_ctx* c, bool fused = false);
 void drop_graphs(mb_ctx* c);
 
-// Launch shapes chosen per grid shape and CPML depth in this process.
+// Launch shapes chosen per grid shape, row length (rows of one shape are
+// padded or not, by the memory left) and CPML depth in this process.
 struct TuneSet {
     mb::PassTune h, e, f;
     bool fused;
 };
 extern std::mutex g_tune_mu;
-extern std::map<std::tuple<int, int, int, int>, TuneSet> g_tune_cache;
+using TuneKey = std::tuple<int, int, int, int, int>;
+inline TuneKey tune_key(const mb_ctx* c) { return {c->nx, c->ny, c->nz, c->px, c->p.npml}; }
+extern std::map<TuneKey, TuneSet> g_tune_cache;
 
 }  // namespace mbi

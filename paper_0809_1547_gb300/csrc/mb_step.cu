@@ -629,7 +629,7 @@ int mb_autotune(mb_ctx* c) {
     c->use_fused = fused;
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
-        g_tune_cache[{c->nx, c->ny, c->nz, c->p.npml}] = TuneSet{bh, be, bf, fused};
+        g_tune_cache[tune_key(c)] = TuneSet{bh, be, bf, fused};
     }
     drop_graphs(c);
     return MB_OK;
