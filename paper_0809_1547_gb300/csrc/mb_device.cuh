@@ -450,11 +450,6 @@ __device__ __forceinline__ void h_core(const StepArgs& a, int i, int j, int k, u
     f.hz[c] = hz;
 }
 
-__device__ __forceinline__ void h_update_cell(const StepArgs& a, int i, int j, int k) {
-    const uint32_t c = cell_place(a.g, i, j, k);
-    h_core<true>(a, i, j, k, c, load_e_nbrs(a, i, j, k, c));
-}
-
 // Soft current J_src,s at t = (n + 1/2) dt.
 __device__ __forceinline__ float source_value(const DevSource& s, long long n) {
     const long long q = n - s.n0;
@@ -606,26 +601,6 @@ __device__ __forceinline__ void flux_terms(const DevFlux& F, int i, int j, int k
     }
 }
 
-// ------------------------------------------------- Lorentz step, gain cells
-// J^{n+1/2} and P^{n+1} of gain cell c with the Langevin force of step n.
-// It reads only time-n state (E^n, P^n, J^{n-1/2}, N^n), so it runs in the
-// H half-step launch, before the E pass overwrites E.
-__device__ __forceinline__ void gain_cell_step(const StepArgs& a, uint32_t c, long long n) {
-    const DevFields& f = a.f;
-    const float ex0 = __ldg(f.ex + c), ey0 = __ldg(f.ey + c), ez0 = __ldg(f.ez + c);
-    float* g = f.gs + gain_place(c);
-    const float n1 = g[kN1], n2 = g[kN2];
-    float px = g[kPx], py = g[kPy], pz = g[kPz];
-    float jx = g[kJx], jy = g[kJy], jz = g[kJz];
-    lorentz_step(a.gain, c, n, ex0, ey0, ez0, n1, n2, jx, jy, jz, px, py, pz);
-    g[kJx] = jx;
-    g[kJy] = jy;
-    g[kJz] = jz;
-    g[kPx] = px;
-    g[kPy] = py;
-    g[kPz] = pz;
-}
-
 // ------------------------------------------------ E / population pass
 // One cell, after the gain cells' Lorentz step of this time step: E^{n+1}
 // with the current J^{n+1/2}, then N^{n+1}; with FLUX, the face-flux terms.
@@ -717,13 +692,6 @@ __device__ __forceinline__ void e_core(const StepArgs& a, int i, int j, int k, u
     }
     e_apply<FLUX, PML, KEEP>(a, i, j, k, c, h, m, ex0, ey0, ez0, gain, jx, jy, jz, n1, n2, n3, n, fl,
                        flux_plane);
-}
-
-template <bool FLUX>
-__device__ __forceinline__ void e_update_cell(const StepArgs& a, int i, int j, int k,
-                                              long long n, float fl[6]) {
-    const uint32_t c = cell_place(a.g, i, j, k);
-    e_core<FLUX, true>(a, i, j, k, c, load_h_nbrs(a, i, j, k, c), n, fl);
 }
 
 // Warp-level flux reduction: FP32 sums within the warp (skipped for faces
