@@ -898,6 +898,14 @@ static int create_ctx(mb_ctx** out, const int grid[3], int gnz, int kz0, int own
         } else if (ncell < mb::kSmallPassCells) {
             c->tune_h = mb::PassTune{mb::kVariant3D, dim3(64, 4, 1), 1};
             c->tune_e = mb::PassTune{mb::kVariantZmarch, dim3(32, 4, 1), mb::kSmallPassPlanes};
+        } else {
+            const bool tma = mb::tma_e_supported(c->args);
+            const dim3 b(32, 4, 1);
+            c->tune_h = tma && ncell >= mb::kTmaPassCellsH ? mb::PassTune{mb::kVariantTma, b, 8}
+                                                           : mb::PassTune{mb::kVariantZmarch, b, 4};
+            c->tune_e = tma && ncell >= mb::kTmaPassCellsE
+                            ? mb::PassTune{mb::kVariantTma, b, 8}
+                            : mb::PassTune{mb::kVariantZmarch, b, ncell < mb::kLongWalkCells ? 8 : 16};
         }
     }
     *out = c;

@@ -110,6 +110,19 @@ struct PassTune {
 // 48^3; at 96^3 the longer walks are the faster).
 constexpr int64_t kSmallPassCells = 400000;
 constexpr int kSmallPassPlanes = 4;
+// The default shapes of larger grids, H pass then E pass (an untuned context
+// steps with them; a tuned one of such a size takes the single-pass step).
+// Walks of 4 planes in H and 8 in E (16 from 8 M cells on: E of 6.7 M cells 136
+// against 144 us, of 27.8 M 462 against 454); on rows of a multiple of 16 cells
+// the planes staged by tensor copies, E from about 4 M cells on (160^3 74
+// against 84, 320^3 431 against 500), H from 6 M (192^3 110 against 111, 320^3
+// 466 against 505).  Both passes, us a step of chunks: 96^3 29, 139^3 106,
+// 255 x 250 x 200 406, 320^3 888, 331 x 300 x 280 885.  With an array per gain
+// component and walks of 16 planes they took 43, 115, 399, 961 and 835: the
+// blocks of eight cells cost the gain part of H more lines a request and longer
+// latencies (331 x 300 x 280: 409 -> 455 at the same shape), which the shapes
+// make up for except on the largest grids without tensor copies.
+constexpr int64_t kTmaPassCellsE = 4000000, kTmaPassCellsH = 6000000, kLongWalkCells = 8000000;
 
 // Polls of a bounded mbarrier wait before the kernel gives up (~0.1-1 s).
 constexpr int kWaitLimit = 1 << 20;

@@ -523,13 +523,6 @@ void launch_rows(const void* src, int from, void* dst, int to, int nx, int64_t c
         k_rows<uint8_t><<<blocks, 256, 0, s>>>((const uint8_t*)src, from, (uint8_t*)dst, to, nx, count);
 }
 
-// A load that asks L2 for 64 bytes around the address instead of the 128 that
-// a plain load brings from HBM here.
-__device__ __forceinline__ float load_64(const float* p) {
-    float v;
-    asm volatile("ld.global.L2::64B.f32 %0, [%1];" : "=f"(v) : "l"(p));
-    return v;
-}
 // One component of P, J or the populations (its place comp floats into the
 // blocks) to (OUT) or from the packed array, a row a warp.  Bound by memory:
 // a block's eight values are 32 bytes of 288, of which HBM reads 64 at least,

@@ -338,12 +338,12 @@ __global__ void __launch_bounds__(BX * BY) k_e_tma(StepArgs a, const __grid_cons
     auto gslot = [&](int b, int q) -> float* { return gbuf + (b * 6 + q) * (BX * BY) + tid; };
     auto prefetch_gain = [&](int b, uint32_t cc) {
         const float* g = f.gs + gain_place(cc);
-        cp_async_4(gslot(b, 0), g + kJx);
-        cp_async_4(gslot(b, 1), g + kJy);
-        cp_async_4(gslot(b, 2), g + kJz);
-        cp_async_4(gslot(b, 3), g + kN1);
-        cp_async_4(gslot(b, 4), g + kN2);
-        cp_async_4(gslot(b, 5), g + kN3);
+        cp_async_4_64(gslot(b, 0), g + kJx);
+        cp_async_4_64(gslot(b, 1), g + kJy);
+        cp_async_4_64(gslot(b, 2), g + kJz);
+        cp_async_4_64(gslot(b, 3), g + kN1);
+        cp_async_4_64(gslot(b, 4), g + kN2);
+        cp_async_4_64(gslot(b, 5), g + kN3);
     };
 
     if (tid == 0) {

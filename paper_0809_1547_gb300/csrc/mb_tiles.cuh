@@ -36,13 +36,14 @@ __device__ __forceinline__ void gain_block(const StepArgs& a, unsigned gidx, int
     const int T = blockDim.x * blockDim.y * blockDim.z;
     const uint32_t base = gidx * (uint32_t)q + (uint32_t)linear_tid();
     const DevFields& f = a.f;
-    uint32_t cs[PER];
+    uint32_t cs[PER], nums[PER];
     bool ok[PER];
 #pragma unroll
     for (int r = 0; r < PER; ++r) {
         const uint32_t e = base + (uint32_t)(r * T);
         ok[r] = e < a.glist.count;
         cs[r] = ok[r] ? __ldg(a.glist.cell + e) : 0u;
+        nums[r] = a.glist.number ? (ok[r] ? __ldg(a.glist.number + e) : 0u) : cs[r];
     }
     float ex[PER], ey[PER], ez[PER], n1[PER],
         n2[PER], px[PER], py[PER], pz[PER],
@@ -68,8 +69,7 @@ __device__ __forceinline__ void gain_block(const StepArgs& a, unsigned gidx, int
     for (int r = 0; r < PER; ++r) {
         if (!ok[r]) continue;
         const uint32_t c = cs[r];
-        const uint32_t num = a.glist.number ? __ldg(a.glist.number + base + (uint32_t)(r * T)) : c;
-        lorentz_step(a.gain, num, n, ex[r], ey[r], ez[r], n1[r], n2[r], jx[r], jy[r], jz[r], px[r],
+        lorentz_step(a.gain, nums[r], n, ex[r], ey[r], ez[r], n1[r], n2[r], jx[r], jy[r], jz[r], px[r],
                      py[r], pz[r]);
         float* g = f.gs + gain_place(c);
         g[kJx] = jx[r];

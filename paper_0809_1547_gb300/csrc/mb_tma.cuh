@@ -114,6 +114,12 @@ __device__ __forceinline__ void cp_async_4(void* dst, const void* src) {
                  : "memory");
 }
 
+// The same, L2 asking HBM for 64 bytes (load_64).
+__device__ __forceinline__ void cp_async_4_64(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global.L2::64B [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src)
+                 : "memory");
+}
+
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
