@@ -488,12 +488,20 @@ int mb_autotune(mb_ctx* c) {
         }
     }
     std::vector<mb::PassTune> cands;
-    for (dim3 b : {dim3(32, 4, 2), dim3(32, 8, 1), dim3(64, 4, 1), dim3(32, 2, 4), dim3(128, 2, 1),
-                   dim3(32, 4, 4), dim3(64, 2, 2)})
-        cands.push_back({mb::kVariant3D, b, 1});
+    // from 4 M cells on a cell per thread (H at least 4 % behind, E 37 %), rows of
+    // 128 threads and more and tiles of 512 threads (H 4 to 18 %, E 1 to 35 %)
+    // never came first at 157 x 160 x 170 to 331 x 300 x 280, 64 x 400 x 400 and
+    // 500 x 400 x 50, and each costs the trial as long as steps do
+    const bool large = c->ncell > 4000000;
+    if (!large)
+        for (dim3 b : {dim3(32, 4, 2), dim3(32, 8, 1), dim3(64, 4, 1), dim3(32, 2, 4), dim3(128, 2, 1),
+                       dim3(32, 4, 4), dim3(64, 2, 2)})
+            cands.push_back({mb::kVariant3D, b, 1});
     for (dim3 b : {dim3(32, 4, 1), dim3(32, 8, 1), dim3(64, 4, 1), dim3(64, 2, 1), dim3(128, 2, 1),
-                   dim3(32, 16, 1), dim3(64, 8, 1), dim3(128, 4, 1), dim3(256, 1, 1)})
+                   dim3(32, 16, 1), dim3(64, 8, 1), dim3(128, 4, 1), dim3(256, 1, 1)}) {
+        if (large && (b.x > 64 || b.x * b.y > 256)) continue;
         for (int kz : {4, 8, 16, 32}) cands.push_back({mb::kVariantZmarch, b, kz});
+    }
     if (mb::vec_supported(c->args))
         for (dim3 b : {dim3(32, 2, 1), dim3(32, 4, 1), dim3(32, 8, 1), dim3(64, 2, 1), dim3(64, 4, 1),
                        dim3(128, 2, 1)})
@@ -507,10 +515,10 @@ int mb_autotune(mb_ctx* c) {
     cudaEventCreate(&e1);
     float best_h = 1e30f, best_e = 1e30f;
     mb::PassTune bh = c->tune_h, be = c->tune_e;
-    const int reps = c->ncell > 4000000 ? 2 : 6;
+    const int reps = large ? 2 : 6;
     // every shape by a launch or two, then the four fastest again, longer and
     // twice interleaved
-    const int coarse = c->ncell > 4000000 ? 1 : 2;
+    const int coarse = large ? 1 : 2;
     for (int pass = 0; pass < 2; ++pass) {
         auto time_pass = [&](const mb::PassTune& t, int n) -> float {
             const mb::TmaMaps* m = tma_for(c, t);
