@@ -443,9 +443,10 @@ int mb_batch_step(mb_batch* batch, int n);
 int mb_batch_synchronize(mb_batch* batch);
 
 /* Time the candidate tile shapes of the persistent kernel, tune each
- * instance's own launches (mb_autotune), time the two modes over a few
- * steps (states are saved and restored around every trial) and keep the
- * fastest shape and mode. */
+ * instance's own launches (mb_autotune; launches of many steps a launch are
+ * kept where they are the faster with all instances running), time the two
+ * modes over a few steps (states are saved and restored around every trial)
+ * and keep the fastest shape and mode. */
 int mb_batch_autotune(mb_batch* batch);
 
 #define MB_BATCH_PERSISTENT 0

@@ -4,6 +4,7 @@
 #include "mb_ctx.h"
 
 #include <algorithm>
+#include <cmath>
 #include <map>
 #include <string>
 #include <tuple>
@@ -240,6 +241,9 @@ int mb_batch_create(mb_batch** out, int B, const int* grids, double dx, double d
         mb_ctx* c = nullptr;
         int rc = mb_create(&c, grids + 3 * q, dx, dt, p, b->stream);
         if (rc) return bail(rc);
+        // a launch of many steps that a lone context of this grid was tuned to
+        // fills the GPU by itself: not beside other members untried
+        if (c->tune_f.variant == mb::kVariantSmall) c->use_fused = false;
         b->inst.push_back(c);
     }
     int64_t largest = 0;
@@ -414,7 +418,7 @@ int mb_batch_autotune(mb_batch* b) {
     b->kz = pick.kz;
     // The instances' own launch shapes (tuned once per grid shape and CPML
     // depth in the process), then each mode from the same state: a warm-up
-    // of 2 steps (graph captures) and 4 timed steps; even counts, so a
+    // of 2 steps (graph captures) and the timed steps; even counts, so a
     // single-pass instance ends in the copy it started from.
     int rc = MB_OK;
     {
@@ -440,6 +444,51 @@ int mb_batch_autotune(mb_batch* b) {
         n_keep.push_back(c->n);
         l_keep.push_back(c->launches);
     }
+    // ms of a call of n steps of the members' own launches, after one untimed
+    auto concurrent_ms = [&](int n) -> float {
+        float ms = 1e30f;
+        restore_all();
+        if (step_concurrent(b, n) == MB_OK && cudaEventRecord(e0, b->stream) == cudaSuccess &&
+            step_concurrent(b, n) == MB_OK && cudaEventRecord(e1, b->stream) == cudaSuccess &&
+            cudaEventSynchronize(e1) == cudaSuccess)
+            cudaEventElapsedTime(&ms, e0, e1);
+        return ms;
+    };
+    // Members tuned (alone) to many steps a launch: such a launch holds most of
+    // the GPU's shared memory, so that two members' launches run one after the
+    // other, where their two passes run beside each other (sides 48, 52 and 60:
+    // 26.7 us a step against 22.4; 24, 28 and 30: 4.7 against 10.1).  Both are
+    // timed with all members running, in calls of 4 and of 32 steps; the launch
+    // stays where a step of it is the shorter, for calls long enough to repay
+    // the members' loading and storing of their states.
+    std::vector<mb_ctx*> many;
+    for (mb_ctx* c : b->inst)
+        if (rc == MB_OK && c->use_fused && c->tune_f.variant == mb::kVariantSmall) many.push_back(c);
+    bool kept = false;
+    if (!many.empty()) {
+        float t[2][2];   // [launch of many steps][calls of 4, of 32 steps]
+        for (int on = 1; on >= 0; --on) {
+            for (mb_ctx* c : many) {
+                c->use_fused = on != 0;
+                mbi::drop_graphs(c);
+            }
+            for (int q = 0; q < 2; ++q) t[on][q] = std::min(concurrent_ms(q ? 32 : 4), concurrent_ms(q ? 32 : 4));
+        }
+        const float step1 = (t[1][1] - t[1][0]) / 28.0f, step0 = (t[0][1] - t[0][0]) / 28.0f;
+        if (step1 < 0.97f * step0) {
+            const float fixed = (t[1][0] - 4.0f * step1) - (t[0][0] - 4.0f * step0);
+            const int least = (int)std::ceil(std::max(fixed, 0.0f) / (step0 - step1));
+            kept = least <= mb::kSmallMaxSteps;
+            for (mb_ctx* c : many) {
+                c->use_fused = kept;
+                c->tune_f.kz = std::max(c->tune_f.kz, std::max(least, 1));
+                mbi::drop_graphs(c);
+            }
+        }
+    }
+    // each mode over calls of 4 steps, of 32 where the members take the launch
+    // of many (a few microseconds a step)
+    const int n_mode = kept ? 32 : 4;
     float t_mode[2] = {1e30f, 1e30f};
     for (int m = 0; m < 2 && rc == MB_OK; ++m) {
         restore_all();
@@ -449,10 +498,10 @@ int mb_batch_autotune(mb_batch* b) {
                  cudaMemcpyAsync(b->d_ctr, &n0, sizeof(long long), cudaMemcpyHostToDevice, b->stream) ==
                      cudaSuccess &&
                  launch_steps(b, 2) == MB_OK && cudaEventRecord(e0, b->stream) == cudaSuccess &&
-                 launch_steps(b, 4) == MB_OK;
+                 launch_steps(b, n_mode) == MB_OK;
         } else {
             ok = step_concurrent(b, 2) == MB_OK && cudaEventRecord(e0, b->stream) == cudaSuccess &&
-                 step_concurrent(b, 4) == MB_OK;
+                 step_concurrent(b, n_mode) == MB_OK;
         }
         if (ok && cudaEventRecord(e1, b->stream) == cudaSuccess && cudaEventSynchronize(e1) == cudaSuccess)
             cudaEventElapsedTime(&t_mode[m], e0, e1);

@@ -10,7 +10,7 @@ from parity_util import DT, DX
 pytestmark = pytest.mark.gpu
 
 STATE = ("Ex", "Ey", "Ez", "Hx", "Hy", "Hz", "Px", "Jy", "N1", "N2", "N3")
-GRIDS = [(48, 20, 18), (51, 19, 23), (33, 26, 20)]
+GRIDS = [(48, 21, 19), (51, 19, 23), (33, 27, 20)]   # (sizes no other test uses: tuned here)
 
 
 def _batch(tuned):
@@ -60,4 +60,36 @@ def test_adjoint_on_a_member_between_calls():
         for f in STATE:
             np.testing.assert_array_equal(a.instances[q].field(f), r.instances[q].field(f), err_msg=f"{q} {f}")
     for b in (a, r):
+        b.close()
+
+
+@pytest.mark.parametrize("grids", [[(24, 23, 21), (28, 25, 24)], [(48, 40, 44), (51, 47, 40), (40, 44, 36)]])
+def test_autotuned_small_members(grids):
+    """The trials of a batch of small grids (many steps a launch or two passes,
+    all members running) leave the states, and what they pick steps the same."""
+    from paper_0809_1547_gb300 import inputs
+    from paper_0809_1547_gb300.binding import MB_BATCH_CONCURRENT, MBBatch, mb_default_params
+    out = []
+    for tuned in (True, False):
+        b = MBBatch(grids, DX, DT, mb_default_params(npml=4))
+        for q, grid in enumerate(grids):
+            eps, gain = inputs.random_small(grid, seed=q, npml=4, d_cells=4.0)
+            b.set_instance(q, eps, gain, 4e24, 1e13, 40 + q)
+            b.instances[q].set_source((9, 9, 9), 2, 532e-9, 1.0e-15, 0.4e-15, 1e9)
+            b.instances[q].add_point_probe((9, 9, 10), 9, 480e-9, 700e-9)
+        b.step(5)
+        if tuned:
+            b.autotune()
+            b.set_mode(MB_BATCH_CONCURRENT)
+        for n in (1, 3, 64, 33):
+            b.step(n)
+        b.synchronize()
+        out.append(b)
+    a, r = out
+    for q in range(len(grids)):
+        assert a.instances[q].n == r.instances[q].n == 106
+        for f in STATE:
+            np.testing.assert_array_equal(a.instances[q].field(f), r.instances[q].field(f), err_msg=f"{q} {f}")
+        np.testing.assert_array_equal(a.instances[q].probe_spectrum(0)[0], r.instances[q].probe_spectrum(0)[0])
+    for b in out:
         b.close()
