@@ -113,12 +113,8 @@ size_t gain_offset(const mb_ctx* c) { return (6 * (size_t)c->pcell + 63) / 64 * 
 // An E or H array of the current copy.
 float* eh_ptr(mb_ctx* c, int which) { return eh_of(c, c->parity) + (int64_t)which * c->pcell; }
 
-// Where a field of P, J or the populations sits in the gain blocks.
-int gain_comp(int which) {
-    if (which <= MB_PZ) return mb::kPx + (which - MB_PX) * mb::kGainCells;
-    if (which <= MB_JZ) return mb::kJx + (which - MB_JX) * mb::kGainCells;
-    return mb::kN1 + (which - MB_N1) * mb::kGainCells;
-}
+// The number of a field of P, J or the populations in blob order.
+int gain_field(int which) { return which < MB_N0 ? which - MB_PX : which - MB_N1 + 6; }
 
 // Points the step arguments' E, H and CPML memories at copy p.
 void point_args_at(mb::StepArgs& a, const mb_ctx* c, int p) {
@@ -303,23 +299,30 @@ size_t host_bytes(const mb_ctx* c, const StatePart& p) {
     return p.arrays ? sizeof(float) * (size_t)p.arrays * c->ncell : p.bytes;
 }
 
-// Where fields cross packed between host and device, an array at a time: the
-// material's upload buffer (made here where no material is set yet) or, where
-// the device has no memory left for it, page-locked host memory, which the
-// kernels reach as well; null where neither can be had.
-uint8_t* staging(mb_ctx* c) {
-    if (c->d_upload) return c->d_upload;
-    const size_t bytes = 5 * (size_t)c->ncell + 16;
-    if (device_malloc((void**)&c->d_upload, bytes) == cudaSuccess) {
-        c->upload_bytes = bytes;
+// Where fields cross packed between host and device: the material's upload
+// buffer (made here where no material is set yet), which holds as many fields
+// at a time as go into 16 MB, or one (a state of 24 x 22 x 20 cells saved field
+// by field takes 250 us, at once 145); where the device has no memory left for
+// it, page-locked host memory for one, which the kernels reach as well; null
+// where neither can be had.
+size_t upload_bytes(const mb_ctx* c) {
+    const size_t N = (size_t)c->ncell;
+    return std::max(5 * N + 16, std::min(15 * sizeof(float) * N, (size_t)16 << 20));
+}
+uint8_t* staging(mb_ctx* c, int& fields) {
+    const size_t field = sizeof(float) * (size_t)c->ncell;
+    if (!c->d_upload && device_malloc((void**)&c->d_upload, upload_bytes(c)) == cudaSuccess)
+        c->upload_bytes = upload_bytes(c);
+    if (c->d_upload) {
+        fields = (int)std::min<size_t>(c->upload_bytes / field, 15);
         return c->d_upload;
     }
     cudaGetLastError();
-    c->d_upload = nullptr;
-    if (!c->h_stage && cudaMallocHost((void**)&c->h_stage, sizeof(float) * (size_t)c->ncell) != cudaSuccess) {
+    if (!c->h_stage && cudaMallocHost((void**)&c->h_stage, field) != cudaSuccess) {
         cudaGetLastError();
         c->h_stage = nullptr;
     }
+    fields = 1;
     return c->h_stage;
 }
 // bytes between the staging memory and the host, after and before the
@@ -339,9 +342,9 @@ cudaError_t stage_in(mb_ctx* c, uint8_t* stage, const void* host, size_t bytes) 
 
 // Padded rows and the gain blocks are packed and spread by kernels (a 2-D
 // device copy of rows of 157 floats measured 13 us more than the plain copy;
-// the kernel as much as it).  To and from the host they cross packed, an array
-// at a time through the staging memory (2.7 M cells: a field read 1.7 ms as
-// without padding; packed on the host 2.7 ms).
+// the kernel as much as it).  To and from the host they cross packed through
+// the staging memory (2.7 M cells: a field read 1.7 ms as without padding;
+// packed on the host 2.7 ms).
 cudaError_t rows_out(mb_ctx* c, void* packed, const void* rows, size_t esize, int arrays, cudaMemcpyKind kind) {
     if (c->px == c->nx)
         return cudaMemcpyAsync(packed, rows, esize * (size_t)arrays * c->ncell, kind, c->stream);
@@ -351,11 +354,13 @@ cudaError_t rows_out(mb_ctx* c, void* packed, const void* rows, size_t esize, in
         mb::launch_rows(rows, c->px, packed, c->nx, c->nx, nrow * arrays, (int)esize, c->stream);
         return cudaGetLastError();
     }
-    uint8_t* stage = staging(c);
+    int fit = 1;
+    uint8_t* stage = staging(c, fit);
     if (!stage) return cudaErrorMemoryAllocation;
-    for (int q = 0; q < arrays; ++q) {
-        mb::launch_rows((const char*)rows + from * q, c->px, stage, c->nx, c->nx, nrow, (int)esize, c->stream);
-        cudaError_t e = stage_out(c, (char*)packed + to * q, stage, to);
+    for (int q = 0; q < arrays; q += fit) {
+        const int m = std::min(fit, arrays - q);
+        mb::launch_rows((const char*)rows + from * q, c->px, stage, c->nx, c->nx, nrow * m, (int)esize, c->stream);
+        cudaError_t e = stage_out(c, (char*)packed + to * q, stage, to * m);
         if (e != cudaSuccess) return e;
     }
     return cudaGetLastError();
@@ -369,62 +374,80 @@ cudaError_t rows_in(mb_ctx* c, void* rows, const void* packed, size_t esize, int
         mb::launch_rows(packed, c->nx, rows, c->px, c->nx, nrow * arrays, (int)esize, c->stream);
         return cudaGetLastError();
     }
-    uint8_t* stage = staging(c);
+    int fit = 1;
+    uint8_t* stage = staging(c, fit);
     if (!stage) return cudaErrorMemoryAllocation;
-    for (int q = 0; q < arrays; ++q) {
-        cudaError_t e = stage_in(c, stage, (const char*)packed + from * q, from);
+    for (int q = 0; q < arrays; q += fit) {
+        const int m = std::min(fit, arrays - q);
+        cudaError_t e = stage_in(c, stage, (const char*)packed + from * q, from * m);
         if (e != cudaSuccess) return e;
-        mb::launch_rows(stage, c->nx, (char*)rows + to * q, c->px, c->nx, nrow, (int)esize, c->stream);
+        mb::launch_rows(stage, c->nx, (char*)rows + to * q, c->px, c->nx, nrow * m, (int)esize, c->stream);
+    }
+    return cudaGetLastError();
+}
+// Fields first, .. (blob order) of P, J and the populations.
+cudaError_t gain_out(mb_ctx* c, void* packed, int first, int fields, cudaMemcpyKind kind) {
+    const int64_t nrow = (int64_t)c->ny * c->nz;
+    if (kind == cudaMemcpyDeviceToDevice) {
+        mb::launch_gain_rows(c->args.f.gs, first, fields, c->px, (float*)packed, c->nx, nrow, true, c->stream);
+        return cudaGetLastError();
+    }
+    const size_t field = sizeof(float) * (size_t)c->ncell;
+    int fit = 1;
+    uint8_t* stage = staging(c, fit);
+    if (!stage) return cudaErrorMemoryAllocation;
+    for (int q = 0; q < fields; q += fit) {
+        const int m = std::min(fit, fields - q);
+        mb::launch_gain_rows(c->args.f.gs, first + q, m, c->px, (float*)stage, c->nx, nrow, true, c->stream);
+        cudaError_t e = stage_out(c, (char*)packed + field * q, stage, field * m);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaGetLastError();
+}
+cudaError_t gain_in(mb_ctx* c, int first, int fields, const void* packed) {
+    const size_t field = sizeof(float) * (size_t)c->ncell;
+    int fit = 1;
+    uint8_t* stage = staging(c, fit);
+    if (!stage) return cudaErrorMemoryAllocation;
+    for (int q = 0; q < fields; q += fit) {
+        const int m = std::min(fit, fields - q);
+        cudaError_t e = stage_in(c, stage, (const char*)packed + field * q, field * m);
+        if (e != cudaSuccess) return e;
+        mb::launch_gain_rows(c->args.f.gs, first + q, m, c->px, (float*)stage, c->nx, (int64_t)c->ny * c->nz, false,
+                             c->stream);
     }
     return cudaGetLastError();
 }
 cudaError_t field_out(mb_ctx* c, void* packed, int which, cudaMemcpyKind kind) {
-    if (which < MB_PX) return rows_out(c, packed, eh_ptr(c, which), 4, 1, kind);
-    const bool dev = kind == cudaMemcpyDeviceToDevice;
-    uint8_t* stage = dev ? nullptr : staging(c);
-    if (!dev && !stage) return cudaErrorMemoryAllocation;
-    mb::launch_gain_rows(c->args.f.gs, gain_comp(which), c->px, dev ? (float*)packed : (float*)stage, c->nx,
-                         (int64_t)c->ny * c->nz, true, c->stream);
-    const cudaError_t e = dev ? cudaSuccess : stage_out(c, packed, stage, sizeof(float) * (size_t)c->ncell);
-    return e != cudaSuccess ? e : cudaGetLastError();
-}
-cudaError_t field_in(mb_ctx* c, int which, const void* packed, cudaMemcpyKind kind) {
-    if (which < MB_PX) return rows_in(c, eh_ptr(c, which), packed, 4, 1, kind);
-    uint8_t* stage = staging(c);
-    if (!stage) return cudaErrorMemoryAllocation;
-    cudaError_t e = stage_in(c, stage, packed, sizeof(float) * (size_t)c->ncell);
-    if (e != cudaSuccess) return e;
-    mb::launch_gain_rows(c->args.f.gs, gain_comp(which), c->px, (float*)stage, c->nx, (int64_t)c->ny * c->nz, false,
-                         c->stream);
-    return cudaGetLastError();
+    return which < MB_PX ? rows_out(c, packed, eh_ptr(c, which), 4, 1, kind)
+                         : gain_out(c, packed, gain_field(which), 1, kind);
 }
 // Can a kernel of this context store `bytes` of floats at p: memory of its own
 // device, aligned, inside one allocation?  A copy takes any address and turns
 // a bad one into an error; a store there would fault.
 bool kernel_writes(const mb_ctx* c, const float* p, size_t bytes) {
-    using RangeFn = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
-    static const RangeFn range = []() -> RangeFn {
+    using AttrFn = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+    static const AttrFn attributes = []() -> AttrFn {
         void* f = nullptr;
         cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
             q == cudaDriverEntryPointSuccess)
-            return (RangeFn)f;
+            return (AttrFn)f;
         cudaGetLastError();
         return nullptr;
     }();
-    cudaPointerAttributes at{};
-    if (!range || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
+    unsigned type = 0;
+    int device = -1;
     CUdeviceptr base = 0;
     size_t size = 0;
-    return (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) && at.device == c->device &&
-           (uintptr_t)p % sizeof(float) == 0 && range(&base, &size, (CUdeviceptr)p) == CUDA_SUCCESS &&
-           (CUdeviceptr)p + bytes <= base + size;
+    CUpointer_attribute what[4] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL,
+                                   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* value[4] = {&type, &device, &base, &size};
+    return (uintptr_t)p % sizeof(float) == 0 && attributes &&
+           attributes(4, what, value, (CUdeviceptr)p) == CUDA_SUCCESS && type == CU_MEMORYTYPE_DEVICE &&
+           device == c->device && (CUdeviceptr)p >= base && (CUdeviceptr)p - base <= size &&
+           bytes <= size - ((CUdeviceptr)p - base);
 }
-// The gain fields in blob order.
-constexpr int kGainFields[9] = {MB_PX, MB_PY, MB_PZ, MB_JX, MB_JY, MB_JZ, MB_N1, MB_N2, MB_N3};
 
 // Tensor maps for a TMA tuning over the current copy (encoded once per tile
 // shape and copy), else nullptr.
@@ -1005,9 +1028,8 @@ int mb_set_material(mb_ctx* c, const float* eps_map, const uint8_t* gain_mask, d
         return true;
     };
     const bool rows = c->px != c->nx;
-    const size_t up_bytes = 5 * (size_t)N + 16;
     const size_t key_bytes = 2 * sizeof(uint32_t) * mb::kMatKeys + 2 * sizeof(int);
-    if (!grow((void**)&c->d_upload, c->upload_bytes, up_bytes) ||
+    if (!grow((void**)&c->d_upload, c->upload_bytes, upload_bytes(c)) ||
         !grow((void**)&c->d_keys, c->keys_bytes, key_bytes))
         return fail(c, MB_ERR_OOM, "material map scratch allocation failed");
     float* d_eps = reinterpret_cast<float*>(c->d_upload);
@@ -1582,7 +1604,6 @@ int mb_get_material(mb_ctx* c, uint8_t* host_out) {
     if (int rc = check_ctx(c)) return rc;
     if (!host_out) return fail(c, MB_ERR_ARG, "null output");
     if (!c->have_material) return fail(c, MB_ERR_STATE, "no material set");
-    MB_CUDA(c, cudaStreamSynchronize(c->stream));
     MB_CUDA(c, rows_out(c, host_out, c->d_mat, 1, 1, cudaMemcpyDeviceToHost));
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
     return MB_OK;
@@ -1611,20 +1632,17 @@ int mb_get_field(mb_ctx* c, int which, float* host_out) {
     if (int rc = check_ctx(c)) return rc;
     if (!host_out || which < 0 || which >= MB_NUM_FIELDS) return fail(c, MB_ERR_ARG, "bad field id or null output");
     const int64_t N = c->ncell;
-    std::vector<float> tmp((size_t)N);
     if (which == MB_N0) {
-        std::vector<float> a((size_t)N), b((size_t)N), d((size_t)N);
-        std::vector<uint8_t> m((size_t)N, 0);
-        MB_CUDA(c, field_out(c, a.data(), MB_N1, cudaMemcpyDeviceToHost));
-        MB_CUDA(c, field_out(c, b.data(), MB_N2, cudaMemcpyDeviceToHost));
-        MB_CUDA(c, field_out(c, d.data(), MB_N3, cudaMemcpyDeviceToHost));
-        if (c->have_material)
-            MB_CUDA(c, rows_out(c, m.data(), c->d_mat, 1, 1, cudaMemcpyDeviceToHost));
+        int fit = 1;
+        uint8_t* stage = staging(c, fit);
+        if (!stage) return fail(c, MB_ERR_OOM, "no memory for the packed field");
+        mb::launch_n0(c->args.f.gs, c->d_mat, c->px, (float*)stage, c->nx, (int64_t)c->ny * c->nz, c->N_a, c->stream);
+        MB_CUDA(c, cudaGetLastError());
+        MB_CUDA(c, stage_out(c, host_out, stage, sizeof(float) * (size_t)N));
         MB_CUDA(c, cudaStreamSynchronize(c->stream));
-        for (int64_t q = 0; q < N; ++q)
-            host_out[q] = (m[q] & 0x80) ? (float)(c->N_a * (1.0 - (double)a[q] - (double)b[q] - (double)d[q])) : 0.0f;
         return MB_OK;
     }
+    std::vector<float> tmp((size_t)N);
     MB_CUDA(c, field_out(c, tmp.data(), which, cudaMemcpyDeviceToHost));
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
     const double s = field_scale(c, which);
@@ -1641,8 +1659,13 @@ int mb_set_field(mb_ctx* c, int which, const float* host_in) {
     const double s = 1.0 / field_scale(c, which);
     std::vector<float> tmp((size_t)N);
     for (int64_t q = 0; q < N; ++q) tmp[q] = (float)(s * (double)host_in[q]);
-    MB_CUDA(c, cudaStreamSynchronize(c->stream));
-    MB_CUDA(c, field_in(c, which, tmp.data(), cudaMemcpyHostToDevice));
+    if (which < MB_PX && c->px == c->nx) {
+        MB_CUDA(c, cudaStreamSynchronize(c->stream));
+        MB_CUDA(c, cudaMemcpy(eh_ptr(c, which), tmp.data(), sizeof(float) * (size_t)N, cudaMemcpyHostToDevice));
+        return MB_OK;
+    }
+    if (which < MB_PX) MB_CUDA(c, rows_in(c, eh_ptr(c, which), tmp.data(), 4, 1, cudaMemcpyHostToDevice));
+    else MB_CUDA(c, gain_in(c, gain_field(which), 1, tmp.data()));
     MB_CUDA(c, cudaStreamSynchronize(c->stream));
     return MB_OK;
 }
@@ -1655,7 +1678,8 @@ int mb_get_field_device(mb_ctx* c, int which, float* dev_out, double* scale) {
     if ((which < MB_PX && c->px == c->nx) || kernel_writes(c, dev_out, bytes)) {
         MB_CUDA(c, field_out(c, dev_out, which, cudaMemcpyDeviceToDevice));
     } else {
-        uint8_t* stage = staging(c);
+        int fit = 1;
+        uint8_t* stage = staging(c, fit);
         if (!stage) return fail(c, MB_ERR_OOM, "no memory for the packed field");
         MB_CUDA(c, field_out(c, stage, which, cudaMemcpyDeviceToDevice));
         MB_CUDA(c, cudaMemcpyAsync(dev_out, stage, bytes,
@@ -1682,9 +1706,7 @@ int mb_save_state(mb_ctx* c, void* host_blob, size_t* bytes) {
     std::memcpy(o, hdr, sizeof(hdr));
     o += sizeof(hdr);
     for (auto& p : parts) {
-        if (p.gain)
-            for (int q = 0; q < 9; ++q)
-                MB_CUDA(c, field_out(c, o + sizeof(float) * (size_t)c->ncell * q, kGainFields[q], cudaMemcpyDeviceToHost));
+        if (p.gain) MB_CUDA(c, gain_out(c, o, 0, 9, cudaMemcpyDeviceToHost));
         else if (p.arrays) MB_CUDA(c, rows_out(c, o, p.ptr, 4, p.arrays, cudaMemcpyDeviceToHost));
         else MB_CUDA(c, cudaMemcpyAsync(o, p.ptr, p.bytes, cudaMemcpyDeviceToHost, c->stream));
         o += host_bytes(c, p);
@@ -1704,11 +1726,8 @@ int mb_load_state(mb_ctx* c, const void* host_blob, size_t bytes) {
     if (bytes != total || hdr[0] != 0x4D42464454445331LL || hdr[1] != c->ncell || hdr[2] != (int64_t)parts.size())
         return fail(c, MB_ERR_ARG, "blob does not match this context's layout");
     const char* o = (const char*)host_blob + 4 * sizeof(int64_t);
-    MB_CUDA(c, cudaStreamSynchronize(c->stream));
     for (auto& p : parts) {
-        if (p.gain)
-            for (int q = 0; q < 9; ++q)
-                MB_CUDA(c, field_in(c, kGainFields[q], o + sizeof(float) * (size_t)c->ncell * q, cudaMemcpyHostToDevice));
+        if (p.gain) MB_CUDA(c, gain_in(c, 0, 9, o));
         else if (p.arrays) MB_CUDA(c, rows_in(c, p.ptr, o, 4, p.arrays, cudaMemcpyHostToDevice));
         else MB_CUDA(c, cudaMemcpyAsync(p.ptr, o, p.bytes, cudaMemcpyHostToDevice, c->stream));
         o += host_bytes(c, p);

@@ -72,7 +72,6 @@ size_t host_bytes(const mb_ctx* c, const StatePart& p);
 cudaError_t rows_out(mb_ctx* c, void* packed, const void* rows, size_t esize, int arrays, cudaMemcpyKind kind);
 cudaError_t rows_in(mb_ctx* c, void* rows, const void* packed, size_t esize, int arrays, cudaMemcpyKind kind);
 cudaError_t field_out(mb_ctx* c, void* packed, int which, cudaMemcpyKind kind);
-cudaError_t field_in(mb_ctx* c, int which, const void* packed, cudaMemcpyKind kind);
 // P, J and the populations: the context's blocks of them and their floats.
 size_t gain_offset(const mb_ctx* c);
 std::vector<StatePart> state_parts(mb_ctx* c);

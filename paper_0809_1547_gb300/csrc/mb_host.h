@@ -293,9 +293,12 @@ void launch_gain_numbers(const uint32_t* list, uint32_t n, int nx, int px, uint3
 // `count` rows of nx elements (1 or 4 bytes) from rows `from` elements apart
 // to rows `to` elements apart.
 void launch_rows(const void* src, int from, void* dst, int to, int nx, int64_t count, int esize, cudaStream_t s);
-// Component comp (kJx, ..) of the cells of `count` rows of nx between the gain
-// blocks (rows px cells apart) and a packed device array.
-void launch_gain_rows(float* gs, int comp, int px, float* packed, int nx, int64_t count, bool out, cudaStream_t s);
+// Fields first, .. (0: Px, .. 3: Jx, .. 6: n1, ..) of the cells of `count` rows
+// of nx between the gain blocks (rows px cells apart) and packed device arrays.
+void launch_gain_rows(float* gs, int first, int fields, int px, float* packed, int nx, int64_t count, bool out,
+                      cudaStream_t s);
+void launch_n0(const float* gs, const uint8_t* mat, int px, float* packed, int nx, int64_t count, double N_a,
+               cudaStream_t s);
 // The material map on the device: the distinct eps_r values into keys
 // (kMatKeys entries, kNoKey where unused, filled as a prefix) with the first
 // cell of each into first (initialised to kNoKey; flags[0]: a value not

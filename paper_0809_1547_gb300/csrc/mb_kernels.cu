@@ -523,15 +523,18 @@ void launch_rows(const void* src, int from, void* dst, int to, int nx, int64_t c
         k_rows<uint8_t><<<blocks, 256, 0, s>>>((const uint8_t*)src, from, (uint8_t*)dst, to, nx, count);
 }
 
-// One component of P, J or the populations (its place comp floats into the
-// blocks) to (OUT) or from the packed array, a row a warp.  Bound by memory:
-// a block's eight values are 32 bytes of 288, of which HBM reads 64 at least,
-// so a read moves 1.5 times the bytes of a copy; a plain load moved 2.5 times.
+// Fields first, first + 1, .. (blockIdx.y) of P, J and the populations, in the
+// order Px, .., Jx, .., n1, n2, n3, to (OUT) or from packed arrays one after
+// the other, a row a warp.  Bound by memory: a block's eight values are 32
+// bytes of 288, of which HBM reads 64 at least, so a read of one field moves
+// 1.5 times the bytes of a copy; a plain load moved 2.5 times.
 template <bool OUT>
-__global__ void __launch_bounds__(256) k_gain_rows(float* __restrict__ gs, int comp, int px, float* __restrict__ packed,
+__global__ void __launch_bounds__(256) k_gain_rows(float* __restrict__ gs, int first, int px, float* __restrict__ packed,
                                                    int nx, int64_t count) {
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, field = first + blockIdx.y;
+    const int comp = (field < 3 ? kPx : field < 6 ? kJx : kN1) + field % 3 * kGainCells;
     const int64_t step = (int64_t)gridDim.x * 8;
+    packed += (int64_t)blockIdx.y * nx * count;
     for (int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); r < count; r += step) {
         float* b = packed + r * nx;
         for (int i = lane; i < nx; i += 128) {
@@ -552,10 +555,30 @@ __global__ void __launch_bounds__(256) k_gain_rows(float* __restrict__ gs, int c
         }
     }
 }
-void launch_gain_rows(float* gs, int comp, int px, float* packed, int nx, int64_t count, bool out, cudaStream_t s) {
+void launch_gain_rows(float* gs, int first, int fields, int px, float* packed, int nx, int64_t count, bool out,
+                      cudaStream_t s) {
+    const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>((count + 7) / 8, 152 * 64)), fields, 1);
+    if (out) k_gain_rows<true><<<grid, 256, 0, s>>>(gs, first, px, packed, nx, count);
+    else k_gain_rows<false><<<grid, 256, 0, s>>>(gs, first, px, packed, nx, count);
+}
+
+// N0 = N_a (1 - n1 - n2 - n3) of the gain cells (0 elsewhere), packed.
+__global__ void __launch_bounds__(256) k_n0(const float* __restrict__ gs, const uint8_t* __restrict__ mat, int px,
+                                            float* __restrict__ packed, int nx, int64_t count, double N_a) {
+    const int lane = threadIdx.x & 31;
+    const int64_t step = (int64_t)gridDim.x * 8;
+    for (int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); r < count; r += step)
+        for (int i = lane; i < nx; i += 32) {
+            const uint32_t c = (uint32_t)(r * px + i);
+            const float* g = gs + gain_place(c);
+            packed[r * nx + i] =
+                (mat[c] & 0x80) ? (float)(N_a * (1.0 - (double)g[kN1] - (double)g[kN2] - (double)g[kN3])) : 0.0f;
+        }
+}
+void launch_n0(const float* gs, const uint8_t* mat, int px, float* packed, int nx, int64_t count, double N_a,
+               cudaStream_t s) {
     const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((count + 7) / 8, 152 * 64));
-    if (out) k_gain_rows<true><<<blocks, 256, 0, s>>>(gs, comp, px, packed, nx, count);
-    else k_gain_rows<false><<<blocks, 256, 0, s>>>(gs, comp, px, packed, nx, count);
+    k_n0<<<blocks, 256, 0, s>>>(gs, mat, px, packed, nx, count, N_a);
 }
 
 // ------------------------------------------------------------ material map
