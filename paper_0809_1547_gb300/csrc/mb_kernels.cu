@@ -190,7 +190,9 @@ __global__ void k_energy_final(const double* partial, int nparts, const double* 
 // Re(Ea conj(Hb) - Eb conj(Ha)) with the FP64 sums plus the FP32 sums since
 // their last flush.  On the device because the sums are 6 x 3 MB at 160^3
 // (six copies and 1.3 M host terms took 3.3 ms) and the result 1 KB.
-__global__ void __launch_bounds__(256) k_face_spectrum(DevFaceProbes fp, int face, int chunks, double* partial) {
+// With one chunk (few points) the scaled sum is the result: one launch less.
+__global__ void __launch_bounds__(256) k_face_spectrum(DevFaceProbes fp, int face, int chunks, double scale,
+                                                       double* partial) {
     __shared__ double red[8][32];
     const int K = fp.nfreq, np = fp.npts[face];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -213,7 +215,7 @@ __global__ void __launch_bounds__(256) k_face_spectrum(DevFaceProbes fp, int fac
     __syncthreads();
     if (warp == 0 && kk < K) {
         for (int w = 1; w < 8; ++w) s += red[w][lane];
-        partial[(size_t)blockIdx.y * K + kk] = s;
+        partial[(size_t)blockIdx.y * K + kk] = chunks == 1 ? s * scale : s;
     }
 }
 // out[k] = scale * sum over the chunks, in order.
@@ -313,13 +315,15 @@ void launch_plane_energy(const DevFields& f, const DevGrid& g, int k, const floa
     k_plane_energy<<<blocks, 256, 0, s>>>(f, g, k, lut_eps, u0, out);
 }
 
-int face_spectrum_chunks(int np) { return std::max(1, std::min(kFaceSpecChunks, np / 8)); }
+// (eight points a warp at least; up to 128 points by one block alone)
+int face_spectrum_chunks(int np) { return np <= 128 ? 1 : std::min(kFaceSpecChunks, np / 8); }
 
 void launch_face_spectrum(const DevFaceProbes& fp, int face, double scale, double* scratch, double* out,
                           cudaStream_t s) {
     const int chunks = face_spectrum_chunks(fp.npts[face]);
-    k_face_spectrum<<<dim3((fp.nfreq + 31) / 32, chunks, 1), 256, 0, s>>>(fp, face, chunks, scratch);
-    k_face_spectrum_sum<<<(fp.nfreq + 127) / 128, 128, 0, s>>>(scratch, chunks, fp.nfreq, scale, out);
+    k_face_spectrum<<<dim3((fp.nfreq + 31) / 32, chunks, 1), 256, 0, s>>>(fp, face, chunks, scale,
+                                                                          chunks == 1 ? out : scratch);
+    if (chunks > 1) k_face_spectrum_sum<<<(fp.nfreq + 127) / 128, 128, 0, s>>>(scratch, chunks, fp.nfreq, scale, out);
 }
 
 __global__ void k_flux_sum(const double* slots, double* out, double scale) {
