@@ -435,6 +435,7 @@ int mb_batch_autotune(mb_batch* b) {
                 c->tune_e = t->tune_e;
                 c->tune_f = t->tune_f;
                 c->use_fused = t->use_fused;
+                c->fused_ratio = t->fused_ratio;
                 mbi::drop_graphs(c);
             }
         }
@@ -485,6 +486,30 @@ int mb_batch_autotune(mb_batch* b) {
                 mbi::drop_graphs(c);
             }
         }
+    }
+    // Members tuned (alone) to the two passes by a little: beside others, whose
+    // launches fill the gaps of either, the single-pass step's fewer bytes count
+    // (sides 97, 126 and 148, four of each: 26.1 ms with the smallest on two
+    // passes, 24.1 without; alone both take 27.5 us).
+    std::vector<mb_ctx*> close;
+    for (mb_ctx* c : b->inst)
+        if (rc == MB_OK && !c->use_fused && c->tune_f.variant == mb::kVariantTma && c->fused_ratio < 1.1f &&
+            mb::fused_supported(c->args))
+            close.push_back(c);
+    if (!close.empty() && b->inst.size() > 1) {
+        float t[2];
+        for (int on = 1; on >= 0; --on) {
+            for (mb_ctx* c : close) {
+                c->use_fused = on != 0;
+                mbi::drop_graphs(c);
+            }
+            t[on] = std::min(concurrent_ms(4), concurrent_ms(4));
+        }
+        if (t[1] < t[0])
+            for (mb_ctx* c : close) {
+                c->use_fused = true;
+                mbi::drop_graphs(c);
+            }
     }
     // each mode over calls of 4 steps, of 32 where the members take the launch
     // of many (a few microseconds a step)

@@ -459,6 +459,7 @@ struct mb_ctx {
     // always points at it.  P, J and the populations have one copy.
     bool use_fused = false;
     mb::PassTune tune_f{mb::kVariantTma, dim3(32, 8, 1), 32};
+    float fused_ratio = 1e30f;         // time of the single-pass step over that of the two passes (mb_autotune)
     float* d_fields2 = nullptr;        // second copy of E, H (6 arrays)
     // the small-grid launch: its boxes (bx = 0: not available), and the flag
     // words, step base and probe samples on the device

@@ -619,6 +619,7 @@ int mb_autotune(mb_ctx* c) {
         if (small) bf = mb::PassTune{mb::kVariantSmall, dim3(32, 8, 1), std::max(1, (int)std::ceil(fixed / (other - step)))};
     }
     const bool fused = small || best_f < best_h + best_e;
+    c->fused_ratio = best_f / (best_h + best_e);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     {
