@@ -300,24 +300,29 @@ size_t host_bytes(const mb_ctx* c, const StatePart& p) {
 }
 
 // Where fields cross packed between host and device: the material's upload
-// buffer (made here where no material is set yet), which holds as many fields
-// at a time as go into 16 MB, or one (a state of 24 x 22 x 20 cells saved field
-// by field takes 250 us, at once 145); where the device has no memory left for
-// it, page-locked host memory for one, which the kernels reach as well; null
-// where neither can be had.
-size_t upload_bytes(const mb_ctx* c) {
-    const size_t N = (size_t)c->ncell;
-    return std::max(5 * N + 16, std::min(15 * sizeof(float) * N, (size_t)16 << 20));
-}
-uint8_t* staging(mb_ctx* c, int& fields) {
+// buffer (made here where no material is set yet), enlarged once for as many of
+// `want` fields as go into 16 MB (a state of 24 x 22 x 20 cells saved field by
+// field takes 250 us, at once 145; made that large with every material, an
+// autograd call that makes a context of 40 x 37 x 24 took 0.15 ms longer), and
+// where the device has no memory left for it, page-locked host memory for one
+// field, which the kernels reach as well; null where neither can be had.
+uint8_t* staging(mb_ctx* c, int want, int& fields) {
     const size_t field = sizeof(float) * (size_t)c->ncell;
-    if (!c->d_upload && device_malloc((void**)&c->d_upload, upload_bytes(c)) == cudaSuccess)
-        c->upload_bytes = upload_bytes(c);
+    const size_t bytes = std::max(5 * (size_t)c->ncell + 16, std::min(want * field, (size_t)16 << 20));
+    if (!c->d_upload || c->upload_bytes < bytes) {
+        uint8_t* p = nullptr;
+        if (device_malloc((void**)&p, bytes) == cudaSuccess) {
+            if (c->d_upload) cudaFree(c->d_upload);   // (waits for the copies in flight)
+            c->d_upload = p;
+            c->upload_bytes = bytes;
+        } else {
+            cudaGetLastError();
+        }
+    }
     if (c->d_upload) {
-        fields = (int)std::min<size_t>(c->upload_bytes / field, 15);
+        fields = (int)std::min<size_t>(c->upload_bytes / field, want);
         return c->d_upload;
     }
-    cudaGetLastError();
     if (!c->h_stage && cudaMallocHost((void**)&c->h_stage, field) != cudaSuccess) {
         cudaGetLastError();
         c->h_stage = nullptr;
@@ -355,7 +360,7 @@ cudaError_t rows_out(mb_ctx* c, void* packed, const void* rows, size_t esize, in
         return cudaGetLastError();
     }
     int fit = 1;
-    uint8_t* stage = staging(c, fit);
+    uint8_t* stage = staging(c, arrays, fit);
     if (!stage) return cudaErrorMemoryAllocation;
     for (int q = 0; q < arrays; q += fit) {
         const int m = std::min(fit, arrays - q);
@@ -375,7 +380,7 @@ cudaError_t rows_in(mb_ctx* c, void* rows, const void* packed, size_t esize, int
         return cudaGetLastError();
     }
     int fit = 1;
-    uint8_t* stage = staging(c, fit);
+    uint8_t* stage = staging(c, arrays, fit);
     if (!stage) return cudaErrorMemoryAllocation;
     for (int q = 0; q < arrays; q += fit) {
         const int m = std::min(fit, arrays - q);
@@ -394,7 +399,7 @@ cudaError_t gain_out(mb_ctx* c, void* packed, int first, int fields, cudaMemcpyK
     }
     const size_t field = sizeof(float) * (size_t)c->ncell;
     int fit = 1;
-    uint8_t* stage = staging(c, fit);
+    uint8_t* stage = staging(c, fields, fit);
     if (!stage) return cudaErrorMemoryAllocation;
     for (int q = 0; q < fields; q += fit) {
         const int m = std::min(fit, fields - q);
@@ -407,7 +412,7 @@ cudaError_t gain_out(mb_ctx* c, void* packed, int first, int fields, cudaMemcpyK
 cudaError_t gain_in(mb_ctx* c, int first, int fields, const void* packed) {
     const size_t field = sizeof(float) * (size_t)c->ncell;
     int fit = 1;
-    uint8_t* stage = staging(c, fit);
+    uint8_t* stage = staging(c, fields, fit);
     if (!stage) return cudaErrorMemoryAllocation;
     for (int q = 0; q < fields; q += fit) {
         const int m = std::min(fit, fields - q);
@@ -1029,7 +1034,7 @@ int mb_set_material(mb_ctx* c, const float* eps_map, const uint8_t* gain_mask, d
     };
     const bool rows = c->px != c->nx;
     const size_t key_bytes = 2 * sizeof(uint32_t) * mb::kMatKeys + 2 * sizeof(int);
-    if (!grow((void**)&c->d_upload, c->upload_bytes, upload_bytes(c)) ||
+    if (!grow((void**)&c->d_upload, c->upload_bytes, 5 * (size_t)N + 16) ||
         !grow((void**)&c->d_keys, c->keys_bytes, key_bytes))
         return fail(c, MB_ERR_OOM, "material map scratch allocation failed");
     float* d_eps = reinterpret_cast<float*>(c->d_upload);
@@ -1634,7 +1639,7 @@ int mb_get_field(mb_ctx* c, int which, float* host_out) {
     const int64_t N = c->ncell;
     if (which == MB_N0) {
         int fit = 1;
-        uint8_t* stage = staging(c, fit);
+        uint8_t* stage = staging(c, 1, fit);
         if (!stage) return fail(c, MB_ERR_OOM, "no memory for the packed field");
         mb::launch_n0(c->args.f.gs, c->d_mat, c->px, (float*)stage, c->nx, (int64_t)c->ny * c->nz, c->N_a, c->stream);
         MB_CUDA(c, cudaGetLastError());
@@ -1679,7 +1684,7 @@ int mb_get_field_device(mb_ctx* c, int which, float* dev_out, double* scale) {
         MB_CUDA(c, field_out(c, dev_out, which, cudaMemcpyDeviceToDevice));
     } else {
         int fit = 1;
-        uint8_t* stage = staging(c, fit);
+        uint8_t* stage = staging(c, 1, fit);
         if (!stage) return fail(c, MB_ERR_OOM, "no memory for the packed field");
         MB_CUDA(c, field_out(c, stage, which, cudaMemcpyDeviceToDevice));
         MB_CUDA(c, cudaMemcpyAsync(dev_out, stage, bytes,
