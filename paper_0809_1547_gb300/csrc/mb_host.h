@@ -95,7 +95,7 @@ struct DevPlaneProbe {
 // each thread walks kz planes).
 constexpr int kVariant3D = 0;
 constexpr int kVariantZmarch = 1;
-constexpr int kVariantTma = 2;   // TMA-staged z-walk (nx % 16 == 0)
+constexpr int kVariantTma = 2;   // TMA-staged z-walk (nx % 16 == 0); in tune_f: the single-pass step (px % 4 == 0)
 constexpr int kVariantVec = 3;   // z-walk over quads of 4 x-cells, 16-byte accesses (nx % 4 == 0)
 constexpr int kVariantSmall = 4; // many steps per launch, state in shared memory (small grids; tune_f only)
 struct PassTune {

@@ -24,6 +24,9 @@
 // Every update uses the per-cell helpers' operations, so the fields equal
 // those of the other launches bit for bit.
 //
+// Only one such launch fits the GPU at a time (its blocks take nearly all of an
+// SM's shared memory): a batch of small grids tries it with all members running.
+//
 // Measured, per step with a point probe: 24 x 22 x 20 cells 3.1 us, 48^3 4.6
 // us (two passes and the probe's launch, tuned: 8.0 and 11.7), plus 10 and 16
 // us per launch to load and store the state; the tuner times both parts and
