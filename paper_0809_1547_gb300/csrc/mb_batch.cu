@@ -503,7 +503,7 @@ int mb_batch_autotune(mb_batch* b) {
                 c->use_fused = on != 0;
                 mbi::drop_graphs(c);
             }
-            t[on] = std::min(concurrent_ms(4), concurrent_ms(4));
+            t[on] = concurrent_ms(4);
         }
         if (t[1] < t[0])
             for (mb_ctx* c : close) {

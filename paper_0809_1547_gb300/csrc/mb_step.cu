@@ -551,7 +551,7 @@ int mb_autotune(mb_ctx* c) {
     }
     // the single-pass step against the best pair of passes
     mb::PassTune bf = c->tune_f;
-    float best_f = 1e30f;
+    float best_f = 1e30f, best_two = best_h + best_e;
     const bool tma = mb::fused_supported(c->args);
     if (tma || small_ready(c)) ensure_second_copy(c);
     if (tma && c->d_fields2) {
@@ -593,6 +593,35 @@ int mb_autotune(mb_ctx* c) {
                 bf = tf[q].second;
             }
         best_f *= reps;   // back to the passes' unit: ms per reps launches
+        // A pass repeated by itself finds more of its arrays in L2 than one
+        // between the others (157 x 131 x 110: H and E 34 + 33 us alone, 34 + 43
+        // in steps): within a quarter of each other the two are timed as steps.
+        if (best_f < 1.25f * best_two && best_two < 1.25f * best_f) {
+            const int steps = large ? 2 : 8;   // even: the state's own copy is the last written
+            const auto* fm = fused_maps_for(c, bf);
+            const mb::TmaMaps *mh = tma_for(c, bh), *me = tma_for(c, be);
+            const mb::StepArgs view[2] = {view_of(c, 0), view_of(c, 1)};
+            best_f = best_two = 1e30f;
+            for (int round = 0; round < 6; ++round) {
+                cudaEventRecord(e0, c->stream);
+                for (int r = 0, p = c->parity; r < steps; ++r) {
+                    if (round & 1) {
+                        mb::launch_fused_step(view[p], ping_of(c, view[1 - p], 1 - p), bf, p ? fm->second : fm->first,
+                                              c->stream);
+                        p = 1 - p;
+                    } else {
+                        mb::launch_h_pass(c->args, bh, mh, c->stream);
+                        mb::launch_e_pass(c->args, be, me, c->stream);
+                    }
+                }
+                cudaEventRecord(e1, c->stream);
+                cudaEventSynchronize(e1);
+                float ms = 0;
+                cudaEventElapsedTime(&ms, e0, e1);
+                float& best = round & 1 ? best_f : best_two;
+                best = std::min(best, ms * reps / steps);
+            }
+        }
     } else {
         cudaGetLastError();
         c->err.clear();
@@ -613,13 +642,13 @@ int mb_autotune(mb_ctx* c) {
             if (r >= 2) t[r & 1] = std::min(t[r & 1], ms);
         }
         const float step = std::max((t[1] - t[0]) / 12.0f, 0.0f), fixed = std::max(t[0] - 4.0f * step, 0.0f);
-        const float other = std::min(best_f, best_h + best_e) / reps;
+        const float other = std::min(best_f, best_two) / reps;
         small = cudaGetLastError() == cudaSuccess && step + fixed / 16.0f < other;
         // kz: the fewest steps of a call that repay the launch's fixed part
         if (small) bf = mb::PassTune{mb::kVariantSmall, dim3(32, 8, 1), std::max(1, (int)std::ceil(fixed / (other - step)))};
     }
-    const bool fused = small || best_f < best_h + best_e;
-    c->fused_ratio = best_f / (best_h + best_e);
+    const bool fused = small || best_f < best_two;
+    c->fused_ratio = best_f / best_two;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     {
